@@ -1406,20 +1406,17 @@ sp_status sp_tc_init(sp_graph *g, int64_t *count) {
   if (!g || !count) return SP_EINVAL;
   int launches = 0;
   sp::launch_ctl_reset(g, 0, &launches);
-  sp::launch_tc_sym_check(g, &launches);
+  sp::launch_tc_static(g, &launches);   // checks the symmetry first
+  if (cudaGetLastError() != cudaSuccess) {
+    cudaStreamSynchronize(g->stream);
+    return SP_ECUDA;
+  }
   sp_status rc = read_ctl(g);
   if (rc != SP_OK) return rc;
   if (g->ctl_host->status != 0) {
     g->tc_state = 0;
     return (sp_status)g->ctl_host->status;
   }
-  sp::launch_tc_static(g, &launches);
-  if (cudaGetLastError() != cudaSuccess) {
-    cudaStreamSynchronize(g->stream);
-    return SP_ECUDA;
-  }
-  rc = read_ctl(g);
-  if (rc != SP_OK) return rc;
   g->tc_count = (long long)g->ctl_host->tc_static;
   g->tc_state = 1;
   *count = g->tc_count;

@@ -304,7 +304,6 @@ void launch_state_check(sp_graph *g, const int *dist_d, const int *parent_d, int
                         int *launches);
 void launch_state_pack(sp_graph *g, const int *dist_d, const int *parent_d, int *launches);
 // sp_tc.cu
-void launch_tc_sym_check(sp_graph *g, int *launches);
 void launch_tc_static(sp_graph *g, int *launches);
 void launch_tc_batch_sym(sp_graph *g, long long nb, int *launches);
 void launch_tc_delta(sp_graph *g, long long nb, int kind, int *launches);

@@ -2,8 +2,9 @@
 // coded in StarPlat DSL": staticTC, Decremental, Incremental, DynTC).
 //
 // The graph is read as undirected: every edge is stored in both directions
-// (checked).  staticTC counts, for every vertex v, the pairs of neighbours
-// u < v < w with u -> w an edge: every triangle once, at its middle vertex.
+// (checked).  staticTC counts every triangle once; the listing sees it at its
+// middle vertex by id (u < v < w), the kernels here at its smallest one by
+// (degree, id), which is the same number.
 // A batch changes the count by the listing's corrections.  For every
 // applied update (v1, v2) (each pair appears in both directions) and every
 // common neighbour v3 of v1 and v2, the triangle {v1, v2, v3} is seen once
@@ -16,6 +17,8 @@
 // neighbours are found by walking the shorter of the two sorted rows and
 // binary-searching the other, which finds the same set as the listing's
 // walk over v1's row.
+#include <algorithm>
+
 #include "sp_graph.cuh"
 
 namespace sp {
@@ -34,67 +37,363 @@ __device__ __forceinline__ bool row_has(const int2 *row, int deg, int x) {
   return lo < deg && __ldg(&row[lo].x) == x;
 }
 
-__device__ __forceinline__ int row_lower(const int2 *row, int deg, int x) {
-  int lo = 0, hi = deg;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (__ldg(&row[mid].x) < x) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
 __device__ __forceinline__ u64 warp_sum64(u64 x) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
   return x;
 }
 
-// Every edge u -> v has its reverse v -> u (a warp per vertex).
-__global__ void __launch_bounds__(kThreads) k_tc_sym_check(Store st, int n, Ctl *c) {
+__device__ __forceinline__ u32 warp_incl_scan(u32 x) {
   const int lane = threadIdx.x & 31;
-  const long long w0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long u = w0; u < n; u += nw) {
-    const RowMeta ru = st.row[u];
-    for (int e = lane; e < ru.deg; e += 32) {
-      const int v = __ldg(&st.adj[ru.start + e].x);
-      const RowMeta rv = st.row[v];
-      if (!row_has(st.adj + rv.start, rv.deg, (int)u)) atomicCAS(&c->status, 0, SP_EINVAL);
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const u32 y = __shfl_up_sync(kFull, x, o);
+    if (lane >= o) x += y;
+  }
+  return x;
+}
+
+// Lane holding the warp-wide element t, given the lanes' inclusive counts
+// (t < the total): the number of lanes whose count is at most t.
+__device__ __forceinline__ int owner_lane(u32 incl, u32 t) {
+  int o = 0;
+#pragma unroll
+  for (int step = 16; step > 0; step >>= 1)
+    if (__shfl_sync(kFull, incl, o + step - 1) <= t) o += step;
+  return o;
+}
+
+// --- staticTC ---------------------------------------------------------------
+//
+// Every undirected edge {u, v} is kept once, from the end that is smaller by
+// (degree, id), which bounds the lists by sqrt(2 m) whatever the hubs; a
+// triangle is then seen once, at its smallest vertex u: v in out(u), w in
+// out(u) and w in out(v).  k_tc_orient writes out(v) as plain u32 ids into
+// row v's alternate region of the forward store (free between merges, and at
+// least as long as the row), so the count needs no memory of its own.  In the
+// same pass every row is compared with the same row of the reverse store:
+// equal rows everywhere mean that every edge has its reverse, which is the
+// symmetry check without a search per edge.  R-MAT 18, edge factor 8: check and
+// count 0.98 ms; a warp per vertex v walking its lower neighbours one by one,
+// behind a binary search per edge, took 29.3 ms (1.14 ms of it the check):
+// the hubs' rows were serial.
+constexpr int kOrientRow = 256;      // longer rows are taken by a whole block
+constexpr int kOrientGiant = 65536;  // ... and these by the whole grid
+constexpr int kOK = 4;               // edges per thread in flight
+
+struct OrientArgs {
+  Store fwd, rev;
+  u32 *cnt;       // [n] |out(v)|
+  u32 *giant;     // rows for k_tc_orient_giant
+  Ctl *c;
+  int n, rpw;     // rows per warp (1..32)
+};
+
+struct OrientEdge {   // one edge of row v, its loads issued apart from their use
+  int x, y, dx;
+};
+
+__device__ __forceinline__ void orient_load(const OrientArgs &a, long long fs, long long rs, u32 e,
+                                            bool on, OrientEdge &g) {
+  g.x = on ? __ldg(&a.fwd.adj[fs + e].x) : 0;
+  g.y = on ? __ldg(&a.rev.adj[rs + e].x) : 0;
+}
+
+// Does v keep the edge to x: is v smaller by (degree, id)?
+__device__ __forceinline__ bool orient_keeps(int v, int dv, int x, int dx) {
+  return x != v && (dx > dv || (dx == dv && x > v));
+}
+
+__global__ void __launch_bounds__(kThreads) k_tc_orient(OrientArgs a) {
+  __shared__ u32 s_cnt[kThreads / 32][32];
+  __shared__ u32 s_row[kThreads], s_nrow, s_out;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rpb = a.rpw * (kThreads / 32);
+  bool bad = false;
+  for (long long b0 = (long long)blockIdx.x * rpb; b0 < a.n; b0 += (long long)gridDim.x * rpb) {
+    if (threadIdx.x == 0) s_nrow = 0;
+    s_cnt[warp][lane] = 0;
+    __syncthreads();
+    // the warp's rows, one per lane, then their edges spread over the lanes
+    const long long r = b0 + (long long)warp * a.rpw + lane;
+    const bool mine = lane < a.rpw && r < a.n;
+    int deg = 0;
+    long long fs = 0, rs = 0, alt = 0;
+    if (mine) {
+      const RowMeta f = a.fwd.row[r], q = a.rev.row[r];
+      deg = f.deg;
+      fs = f.start;
+      rs = q.start;
+      alt = a.fwd.alt[r];
+      if (q.deg != f.deg) {
+        bad = true;
+        deg = 0;     // not symmetric: the count is not kept
+      }
     }
+    u32 len = (u32)deg;
+    if (deg > kOrientGiant) {
+      a.giant[atomicAdd(&a.c->tc_ngiant, 1u)] = (u32)r;
+      a.cnt[r] = 0;
+      len = 0;
+    } else if (deg > kOrientRow) {
+      s_row[atomicAdd(&s_nrow, 1u)] = (u32)r;
+      len = 0;
+    }
+    const u32 incl = warp_incl_scan(len), total = __shfl_sync(kFull, incl, 31);
+    const u32 excl = incl - len;
+    for (u32 t0 = 0; t0 < total; t0 += 32 * kOK) {
+      OrientEdge g[kOK];
+      int o[kOK];
+      bool on[kOK];
+#pragma unroll
+      for (int k = 0; k < kOK; ++k) {
+        const u32 t = t0 + 32 * k + lane;
+        on[k] = t < total;
+        o[k] = owner_lane(incl, on[k] ? t : 0u) & 31;
+        const u32 e = t - __shfl_sync(kFull, excl, o[k]);
+        orient_load(a, __shfl_sync(kFull, fs, o[k]), __shfl_sync(kFull, rs, o[k]), e, on[k], g[k]);
+      }
+#pragma unroll
+      for (int k = 0; k < kOK; ++k) g[k].dx = on[k] ? __ldg(&a.fwd.row[g[k].x].deg) : 0;
+#pragma unroll
+      for (int k = 0; k < kOK; ++k) {
+        const int dv = __shfl_sync(kFull, deg, o[k]);
+        const long long av = __shfl_sync(kFull, alt, o[k]);
+        const int v = (int)__shfl_sync(kFull, (u32)r, o[k]);
+        if (!on[k]) continue;
+        bad |= g[k].x != g[k].y;
+        if (orient_keeps(v, dv, g[k].x, g[k].dx))
+          ((u32 *)(a.fwd.adj + av))[atomicAdd(&s_cnt[warp][o[k]], 1u)] = (u32)g[k].x;
+      }
+    }
+    __syncwarp();
+    if (mine && (u32)deg == len) a.cnt[r] = s_cnt[warp][lane];
+    __syncthreads();
+    const u32 nrow = s_nrow;
+    for (u32 i = 0; i < nrow; ++i) {   // long rows, the whole block on each
+      const int v = (int)s_row[i];
+      const RowMeta f = a.fwd.row[v];
+      const long long rv = a.rev.row[v].start;
+      u32 *out = (u32 *)(a.fwd.adj + a.fwd.alt[v]);
+      if (threadIdx.x == 0) s_out = 0;
+      __syncthreads();
+      for (u32 e0 = threadIdx.x; e0 < (u32)f.deg; e0 += kThreads * kOK) {
+        OrientEdge g[kOK];
+#pragma unroll
+        for (int k = 0; k < kOK; ++k)
+          orient_load(a, f.start, rv, e0 + k * kThreads, e0 + k * kThreads < (u32)f.deg, g[k]);
+#pragma unroll
+        for (int k = 0; k < kOK; ++k)
+          g[k].dx = e0 + k * kThreads < (u32)f.deg ? __ldg(&a.fwd.row[g[k].x].deg) : 0;
+#pragma unroll
+        for (int k = 0; k < kOK; ++k) {
+          if (e0 + k * kThreads >= (u32)f.deg) continue;
+          bad |= g[k].x != g[k].y;
+          if (orient_keeps(v, f.deg, g[k].x, g[k].dx)) out[atomicAdd(&s_out, 1u)] = (u32)g[k].x;
+        }
+      }
+      __syncthreads();
+      if (threadIdx.x == 0) a.cnt[v] = s_out;
+    }
+    __syncthreads();
+  }
+  if (bad) atomicCAS(&a.c->status, 0, SP_EINVAL);
+}
+
+// Rows longer than kOrientGiant (at most m / kOrientGiant of them): every
+// block takes its share of each.
+__global__ void __launch_bounds__(kThreads) k_tc_orient_giant(OrientArgs a) {
+  const u32 ng = ld_cg_u32(&a.c->tc_ngiant);
+  bool bad = false;
+  for (u32 i = 0; i < ng; ++i) {
+    const int v = (int)a.giant[i];
+    const RowMeta f = a.fwd.row[v];
+    const long long rv = a.rev.row[v].start;
+    u32 *out = (u32 *)(a.fwd.adj + a.fwd.alt[v]);
+    for (long long e = blockIdx.x * (long long)kThreads + threadIdx.x; e < f.deg;
+         e += (long long)gridDim.x * kThreads) {
+      OrientEdge g;
+      orient_load(a, f.start, rv, (u32)e, true, g);
+      bad |= g.x != g.y;
+      if (orient_keeps(v, f.deg, g.x, __ldg(&a.fwd.row[g.x].deg)))
+        out[atomicAdd(a.cnt + v, 1u)] = (u32)g.x;
+    }
+  }
+  if (bad) atomicCAS(&a.c->status, 0, SP_EINVAL);
+}
+
+// The lists longer than kWarpList, one block each, in a list of their own;
+// the shorter ones are taken from the vertices in order, a warp each.
+constexpr u32 kWarpList = 32;
+
+__global__ void __launch_bounds__(kThreads) k_tc_lists(const u32 *__restrict__ cnt, int n, u32 *big,
+                                                       Ctl *c) {
+  const int lane = threadIdx.x & 31;
+  const long long step = (long long)gridDim.x * kThreads;
+  for (long long b = blockIdx.x * (long long)kThreads + (threadIdx.x & ~31); b < n; b += step) {
+    const long long v = b + lane;
+    const bool is = v < n && cnt[v] > kWarpList;
+    const u32 m = __ballot_sync(kFull, is);
+    if (!m) continue;
+    u32 base = 0;
+    if (lane == 0) base = atomicAdd(&c->tc_nbig, (u32)__popc(m));
+    base = __shfl_sync(kFull, base, 0);
+    if (is) big[base + __popc(m & lanemask_lt())] = (u32)v;
   }
 }
 
-// staticTC (a warp per vertex v): for every neighbour u < v, count the
-// neighbours w > v of v that are neighbours of u.
-__global__ void __launch_bounds__(kThreads) k_tc_static(Store st, int n, Ctl *c) {
+constexpr u32 kEmpty = 0xFFFFFFFFu;       // no vertex has this id (n < 2^31)
+constexpr u32 kTabMax = 8192;             // slots of a block's table: half of them used
+constexpr u32 kWarpTab = 64;
+constexpr u32 kWK = 4;                    // probes per lane in flight
+
+__device__ __forceinline__ u32 hash_slot(u32 x, u32 bits) { return (x * 0x9E3779B1u) >> (32 - bits); }
+
+__device__ __forceinline__ void tab_put(u32 *tab, u32 bits, u32 x) {
+  const u32 mask = (1u << bits) - 1;
+  u32 h = hash_slot(x, bits);
+  while (atomicCAS(tab + h, kEmpty, x) != kEmpty) h = (h + 1) & mask;   // ids are distinct
+}
+
+// (at most half of the slots are used, so every probe ends)
+__device__ __forceinline__ bool tab_has(const u32 *tab, u32 bits, u32 x) {
+  const u32 mask = (1u << bits) - 1;
+  u32 h = hash_slot(x, bits);
+  for (;;) {
+    const u32 y = tab[h];
+    if (y == x) return true;
+    if (y == kEmpty) return false;
+    h = (h + 1) & mask;
+  }
+}
+
+// The elements of the lanes' lists (ptr, len) that are in the table: lists of
+// at least 32 elements on average are read one after the other by the whole
+// warp, shorter ones are laid end to end over the lanes.
+__device__ __forceinline__ u32 count_lists(const u32 *ptr, u32 len, const u32 *tab, u32 bits) {
   const int lane = threadIdx.x & 31;
-  const long long w0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-  u64 cnt = 0;
-  for (long long v = w0; v < n; v += nw) {
-    const RowMeta rv = st.row[v];
-    const int2 *row = st.adj + rv.start;
-    const int lo_end = row_lower(row, rv.deg, (int)v);        // neighbours < v
-    int up = lo_end;
-    if (up < rv.deg && __ldg(&row[up].x) == (int)v) ++up;     // skip a self-loop
-    const int nup = rv.deg - up;                               // neighbours > v
-    if (nup == 0) continue;
-    for (int a = 0; a < lo_end; ++a) {
-      const int u = __ldg(&row[a].x);
-      const RowMeta ru = st.row[u];
-      const int2 *urow = st.adj + ru.start;
-      if (nup <= ru.deg) {
-        for (int b = lane; b < nup; b += 32) cnt += row_has(urow, ru.deg, __ldg(&row[up + b].x));
-      } else {
-        // walk u's neighbours above v, search v's upper part
-        const int s = row_lower(urow, ru.deg, (int)v + 1);
-        for (int b = s + lane; b < ru.deg; b += 32)
-          cnt += row_has(row + up, nup, __ldg(&urow[b].x));
+  const u32 incl = warp_incl_scan(len), total = __shfl_sync(kFull, incl, 31);
+  u32 c = 0;
+  u32 lists = __ballot_sync(kFull, len > 0);
+  if (total >= 32u * __popc(lists)) {
+    while (lists) {
+      const int o = __ffs(lists) - 1;
+      lists &= lists - 1;
+      const u32 *p = (const u32 *)__shfl_sync(kFull, (u64)ptr, o);
+      const u32 n = __shfl_sync(kFull, len, o);
+      for (u32 e = lane; e < n; e += 32 * kWK) {
+        u32 x[kWK];
+#pragma unroll
+        for (u32 k = 0; k < kWK; ++k) x[k] = e + 32 * k < n ? __ldg(p + e + 32 * k) : kEmpty;
+#pragma unroll
+        for (u32 k = 0; k < kWK; ++k) c += x[k] != kEmpty && tab_has(tab, bits, x[k]);
+      }
+    }
+  } else {
+    const u32 excl = incl - len;
+    for (u32 t0 = 0; t0 < total; t0 += 32 * kWK) {
+      u32 x[kWK];
+#pragma unroll
+      for (u32 k = 0; k < kWK; ++k) {
+        const u32 t = t0 + 32 * k + lane;
+        const int o = owner_lane(incl, t < total ? t : 0u) & 31;
+        const u32 *p = (const u32 *)__shfl_sync(kFull, (u64)ptr, o);
+        const u32 e = t - __shfl_sync(kFull, excl, o);
+        x[k] = t < total ? __ldg(p + e) : kEmpty;
+      }
+#pragma unroll
+      for (u32 k = 0; k < kWK; ++k) c += x[k] != kEmpty && tab_has(tab, bits, x[k]);
+    }
+  }
+  return c;
+}
+
+// One vertex u at a time: out(u) in a hash table in shared memory, then the
+// lists of its members walked coalesced and looked up there.  A list longer
+// than half a block's table is taken in parts (a triangle's w lies in exactly
+// one of them).  What bounds it is the walk: sum over the oriented edges
+// u -> v of |out(v)| list words through L2, one or two shared-memory probes
+// each.
+__global__ void __launch_bounds__(kThreads) k_tc_count(Store st, int n, const u32 *__restrict__ cnt,
+                                                       const u32 *__restrict__ big, Ctl *c) {
+  __shared__ u32 tab[kTabMax];
+  __shared__ u32 s_u, s_pos;
+  if (ld_cg_i32(&c->status) != 0) return;   // not symmetric (the same answer in every block)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u32 nbig = ld_cg_u32(&c->tc_nbig);
+  u64 sum = 0;
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_u = atomicAdd(&c->tc_bpos, 1u);
+    __syncthreads();
+    if (s_u >= nbig) break;
+    const u32 u = big[s_u];
+    const u32 d = cnt[u];
+    const u32 *out = (const u32 *)(st.adj + st.alt[u]);
+    // members per grab: every warp gets some, a lane each
+    const u32 grab = min(32u, max(4u, (d + kThreads / 32 - 1) / (kThreads / 32)));
+    for (u32 part = 0; part < d; part += kTabMax / 2) {
+      const u32 np = min(d - part, kTabMax / 2);
+      u32 bits = 7;
+      while ((1u << bits) < 2 * np) ++bits;
+      __syncthreads();
+      for (u32 i = threadIdx.x; i < (1u << bits); i += kThreads) tab[i] = kEmpty;
+      if (threadIdx.x == 0) s_pos = 0;
+      __syncthreads();
+      for (u32 i = threadIdx.x; i < np; i += kThreads) tab_put(tab, bits, out[part + i]);
+      __syncthreads();
+      for (;;) {
+        u32 at = 0;
+        if (lane == 0) at = atomicAdd(&s_pos, grab);
+        at = __shfl_sync(kFull, at, 0);
+        if (at >= d) break;
+        const u32 i = at + lane;
+        u32 len = 0;
+        const u32 *p = nullptr;
+        if (lane < (int)grab && i < d) {
+          const u32 v = out[i];
+          len = cnt[v];
+          p = (const u32 *)(st.adj + st.alt[v]);
+        }
+        sum += count_lists(p, len, tab, bits);
       }
     }
   }
-  cnt = warp_sum64(cnt);
-  if (lane == 0 && cnt) atomicAdd(&c->tc_static, cnt);
+  __syncthreads();
+  // short lists: a warp takes 32 vertices, then those with two members or more
+  u32 *wtab = tab + warp * kWarpTab;
+  for (;;) {
+    u32 v0 = 0;
+    if (lane == 0) v0 = atomicAdd(&c->tc_spos, 1u);
+    const long long b = 32LL * __shfl_sync(kFull, v0, 0);
+    if (b >= n) break;
+    const u32 dl = b + lane < n ? cnt[b + lane] : 0u;
+    const long long al = b + lane < n ? st.alt[b + lane] : 0;
+    u32 todo = __ballot_sync(kFull, dl >= 2 && dl <= kWarpList);
+    while (todo) {
+      const int o = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const u32 d = __shfl_sync(kFull, dl, o);
+      const u32 *out = (const u32 *)(st.adj + __shfl_sync(kFull, al, o));
+      wtab[lane] = kEmpty;
+      wtab[lane + 32] = kEmpty;
+      u32 len = 0;
+      const u32 *p = nullptr;
+      u32 v = 0;
+      if ((u32)lane < d) {
+        v = out[lane];
+        len = cnt[v];
+        p = (const u32 *)(st.adj + st.alt[v]);
+      }
+      __syncwarp();
+      if ((u32)lane < d) tab_put(wtab, 6, v);
+      __syncwarp();
+      sum += count_lists(p, len, wtab, 6);
+      __syncwarp();
+    }
+  }
+  sum = warp_sum64(sum);
+  if (lane == 0 && sum) atomicAdd(&c->tc_static, sum);
 }
 
 // Is (x, y) an applied update of `kind` in the sorted forward items [0, nb)?
@@ -185,16 +484,32 @@ inline unsigned grid_for(long long work, int per_block, int cap) {
 
 }  // namespace
 
-void launch_tc_sym_check(sp_graph *g, int *launches) {
-  k_tc_sym_check<<<grid_for((long long)g->n * 32, kThreads, g->num_sms * 16), kThreads, 0,
-                   g->stream>>>(g->fwd, g->n, g->ctl);
-  ++*launches;
-}
-
+// staticTC with the symmetry check: the count (or status SP_EINVAL) in ctl.
+// Scratch: the forward store's alternate regions and the per-vertex words of
+// the invalidation (g->jmp, g->cut, g->asv), all rewritten before their next
+// use.
 void launch_tc_static(sp_graph *g, int *launches) {
-  k_tc_static<<<grid_for((long long)g->n * 32, kThreads, g->num_sms * 16), kThreads, 0,
-                g->stream>>>(g->fwd, g->n, g->ctl);
+  OrientArgs a;
+  a.fwd = g->fwd;
+  a.rev = g->rev;
+  a.cnt = g->jmp;
+  a.giant = g->asv;
+  a.c = g->ctl;
+  a.n = g->n;
+  const int warps = g->num_sms * 6 * (kThreads / 32);
+  a.rpw = std::max(1, std::min(32, (int)(((long long)g->n + warps - 1) / warps)));
+  k_tc_orient<<<grid_for(g->n, a.rpw * (kThreads / 32), g->num_sms * 16), kThreads, 0, g->stream>>>(
+      a);
   ++*launches;
+  if (g->m > kOrientGiant) {   // such a row can be there
+    k_tc_orient_giant<<<(unsigned)g->num_sms * 4, kThreads, 0, g->stream>>>(a);
+    ++*launches;
+  }
+  k_tc_lists<<<grid_for(g->n, kThreads, g->num_sms * 8), kThreads, 0, g->stream>>>(a.cnt, g->n,
+                                                                                   g->cut, g->ctl);
+  k_tc_count<<<(unsigned)g->num_sms * 6, kThreads, 0, g->stream>>>(g->fwd, g->n, a.cnt, g->cut,
+                                                                   g->ctl);
+  *launches += 2;
 }
 
 void launch_tc_batch_sym(sp_graph *g, long long nb, int *launches) {

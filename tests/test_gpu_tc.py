@@ -107,3 +107,62 @@ def test_counts_states():
         assert e.value.code == sp.SP_ESTATE
         ref = oracle.OracleGraph(W.n, *g.export_csr())
         assert g.tc_init() == ref.triangles()
+
+
+def wheel(k, shift):
+    """A hub joined to every vertex of a cycle of k: k triangles.  The hub's
+    id is `shift`, the rim takes the others in order."""
+    rim = np.array([v for v in range(k + 1) if v != shift], np.int64)
+    nxt = np.roll(rim, -1)
+    u = np.concatenate([rim, nxt, rim, np.full(k, shift)])
+    v = np.concatenate([nxt, rim, np.full(k, shift), rim])
+    order = np.lexsort((v, u))
+    ro = np.zeros(k + 2, np.int64)
+    np.cumsum(np.bincount(u, minlength=k + 1), out=ro[1:])
+    return k + 1, ro, v[order].astype(np.int32), np.ones(4 * k, np.int32)
+
+
+# a row at and above what a warp, a block and the whole grid orient
+@pytest.mark.parametrize("k", [4, 255, 256, 257, 1024, 65536, 65537, 200003])
+def test_static_count_of_wheels(k):
+    n, ro, col, w = wheel(k, shift=k // 3)
+    with sp.Graph(n, ro, col, w) as g:
+        assert g.tc_init() == k
+        # a spoke and a rim edge beside it go: the spoke's two triangles are lost
+        hub, a = k // 3, 0 if k // 3 else 1
+        b = a + 1 if a + 1 != hub else a + 2
+        ds = np.array([hub, a, a, b], np.int32)
+        dd = np.array([a, hub, b, a], np.int32)
+        z = np.zeros(0, np.int32)
+        assert g.tc_apply_batch(ds, dd, z, z, z) == k - 2
+        assert g.tc_apply_batch(z, z, ds, dd, np.ones(4, np.int32)) == k
+
+
+# lists at the bounds of a warp's table (32 members), a block's smallest table
+# and a block's largest one (4,096, beyond which a list is taken in parts)
+@pytest.mark.parametrize("n", [2, 3, 33, 34, 35, 65, 66, 1000, 4097, 4098, 4200])
+def test_static_count_of_complete_graphs(n):
+    v = np.tile(np.arange(n, dtype=np.int32), n).reshape(n, n)
+    col = v[~np.eye(n, dtype=bool)]
+    ro = np.arange(n + 1, dtype=np.int64) * (n - 1)
+    with sp.Graph(n, ro, col, np.ones(col.size, np.int32)) as g:
+        assert g.tc_init() == n * (n - 1) * (n - 2) // 6
+
+
+@pytest.mark.parametrize("at", [0, 300, 69999])
+def test_an_asymmetric_edge_is_found(at):
+    # the wheel with one direction of one rim edge turned elsewhere: the rows'
+    # lengths stay equal in all but two
+    n, ro, col, w = wheel(70000, shift=70000)
+    u = np.repeat(np.arange(n), np.diff(ro))
+    i = np.nonzero((u == at) & (col == (at + 1) % 70000))[0][0]
+    far = (at + 5000) % 70000
+    col = col.copy()
+    col[i] = far
+    lo, hi = ro[at], ro[at + 1]
+    order = np.argsort(col[lo:hi])
+    col[lo:hi] = col[lo:hi][order]
+    with sp.Graph(n, ro, col, w) as g:
+        with pytest.raises(sp.SpError) as e:
+            g.tc_init()
+        assert e.value.code == sp.SP_EINVAL
