@@ -1463,6 +1463,7 @@ sp_status sp_tc_apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
     rec(g, true, 1);
     sp::launch_count(g, ni, &launches);
     sp::launch_tc_batch_sym(g, nb, &launches);     // before anything changes
+    sp::launch_tc_tasks(g, nb, &launches);
     rec(g, true, 2);
     sp::launch_tc_delta(g, nb, 0, &launches);      // Decremental, old graph
     rec(g, true, 3);

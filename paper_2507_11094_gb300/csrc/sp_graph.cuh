@@ -306,6 +306,7 @@ void launch_state_pack(sp_graph *g, const int *dist_d, const int *parent_d, int 
 // sp_tc.cu
 void launch_tc_static(sp_graph *g, int *launches);
 void launch_tc_batch_sym(sp_graph *g, long long nb, int *launches);
+void launch_tc_tasks(sp_graph *g, long long nb, int *launches);
 void launch_tc_delta(sp_graph *g, long long nb, int kind, int *launches);
 // PageRank
 cudaError_t launch_flag(sp_graph *g, const int *dst, long long n, int *launches);

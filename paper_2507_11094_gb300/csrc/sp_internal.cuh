@@ -120,6 +120,8 @@ struct Ctl {
   u32 tc_ngiant, tc_nbig;          // staticTC: rows oriented by the whole grid, long lists
   alignas(128) u32 tc_bpos;        // ... long lists and short-list groups handed out so far
   alignas(128) u32 tc_spos;
+  u64 tc_ntask[2];                 // corrections: tasks listed (deletions, insertions)
+  alignas(128) u64 tc_tpos[2];     // ... and handed out so far
   // the invalidation's cut vertices (a plain list: the pull stage of the
   // push launch turns them into the affected list A)
   alignas(128) u32 ccnt;

@@ -149,6 +149,29 @@ def test_static_count_of_complete_graphs(n):
         assert g.tc_init() == n * (n - 1) * (n - 2) // 6
 
 
+def test_self_loops_and_repeated_updates():
+    # a triangle with a self-loop on every vertex, and updates listed twice
+    # (also with two weights): one of each applies, in both directions
+    n = 40
+    pairs = [(0, 1), (1, 2), (0, 2), (2, 3), (3, 4)] + [(i, i) for i in range(n)]
+    e = sorted({(a, b) for a, b in pairs} | {(b, a) for a, b in pairs})
+    ro = np.zeros(n + 1, np.int64)
+    for u, _ in e:
+        ro[u + 1] += 1
+    np.cumsum(ro, out=ro)
+    with sp.Graph(n, ro, np.array([v for _, v in e], np.int32), np.ones(len(e), np.int32)) as g:
+        assert g.tc_init() == 1
+        ds = np.array([0, 1, 0, 1, 5], np.int32)
+        dd = np.array([1, 0, 1, 0, 5], np.int32)
+        as_ = np.array([2, 4, 4, 2, 4, 0], np.int32)
+        ad = np.array([4, 2, 2, 4, 0, 4], np.int32)
+        aw = np.array([3, 3, 2, 2, 1, 1], np.int32)
+        c = g.tc_apply_batch(ds, dd, as_, ad, aw)
+        ref = oracle.OracleGraph(n, *g.export_csr())
+        assert c == ref.triangles() == 2
+        assert g.tc_init() == 2
+
+
 @pytest.mark.parametrize("at", [0, 300, 69999])
 def test_an_asymmetric_edge_is_found(at):
     # the wheel with one direction of one rim edge turned elsewhere: the rows'
