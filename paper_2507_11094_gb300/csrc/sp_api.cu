@@ -497,9 +497,7 @@ sp_status sp_graph_destroy(sp_graph *g) {
   al.put(g->cut, n * 4);
   al.put(g->aown, (size_t)g->own_cap * 4);
   al.put(g->out_dist, n * 4); al.put(g->out_parent, n * 4);
-  al.put(g->pr[0], n * 4); al.put(g->pr[1], n * 4);
-  al.put(g->prc[0], n * 4); al.put(g->prc[1], n * 4);
-  al.put(g->pracc, n * 4); al.put(g->prflag, n * 4);
+  sp::pr_free(g);
   al.put(g->ctl, sizeof(Ctl));
   if (g->src_dev) al.put(g->src_dev, (size_t)g->n_src * 4);
   drop_batch_graphs(g);
@@ -1239,8 +1237,7 @@ sp_status pr_phase(sp_graph *g, const int *ds, const int *dd, long long nd, cons
     acc.rounds_inval += c.rounds_inval;
   }
   if (n_flag == 0) return SP_OK;   // nothing flagged: every rank stays
-  sp::launch_pr_select(g, 0, launches);
-  cudaError_t e = sp::launch_pr(g, launches);
+  cudaError_t e = sp::launch_pr(g, 0, 0.0f, launches);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     g->last_err = (int)e;
@@ -1289,18 +1286,9 @@ sp_status sp_pr_init(sp_graph *g, float damping, float beta, int32_t max_iter,
                      sp_batch_stats *stats) {
   if (!g || !(damping >= 0.f && damping <= 1.f) || !(beta >= 0.f) || max_iter < 1)
     return SP_EINVAL;
-  const size_t nn = (size_t)g->n;
-  if (!g->pr[0]) {
-    g->pr[0] = (float *)g->al.get(nn * 4);
-    g->pr[1] = (float *)g->al.get(nn * 4);
-    g->prc[0] = (float *)g->al.get(nn * 4);
-    g->prc[1] = (float *)g->al.get(nn * 4);
-    g->pracc = (float *)g->al.get(nn * 4);
-    g->prflag = (u32 *)g->al.get(nn * 4);
-    if (!g->pr[0] || !g->pr[1] || !g->prc[0] || !g->prc[1] || !g->pracc || !g->prflag)
-      return SP_ENOMEM;
-    cudaMemsetAsync(g->prflag, 0, nn * 4, g->stream);
-    g->prtag = 0;
+  if (!g->pr) {
+    const sp_status rc = sp::pr_alloc(g);
+    if (rc != SP_OK) return rc;
     if (sp::loop_blocks(2, g->num_sms) <= 0) return SP_ECUDA;
   }
   g->pr_damping = damping;
@@ -1309,9 +1297,7 @@ sp_status sp_pr_init(sp_graph *g, float damping, float beta, int32_t max_iter,
   int launches = 0;
   rec(g, true, 0);
   sp::launch_ctl_reset(g, 0, &launches);
-  sp::launch_pr_fill(g, 1.0f / (float)g->n, &launches);
-  sp::launch_pr_select(g, 1, &launches);
-  cudaError_t e = sp::launch_pr(g, &launches);
+  cudaError_t e = sp::launch_pr(g, 1, 1.0f / (float)g->n, &launches);
   rec(g, true, SP_NPHASE);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -1525,7 +1511,7 @@ sp_status sp_tc_apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
 sp_status sp_pr_get(const sp_graph *g, float *pr, int out_on_device) {
   if (!g || !pr) return SP_EINVAL;
   if (g->pr_state != 1) return SP_ESTATE;
-  const cudaError_t e = cudaMemcpyAsync(pr, g->pr[0], (size_t)g->n * 4,
+  const cudaError_t e = cudaMemcpyAsync(pr, g->pr, (size_t)g->n * 4,
                                         out_on_device ? cudaMemcpyDeviceToDevice
                                                       : cudaMemcpyDeviceToHost,
                                         g->stream);

@@ -25,7 +25,7 @@
 // its edges before it uses any of them.
 #include <algorithm>
 
-#include "sp_graph.cuh"
+#include "sp_loop.cuh"
 
 namespace sp {
 
@@ -42,103 +42,7 @@ constexpr size_t kLoopSmem =
     (2 * kStageQ + kStageQS + 2 * kStageA + kStageAS + kStageF) * sizeof(u32);
 // the pool schedule's two entry lists follow the stages
 constexpr size_t kLoopSmemPool = kLoopSmem + 2 * kPoolCap * sizeof(uint4);
-constexpr u32 kStageK = 1024;    // stages of the one-pass kernels (static)
 constexpr u32 kNoEdge = 0xFFFFFFFFu;
-constexpr u32 kFull = 0xffffffffu;
-
-__device__ __forceinline__ u32 warp_incl_scan(u32 x) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    u32 y = __shfl_up_sync(kFull, x, o);
-    if (lane >= o) x += y;
-  }
-  return x;
-}
-
-template <typename T>
-__device__ __forceinline__ T warp_sum(T x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-  return x;
-}
-
-__device__ __forceinline__ u64 shfl64(u64 x, int src) {
-  u32 lo = __shfl_sync(kFull, (u32)x, src), hi = __shfl_sync(kFull, (u32)(x >> 32), src);
-  return ((u64)hi << 32) | lo;
-}
-__device__ __forceinline__ u64 shfl64_down(u64 x, int d) {
-  u32 lo = __shfl_down_sync(kFull, (u32)x, d), hi = __shfl_down_sync(kFull, (u32)(x >> 32), d);
-  return ((u64)hi << 32) | lo;
-}
-
-// Grid barrier over a monotone arrival count: barrier k of a launch waits
-// for k * gridDim.x arrivals (the count is zeroed at the start of every
-// call).  Every wait is bounded by lim.wait_ns; a wait that runs out sets
-// ctl->timeout = 2 and returns, and every later wait returns at once.
-__device__ __forceinline__ u64 ld_acquire_u64(const u64 *p) {
-  u64 v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-
-//
-// Returns whether a timeout has been raised (the same answer in every thread
-// of the block, so that loops leave in step and no __syncthreads is left
-// waiting for threads that have gone).
-// With `src`, thread 0 also reads the next round's frontier counters once
-// the wait is over and hands them to the block in *out: one read per block
-// instead of one per warp, all of them at the same line.
-struct RoundCounts {
-  u64 q;        // next frontier: entries << 32 | edges
-  u32 ns;       // its small list
-  u32 nf, fm;   // far pile: count and smallest distance (0, ~0 without one)
-};
-struct CountSrc {
-  const u64 *q;
-  const u32 *ns, *nf, *fm;   // nf, fm null without a far pile
-};
-
-__device__ __forceinline__ bool grid_sync(u64 *bar, u64 target, Ctl *c, const Limits &lim,
-                                          const CountSrc *src = nullptr,
-                                          RoundCounts *out = nullptr) {
-  __shared__ int s_stop;
-  __shared__ RoundCounts s_rc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    // the count before this arrival says whether it was the last one; the
-    // wait polls the count alone and looks at the timeout flag and the
-    // clock every 16th poll
-    // (the test hook lim.miss_site == 2: block 0 does not arrive)
-    const bool miss = lim.miss_site == 2u && blockIdx.x == 0;
-    const u64 arrived = miss ? ld_acquire_u64(bar) : atomicAdd((unsigned long long *)bar, 1ull) + 1;
-    if (arrived < target) {
-      const u64 t0 = globaltimer_ns();
-      u32 polls = 0;
-      while (ld_acquire_u64(bar) < target) {
-        if ((++polls & 15u) == 0) {
-          if (ld_cg_i32(&c->timeout) != 0) break;
-          if (globaltimer_ns() - t0 > lim.wait_ns || polls > kMaxPolls) {
-            raise_timeout(c, 2, 2, (u32)(target / gridDim.x));
-            break;
-          }
-        }
-        __nanosleep(64);
-      }
-    }
-    s_stop = ld_cg_i32(&c->timeout) != 0;
-    if (src) {
-      s_rc.q = ld_cg_u64(src->q);
-      s_rc.ns = ld_cg_u32(src->ns);
-      s_rc.nf = src->nf ? ld_cg_u32(src->nf) : 0u;
-      s_rc.fm = src->fm ? ld_cg_u32(src->fm) : 0xFFFFFFFFu;
-    }
-  }
-  __syncthreads();
-  if (src) *out = s_rc;
-  return s_stop != 0;
-}
 
 __device__ __forceinline__ u64 *qcnt_ptr(Ctl *c, u32 b) {
   return b == 0 ? &c->qcnt0 : (b == 1 ? &c->qcnt1 : &c->qcnt2);
@@ -264,25 +168,6 @@ __device__ __forceinline__ void enqueue(const Queue &q, const RowMeta *row, cons
 #pragma unroll
   for (int k = 0; k < K; ++k) d[k] = (k < kk && want[k]) ? __ldg(&row[x[k]].deg) : 0;
   enqueue_d(q, x, d, kk, n_enq);
-}
-
-// Block scan helper: exclusive prefix of one value per thread; the block
-// total goes to *total (smem scratch of 33 words).
-__device__ __forceinline__ u32 block_excl_scan(u32 x, u32 *scratch, u32 *total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const u32 incl = warp_incl_scan(x);
-  if (lane == 31) scratch[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    u32 v = lane < nwarps ? scratch[lane] : 0u;
-    v = warp_incl_scan(v);
-    if (lane < nwarps) scratch[lane] = v;
-  }
-  __syncthreads();
-  const u32 r = (warp ? scratch[warp - 1] : 0u) + incl - x;
-  *total = scratch[nwarps - 1];
-  __syncthreads();
-  return r;
 }
 
 // Publish a block's staged appends (block-collective): up to two queues
@@ -1021,23 +906,10 @@ __device__ __forceinline__ void process_chunk(Op &op, const int2 *ent, const u32
   op.run(act, ov, od, ed, sx);
 }
 
-__device__ __forceinline__ bool repair_enabled(Ctl *c) {
-  return ld_cg_i32(&c->status) == 0 && ld_cg_i32(&c->need_grow) == 0 &&
-         ld_cg_i32(&c->timeout) == 0 && ld_cg_i32(&c->bad) == 0;
-}
-
 // The batch passed validation (one answer for the whole block).
 __device__ __forceinline__ bool batch_valid_block(Ctl *c) {
   __shared__ int s_ok;
   if (threadIdx.x == 0) s_ok = ld_cg_i32(&c->status) == 0 ? 1 : 0;
-  __syncthreads();
-  return s_ok != 0;
-}
-
-// The same test with one answer for the whole block (kernels with barriers).
-__device__ __forceinline__ bool repair_enabled_block(Ctl *c) {
-  __shared__ int s_ok;
-  if (threadIdx.x == 0) s_ok = repair_enabled(c) ? 1 : 0;
   __syncthreads();
   return s_ok != 0;
 }
@@ -2149,209 +2021,6 @@ __global__ void k_state_pack(const int *__restrict__ dist, const int *__restrict
     s[v] = pack((u32)dist[v], (u32)parent[v]);
 }
 
-// --- PageRank (appendix listing "Dynamic PR") ---------------------------------
-
-// Select the vertices of a Jacobi phase into the list A (entries over the
-// reverse store): every vertex (staticPR) or those flagged in this phase.
-// Selected vertices without in-edges go to a plain list (zlist, zcnt): their
-// new rank is the constant term.
-__global__ void __launch_bounds__(kLoopThreads) k_pr_select(LoopArgs a, int all) {
-  __shared__ u32 sv[kStageK], sd[kStageK], ssv[kStageK];
-  __shared__ Stage st, sst;
-  __shared__ u32 scratch[40];
-  Ctl *c = a.ctl;
-  if (!repair_enabled(c)) return;
-  if (threadIdx.x == 0) {
-    st.n = 0; st.cap = kStageK; st.vmin = kInf; st.v = sv; st.d = sd;
-    sst.n = 0; sst.cap = kStageK; sst.vmin = kInf; sst.v = ssv; sst.d = nullptr;
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const Queue qa = make_queue(a.aent, a.aown, &c->acnt, a.asv, &c->ascnt, &st, &sst);
-  u64 dummy = 0;
-  const u32 n = (u32)a.n;
-  const u32 step = gridDim.x * blockDim.x;
-  for (u32 base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < n; base += step) {
-    const u32 v = base + lane;
-    bool want[K] = {};
-    u32 x[K] = {};
-    x[0] = v;
-    if (v < n) want[0] = all || __ldcg(a.prflag + v) == a.ptag;
-    const bool z = want[0] && __ldg(&a.rev.row[v].deg) == 0;
-    const u32 bal = __ballot_sync(kFull, z);
-    if (bal) {
-      u32 zb = 0;
-      if (lane == 0) zb = atomicAdd(&c->zcnt, (u32)__popc(bal));
-      zb = __shfl_sync(kFull, zb, 0);
-      if (z) a.jmp[zb + __popc(bal & lanemask_lt())] = v;
-    }
-    enqueue(qa, a.rev.row, x, want, 1, dummy);
-  }
-  flush_queue(qa, scratch);
-}
-
-__global__ void k_pr_fill(float *p0, float *p1, float *acc, int n, float value) {
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n;
-       v += (long long)gridDim.x * blockDim.x) {
-    p0[v] = value;
-    p1[v] = value;
-    acc[v] = 0.0f;
-  }
-}
-
-// Pull body of a Jacobi step: each lane adds the terms pr[u] / outdeg(u)
-// (kept per vertex in `contrib`, rounded exactly as a division per edge
-// would be) over its run of in-edges u -> v in slot order and adds the run's
-// sum to acc[v].  A vertex with at most kSmallDeg in-edges is one lane's
-// single run, so its sum is formed in in-neighbour order, as a sequential
-// loop would.
-struct PrOp {
-  const float *contrib;
-  float *acc;
-  u64 n_edges = 0, n_enq = 0;
-  int range_err = 0;
-
-  __device__ __forceinline__ u32 vdata(u32) { return 0; }
-  __device__ __forceinline__ u64 load(int2 e) { return __float_as_uint(__ldcg(contrib + e.x)); }
-  __device__ __forceinline__ void run(const bool *act, const u32 *ov, const u32 *,
-                                      const int2 *, const u64 *sx) {
-    u32 bv = kNoEdge;
-    float sum = 0.0f;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      if (act[k]) {
-        ++n_edges;
-        if (ov[k] != bv) {
-          if (bv != kNoEdge) atomicAdd(acc + bv, sum);
-          bv = ov[k];
-          sum = 0.0f;
-        }
-        sum = __fadd_rn(sum, __uint_as_float((u32)sx[k]));
-      }
-    }
-    if (bv != kNoEdge) atomicAdd(acc + bv, sum);
-  }
-};
-
-struct PrArgs {
-  LoopArgs la;
-  float *pr[2];
-  float *contrib[2];   // pr / outdeg, kept beside each rank buffer
-  float *acc;
-  float base, damping;
-  double beta;
-  int max_iter;
-};
-
-// Jacobi steps over the list A (persistent, cooperative): pass 1 pulls the
-// in-edge sums into acc, pass 2 forms pr' = base + damping * acc, adds
-// |pr' - pr| to the step's difference and clears acc; a step ends when the
-// difference is at most beta or max_iter steps have run.  The result is left
-// in both rank buffers.
-__device__ __forceinline__ double *prd_ptr(Ctl *c, u32 b) {
-  return b == 0 ? &c->prd0 : (b == 1 ? &c->prd1 : &c->prd2);
-}
-
-__global__ void __launch_bounds__(kPersistThreads, 1) k_pr(PrArgs p) {
-  const LoopArgs &a = p.la;
-  Ctl *c = a.ctl;
-  if (!repair_enabled_block(c)) return;
-  __shared__ double s_sum[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const u32 gw = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-  const u32 nw = (gridDim.x * blockDim.x) >> 5;
-  const u64 ac = ld_cg_u64(&c->acnt);
-  const u32 ne = (u32)(ac >> 32), nedge = (u32)ac;
-  const u32 ns = ld_cg_u32(&c->ascnt);
-  const u32 nz = ld_cg_u32(&c->zcnt);
-  const u32 sgroups = (ns + 31) / 32;
-  const u32 items = sgroups + (nedge + kChunk - 1) / kChunk;
-  u64 *bar = &c->bar_push;
-  u64 target = 0;
-  u64 n_edges = 0;
-  u32 it = 0, cur = 0;
-  bool stop = false;
-  {
-    // the terms of every vertex (out-degrees may have changed since the
-    // last phase); both rank buffers agree here
-    const u32 gt = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    for (u32 v = gt; v < (u32)a.n; v += nt) {
-      const int deg = __ldg(&a.fwd.row[v].deg);
-      const float t = deg > 0 ? __fdiv_rn(__ldcg(p.pr[0] + v), (float)deg) : 0.0f;
-      p.contrib[0][v] = t;
-      p.contrib[1][v] = t;
-    }
-    target += gridDim.x;
-    stop = grid_sync(bar, target, c, a.lim);
-  }
-  for (;;) {
-    if (stop) break;
-    // pass 1: in-edge sums
-    PrOp op{p.contrib[cur], p.acc};
-    for (u32 i = gw; i < items; i += nw) {
-      if (i < sgroups) process_small(op, a.asv, ns, i, a.rev, a.n, c);
-      else process_chunk(op, a.aent, a.aown, ne, nedge, i - sgroups, a.rev, a.n, c);
-    }
-    n_edges += op.n_edges;
-    target += gridDim.x;
-    stop = grid_sync(bar, target, c, a.lim);
-    if (stop) break;
-    // pass 2: new ranks and the step's difference
-    const float *pc = p.pr[cur];
-    float *pn = p.pr[cur ^ 1];
-    if (blockIdx.x == 0 && threadIdx.x == 0) *(volatile double *)prd_ptr(c, (it + 1) % 3) = 0.0;
-    double diff = 0.0;
-    const u32 gt = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    for (u32 i = gt; i < ns + ne + nz; i += nt) {
-      const u32 v = i < ns ? __ldcg(a.asv + i)
-                           : (i < ns + ne ? (u32)__ldcg(&a.aent[i - ns].x) : __ldcg(a.jmp + (i - ns - ne)));
-      const float val = __fadd_rn(p.base, __fmul_rn(p.damping, __ldcg(p.acc + v)));
-      diff += fabs((double)val - (double)__ldcg(pc + v));
-      pn[v] = val;
-      const int deg = __ldg(&a.fwd.row[v].deg);
-      p.contrib[cur ^ 1][v] = deg > 0 ? __fdiv_rn(val, (float)deg) : 0.0f;
-      p.acc[v] = 0.0f;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) diff += __shfl_xor_sync(kFull, diff, o);
-    if (lane == 0) s_sum[warp] = diff;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s_sum[w];
-      if (t != 0.0) atomicAdd(prd_ptr(c, it % 3), t);
-    }
-    target += gridDim.x;
-    stop = grid_sync(bar, target, c, a.lim);
-    if (stop) break;
-    const double d = *(volatile double *)prd_ptr(c, it % 3);
-    ++it;
-    cur ^= 1;
-    if (!(d > p.beta) || it >= (u32)p.max_iter) break;
-  }
-  // leave the result in both buffers
-  if (!stop) {
-    const float *src = p.pr[cur];
-    float *dst = p.pr[cur ^ 1];
-    const u32 gt = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    for (u32 i = gt; i < ns + ne + nz; i += nt) {
-      const u32 v = i < ns ? __ldcg(a.asv + i)
-                           : (i < ns + ne ? (u32)__ldcg(&a.aent[i - ns].x) : __ldcg(a.jmp + (i - ns - ne)));
-      dst[v] = __ldcg(src + v);
-    }
-  }
-  n_edges = warp_sum(n_edges);
-  if (lane == 0 && n_edges) atomicAdd(&c->pull_edges, n_edges);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    volatile Ctl *vc = c;
-    vc->pr_iters = it;
-    vc->rounds_push = it;
-    vc->acnt = 0ull;
-    vc->ascnt = 0u;
-    vc->zcnt = 0u;
-  }
-}
-
 LoopArgs make_args(sp_graph *g) {
   LoopArgs a;
   a.ctl = g->ctl;
@@ -2530,46 +2199,6 @@ cudaError_t launch_flag(sp_graph *g, const int *dst, long long n, int *launches)
   a.del_dst = dst;
   a.n_del = n;
   return launch_loop(g, kOpFlag, a, launches, g->stream);
-}
-
-void launch_pr_fill(sp_graph *g, float value, int *launches) {
-  k_pr_fill<<<(unsigned)std::max(1, g->num_sms * 8), 256, 0, g->stream>>>(
-      g->pr[0], g->pr[1], g->pracc, g->n, value);
-  ++*launches;
-}
-
-void launch_pr_select(sp_graph *g, int all, int *launches) {
-  LoopArgs a = make_args(g);
-  k_pr_select<<<(unsigned)std::max(1, g->num_sms), kLoopThreads, 0, g->stream>>>(a, all);
-  ++*launches;
-}
-
-cudaError_t launch_pr(sp_graph *g, int *launches) {
-  PrArgs p;
-  p.la = make_args(g);
-  p.pr[0] = g->pr[0];
-  p.pr[1] = g->pr[1];
-  p.contrib[0] = g->prc[0];
-  p.contrib[1] = g->prc[1];
-  p.acc = g->pracc;
-  p.base = (1.0f - g->pr_damping) / (float)g->n;
-  p.damping = g->pr_damping;
-  p.beta = (double)g->pr_beta;
-  p.max_iter = g->pr_max_iter;
-  int blocks = g->num_sms;
-  if (g->loop_blocks_user > 0 && g->loop_blocks_user < blocks) blocks = g->loop_blocks_user;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks);
-  cfg.blockDim = dim3(kPersistThreads);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = g->stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  ++*launches;
-  return cudaLaunchKernelEx(&cfg, k_pr, p);
 }
 
 void launch_state_check(sp_graph *g, const int *dist_d, const int *parent_d, int src,

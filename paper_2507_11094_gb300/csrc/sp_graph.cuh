@@ -15,7 +15,6 @@ constexpr int kEdgesPerLane = kChunk / 32;
 // are expanded one lane per vertex; larger ones get edge ranges and chunks.
 constexpr int kSmallDeg = 8;
 constexpr int kLocalRoundCap = 4096;   // frontier edges of a single-block round
-constexpr int kLoopThreads = 1024;      // one-pass frontier kernels (pull, add)
 constexpr int kPersistThreads = 768;    // persistent fixedPoint loops: 80 registers a thread
 // the push loop with block-local relaxation: a sub-round expands about a
 // hundred pool entries per block, so fewer threads with more registers each
@@ -173,11 +172,14 @@ struct sp_graph {
   cudaEvent_t fork0_ev = nullptr, search_ev = nullptr;   // the search beside the sort
   cudaEvent_t ev_inval[2] = {nullptr, nullptr};
   bool last_beside = false;     // the last timed call ran the invalidation beside
-  // PageRank state (allocated by sp_pr_init): ranks in two buffers that
-  // agree between calls, the pull accumulators, phase flags and settings
-  float *pr[2] = {nullptr, nullptr};
-  float *prc[2] = {nullptr, nullptr};   // pr / outdeg (Jacobi work buffers)
-  float *pracc = nullptr;
+  // PageRank state (allocated by sp_pr_init): ranks, the steps' terms and
+  // their places, phase flags and settings
+  float *pr = nullptr;
+  float *prterm[2] = {nullptr, nullptr};
+  sp::u32 *prplace = nullptr;
+  void *prscratch = nullptr;
+  sp::u32 *prlist = nullptr;            // packed in-neighbour lists, or none
+  size_t prlist_bytes = 0;
   sp::u32 *prflag = nullptr;
   sp::u32 prtag = 0;
   int pr_state = 0;            // 0 = no ranks, 1 = valid
@@ -308,11 +310,11 @@ void launch_tc_static(sp_graph *g, int *launches);
 void launch_tc_batch_sym(sp_graph *g, long long nb, int *launches);
 void launch_tc_tasks(sp_graph *g, long long nb, int *launches);
 void launch_tc_delta(sp_graph *g, long long nb, int kind, int *launches);
-// PageRank
+// sp_pr.cu: PageRank
+sp_status pr_alloc(sp_graph *g);
+void pr_free(sp_graph *g);
+cudaError_t launch_pr(sp_graph *g, int all, float init, int *launches);
 cudaError_t launch_flag(sp_graph *g, const int *dst, long long n, int *launches);
-void launch_pr_fill(sp_graph *g, float value, int *launches);
-void launch_pr_select(sp_graph *g, int all, int *launches);
-cudaError_t launch_pr(sp_graph *g, int *launches);
 void launch_gather(sp_graph *g, const int *vs_d, int k, int *out_d, int *launches);
 
 }  // namespace sp

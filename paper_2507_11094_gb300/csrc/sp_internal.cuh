@@ -112,7 +112,6 @@ struct Ctl {
   alignas(128) double prd1;
   alignas(128) double prd2;
   u32 pr_iters;
-  u32 zcnt;              // selected vertices without in-edges (PageRank)
   // triangle count: staticTC, and the sightings of the deletions' and the
   // insertions' corrections by number of updated edges (1, 2, 3)
   alignas(128) u64 tc_static;

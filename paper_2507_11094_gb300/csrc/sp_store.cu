@@ -196,7 +196,6 @@ __global__ void k_ctl_reset(Ctl *c, int full) {
   c->jcnt0 = c->jcnt1 = c->jcnt2 = 0;
   c->prd0 = c->prd1 = c->prd2 = 0.0;
   c->pr_iters = 0;
-  c->zcnt = 0;
   c->tc_static = 0;
   c->tc_ngiant = c->tc_nbig = c->tc_bpos = c->tc_spos = 0;
   c->tc_ntask[0] = c->tc_ntask[1] = c->tc_tpos[0] = c->tc_tpos[1] = 0;

@@ -146,3 +146,79 @@ def test_pagerank_and_sssp_states():
         assert e.value.code == sp.SP_ESTATE
         with pytest.raises(sp.SpError):
             g.pr_init(1.5, BETA, ITERS)
+
+
+def ranks64(n, u, v, iters):
+    """`iters` Jacobi steps over every vertex, in 64 bits (with the 32-bit
+    damping the call takes)."""
+    d = float(np.float32(D))
+    od = np.bincount(u, minlength=n).astype(np.float64)
+    pr = np.full(n, 1.0 / n)
+    for _ in range(iters):
+        term = np.divide(pr, od, out=np.zeros(n), where=od > 0)
+        pr = (1.0 - d) / n + d * np.bincount(v, weights=term[u], minlength=n)
+    return pr
+
+
+# Rows at the bounds of the in-degree classes (a lane's 8, a group's 64, a
+# warp's 1,024, and cut into one to six segments), more vertices than terms in
+# shared memory, and out-degrees that fill those in part, exactly by one
+# out-degree bin, or not at all.  Each step rounds a sum of terms over a tree
+# (at most eight 4-term words a lane, five levels, six parts: under 32 units
+# of 2^-24), and later steps damp it by d: under 32 / (1 - d) * 2^-24 = 1.3e-5.
+@pytest.mark.parametrize("n,extra", [(3000, 0), (7001, 20000), (60000, 150000), (200000, 0),
+                                     (200000, 700000)])
+def test_rows_of_every_class(n, extra):
+    rng = np.random.default_rng(n + extra)
+    degs = [1, 3, 4, 5, 8, 9, 31, 32, 33, 63, 64, 65, 127, 128, 129, 1023, 1024, 1025, 2047, 2048,
+            2049, 2999] + ([6000, 6145] if n > 6200 else [])
+    keys = [rng.choice(n - 1, size=d, replace=False) for d in degs]
+    u = np.concatenate([np.where(k >= 7 * i, k + 1, k) for i, k in enumerate(keys)])
+    v = np.repeat(7 * np.arange(len(degs)), degs)
+    u = np.concatenate([u, rng.integers(0, n, extra)])
+    v = np.concatenate([v, rng.integers(0, n, extra)])
+    key = np.unique(u.astype(np.int64) * n + v)
+    u, v = key // n, key % n
+    ro = np.zeros(n + 1, np.int64)
+    np.cumsum(np.bincount(u, minlength=n), out=ro[1:])
+    with sp.Graph(n, ro, v.astype(np.int32), np.ones(v.size, np.int32)) as g:
+        for iters in (1, 2, 9):
+            st = g.pr_init(D, 0.0, iters, stats=True)
+            assert st.rounds_push <= iters and st.relaxed_edges == v.size * st.rounds_push
+            np.testing.assert_allclose(g.pr_get(), ranks64(n, u, v, iters), rtol=2e-5)
+        # the same ranks bit for bit: a step's sums do not depend on the schedule
+        a = g.pr_get()
+        g.pr_init(D, 0.0, 9)
+        np.testing.assert_array_equal(g.pr_get(), a)
+
+
+def test_lists_without_memory_of_their_own():
+    # the packed in-neighbour lists do not fit: they go to the store's
+    # alternate regions, with the same ranks, and batches keep working
+    W = wl.rmat(12, batch_frac=0.02, seed=8)
+    state = {"refuse": False, "refused": 0}
+
+    def refuse(nbytes):
+        if state["refuse"] and nbytes >= 4 * W.m:
+            state["refused"] += 1
+            return True
+        return False
+    with sp.Graph(W.n, W.row_off, W.col, W.w) as g:
+        g.pr_init(D, BETA, ITERS)
+        want = g.pr_get()
+        b = W.batch(0)
+        g.pr_apply(b)
+        after = g.pr_get()
+    with sp.Graph(W.n, W.row_off, W.col, W.w, refuse_alloc=refuse) as g:
+        g.reserve(4096)
+        state["refuse"] = True
+        g.pr_init(D, BETA, ITERS)
+        assert state["refused"] > 0
+        np.testing.assert_array_equal(g.pr_get(), want)
+        g.pr_apply(b)
+        np.testing.assert_array_equal(g.pr_get(), after)
+        state["refuse"] = False
+        ref = oracle.OracleGraph(W.n, W.row_off, W.col, W.w)
+        ref.apply(b)
+        for x, y in zip(g.export_csr(), ref.csr()):
+            np.testing.assert_array_equal(x, y)
