@@ -638,8 +638,9 @@ sp_status sp_graph_create(int32_t n, int64_t m, const int64_t *row_off, const in
     w_d = ww;
   }
   sp_status rc = sp::csr_validate(g, ro_d, col_d, w_d, m, &launches);
-  if (rc == SP_OK) rc = sp::store_build(g, &g->fwd, ro_d, col_d, w_d, m, 0, &launches);
-  if (rc == SP_OK) rc = sp::store_build(g, &g->rev, ro_d, col_d, w_d, m, 1, &launches);
+  bool in_order = true;
+  if (rc == SP_OK) rc = sp::store_build(g, &g->fwd, ro_d, col_d, w_d, m, 0, &in_order, &launches);
+  if (rc == SP_OK) rc = sp::store_build(g, &g->rev, ro_d, col_d, w_d, m, 1, &in_order, &launches);
   if (rc == SP_OK) rc = sp::ensure_owner_tables(g);
   if (tmp_in) g->al.put(tmp_in, tmp_in_bytes);
   unsigned long long deg_mid = 0;

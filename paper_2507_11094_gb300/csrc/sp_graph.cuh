@@ -242,7 +242,7 @@ namespace sp {
 // sp_store.cu
 sp_status store_build(sp_graph *g, sp::Store *st, const long long *row_off_d,
                       const int *col_d, const int *w_d, long long m, int reverse,
-                      int *launches);
+                      bool *in_order, int *launches);
 sp_status store_export(sp_graph *g, const sp::Store *st, long long *row_off_d,
                        int *col_d, int *w_d, int *launches);
 sp_status store_grow_pool(sp_graph *g, sp::Store *st, long long min_pool_slots);

@@ -306,11 +306,11 @@ void scan_exclusive_u32(const u32 *in, u32 *out, long long n, void *tmp,
 void scan_exclusive_u64(const u64 *in, u64 *out, long long n, void *tmp,
                         cudaStream_t st, int *launches);
 
-// LSD radix sort of (u64 key, u32 value) pairs on the low `key_bits` bits
-// (sp_sort.cu).  Sorts keys/vals in place using alt buffers of the same size
-// and `tmp` of sort_tmp_bytes(n).  Stable.
+// Stable LSD radix sort of (u64 key, u32 value) pairs on the key bits
+// [lo_bit, hi_bit) (sp_sort.cu), with alt buffers of the same size and `tmp`
+// of sort_tmp_bytes(n).  Returns whether the result is in the alt buffers.
 size_t sort_tmp_bytes(long long n);
-void sort_pairs(u64 *keys, u32 *vals, u64 *keys_alt, u32 *vals_alt, long long n,
-                int key_bits, void *tmp, cudaStream_t st, int *launches);
+bool sort_pairs(u64 *keys, u32 *vals, u64 *keys_alt, u32 *vals_alt, long long n, int lo_bit,
+                int hi_bit, void *tmp, cudaStream_t st, int *launches);
 
 }  // namespace sp

@@ -4,16 +4,21 @@
 // merged once (updateCSRDel / updateCSRAdd of the DynSSSP driver, done as a
 // sort-merge), and orders graph edges when a store is built.
 //
-// Per 9-bit digit:
-//   k_hist       per-tile digit counts (count table is digit-major), for the
-//                first digit only;
+// The edge sort, per digit of at most 8 bits, over tiles of 4,096 pairs:
+//   k_hist       a tile's digit counts (the count table is digit-major);
 //   k_digit_scan one block per digit: prefix of its counts over the tiles,
-//                and the digit's total; it also clears the other count table;
-//   k_scatter    digit bases from the totals (block scan), then a stable
-//                in-tile rank with warp match_any + per-warp digit counters;
-//                every item it places also counts the next digit for the
-//                output tile it lands in (into the other table), which
-//                replaces the next pass's k_hist.
+//                and the digit's total;
+//   k_scatter    digit bases from the totals, a stable rank of the tile's
+//                pairs (ballots per digit bit, warp-private digit counters),
+//                the pairs staged in shared memory in digit order, and runs of
+//                a digit written out by consecutive threads.
+// What bounds a pass is its 24 bytes per pair of reads and writes, if the runs
+// are long enough to fill sectors: a tile of 4,096 has 16 or more pairs per
+// digit.  16.8 M pairs (R-MAT 20's reverse store, three 7-bit passes because
+// the input is in row order already): 2.3 -> 0.43 ms, a scatter 190-470 ->
+// 110 us (3.6 TB/s), against five passes over tiles of 1,024 pairs with 512
+// bins: two pairs a run, the next digit counted by 16.8 M global atomics a
+// pass and a count table of 33 MB.
 #include "sp_graph.cuh"
 
 #include <algorithm>
@@ -22,37 +27,35 @@ namespace sp {
 
 namespace {
 
-constexpr int kBits = 9;
+constexpr int kBits = 9;               // digits of the batch sort
 constexpr int kBins = 1 << kBits;
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kItems = 4;
-constexpr int kTile = kThreads * kItems;
-constexpr int kBinsPerThread = kBins / kThreads;
+constexpr int kMaxDigit = 8;           // digits of the edge sort
+constexpr int kSBins = 1 << kMaxDigit;
+constexpr int kST = 512;               // its threads per block,
+constexpr int kSW = kST / 32;
+constexpr int kSItems = 8;             // pairs per thread
+constexpr int kSTile = kST * kSItems;  // and pairs per tile
 
-__global__ void __launch_bounds__(kThreads)
-k_hist(const u64 *__restrict__ keys, long long n, int shift, u32 *__restrict__ counts,
+__global__ void __launch_bounds__(kST)
+k_hist(const u64 *__restrict__ keys, long long n, int shift, int bins, u32 *__restrict__ counts,
        u32 tiles) {
-  __shared__ u32 h[kBins];
-#pragma unroll
-  for (int j = 0; j < kBinsPerThread; ++j) h[threadIdx.x + j * kThreads] = 0;
+  __shared__ u32 h[kSBins];
+  if (threadIdx.x < kSBins) h[threadIdx.x] = 0;
   __syncthreads();
-  const long long base = (long long)blockIdx.x * kTile;
-  u32 d[kItems];
+  const long long base = (long long)blockIdx.x * kSTile;
+  u32 d[kSItems];
 #pragma unroll
-  for (int k = 0; k < kItems; ++k) {   // all loads first, then the counts
-    long long i = base + k * kThreads + threadIdx.x;
-    d[k] = i < n ? (u32)((keys[i] >> shift) & (kBins - 1)) : 0xFFFFFFFFu;
+  for (int k = 0; k < kSItems; ++k) {   // all loads first, then the counts
+    const long long i = base + k * kST + threadIdx.x;
+    d[k] = i < n ? (u32)(keys[i] >> shift) & (u32)(bins - 1) : 0xFFFFFFFFu;
   }
 #pragma unroll
-  for (int k = 0; k < kItems; ++k)
+  for (int k = 0; k < kSItems; ++k)
     if (d[k] != 0xFFFFFFFFu) atomicAdd(&h[d[k]], 1u);
   __syncthreads();
-#pragma unroll
-  for (int j = 0; j < kBinsPerThread; ++j) {
-    const int b = threadIdx.x + j * kThreads;
-    counts[(long long)b * tiles + blockIdx.x] = h[b];
-  }
+  if ((int)threadIdx.x < bins) counts[(long long)threadIdx.x * tiles + blockIdx.x] = h[threadIdx.x];
 }
 
 __device__ __forceinline__ u32 warp_incl_scan(u32 x) {
@@ -84,16 +87,11 @@ __device__ __forceinline__ u32 block_excl_scan(u32 x, u32 *ws, u32 *total) {
 }
 
 // Block d: exclusive prefix of counts[d][0..tiles) in place, total to
-// totals[d]; clears row d of `clear` (the next pass's table) when given.
+// totals[d].
 __global__ void __launch_bounds__(kThreads)
-k_digit_scan(u32 *__restrict__ counts, u32 tiles, u32 *__restrict__ totals,
-             u32 *__restrict__ clear) {
+k_digit_scan(u32 *__restrict__ counts, u32 tiles, u32 *__restrict__ totals) {
   __shared__ u32 ws[kWarps];
   u32 *row = counts + (long long)blockIdx.x * tiles;
-  if (clear) {
-    u32 *crow = clear + (long long)blockIdx.x * tiles;
-    for (u32 i = threadIdx.x; i < tiles; i += kThreads) crow[i] = 0;
-  }
   const u32 per = (tiles + kThreads - 1) / kThreads;
   const u32 b = threadIdx.x * per < tiles ? threadIdx.x * per : tiles;
   const u32 e = b + per < tiles ? b + per : tiles;
@@ -109,84 +107,124 @@ k_digit_scan(u32 *__restrict__ counts, u32 tiles, u32 *__restrict__ totals,
   if (threadIdx.x == 0) totals[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(kThreads)
-k_scatter(const u64 *__restrict__ keys, const u32 *__restrict__ vals, long long n, int shift,
-          const u32 *__restrict__ offs, const u32 *__restrict__ totals, u32 tiles,
-          u64 *__restrict__ keys_out, u32 *__restrict__ vals_out, u32 *__restrict__ next_counts,
-          int next_shift) {
-  __shared__ u32 s_off[kBins];
-  __shared__ u32 s_run[kBins];
-  __shared__ u32 s_cnt[2][kWarps][kBins];
-  __shared__ u32 ws[kWarps];
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const long long base = (long long)blockIdx.x * kTile;
-  u64 rk[kItems];
-  u32 rv[kItems];
-#pragma unroll
-  for (int k = 0; k < kItems; ++k) {   // the whole tile is in flight at once
-    const long long i = base + k * kThreads + t;
-    rk[k] = i < n ? keys[i] : 0ull;
-    rv[k] = i < n ? vals[i] : 0u;
-  }
-  // digit bases: exclusive scan of the digit totals (each thread owns
-  // kBinsPerThread consecutive digits)
-  {
-    u32 tot[kBinsPerThread], sum = 0;
-#pragma unroll
-    for (int j = 0; j < kBinsPerThread; ++j) {
-      tot[j] = totals[t * kBinsPerThread + j];
-      sum += tot[j];
-    }
-    u32 all;
-    u32 run = block_excl_scan(sum, ws, &all);
-#pragma unroll
-    for (int j = 0; j < kBinsPerThread; ++j) {
-      const int dgt = t * kBinsPerThread + j;
-      s_off[dgt] = run + offs[(long long)dgt * tiles + blockIdx.x];
-      run += tot[j];
-      s_run[dgt] = 0;
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < kBinsPerThread; ++j)
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) s_cnt[0][w][t + j * kThreads] = 0;
+// Block-wide exclusive scan over 512 threads.
+__device__ __forceinline__ u32 bscan512(u32 x, u32 *ws, u32 *total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u32 incl = warp_incl_scan(x);
+  if (lane == 31) ws[warp] = incl;
   __syncthreads();
+  if (warp == 0) {
+    u32 v = lane < kSW ? ws[lane] : 0u;
+    v = warp_incl_scan(v);
+    if (lane < kSW) ws[lane] = v;
+  }
+  __syncthreads();
+  const u32 r = (warp ? ws[warp - 1] : 0u) + incl - x;
+  *total = ws[kSW - 1];
+  __syncthreads();
+  return r;
+}
+
+// Lanes of the warp whose valid item has the same kB-bit digit (the answer of
+// a match_any, built from one ballot per digit bit).
+template <int kB>
+__device__ __forceinline__ u32 digit_peers(u32 d, bool valid) {
+  u32 peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+  for (int bb = 0; bb < kB; ++bb) {
+    const bool on = (d >> bb) & 1;
+    const u32 bal = __ballot_sync(0xffffffffu, on);
+    peers &= on ? bal : ~bal;
+  }
+  return peers;
+}
+
+constexpr size_t kSSmem = (size_t)kSTile * (sizeof(u64) + sizeof(u32));
+
+__global__ void __launch_bounds__(kST, 2)
+k_scatter(const u64 *__restrict__ keys, const u32 *__restrict__ vals, long long n, int shift,
+          int bins, const u32 *__restrict__ offs, const u32 *__restrict__ totals, u32 tiles,
+          u64 *__restrict__ keys_out, u32 *__restrict__ vals_out) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  u64 *s_key = (u64 *)smraw;                  // [kSTile]
+  u32 *s_val = (u32 *)(s_key + kSTile);       // [kSTile]
+  __shared__ u32 s_wc[kSW][kSBins];           // digit counts of each warp, then its offsets
+  __shared__ u32 s_off[kSBins];               // where the tile's run of a digit goes, less its
+                                              // place in the tile
+  __shared__ u32 ws[kSW];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const long long base = (long long)blockIdx.x * kSTile;
+  const u32 left = (u32)(n - base < kSTile ? n - base : kSTile);
+  const u32 w0 = (u32)warp * (32 * kSItems);
+  u64 rk[kSItems];
+  u32 rv[kSItems], lr[kSItems];
+#pragma unroll
+  for (int k = 0; k < kSItems; ++k) {   // the whole tile is in flight at once
+    const u32 i = w0 + k * 32 + lane;
+    rk[k] = i < left ? __ldcs(keys + base + i) : 0ull;
+    rv[k] = i < left ? __ldcs(vals + base + i) : 0u;
+  }
+#pragma unroll
+  for (int w = 0; w < kSW * kSBins / kST; ++w) ((u32 *)s_wc)[w * kST + t] = 0;
+  u32 tot_d = 0, off_d = 0;
+  if (t < bins) {
+    tot_d = totals[t];
+    off_d = offs[(long long)t * tiles + blockIdx.x];
+  }
+  u32 all;
+  off_d += bscan512(tot_d, ws, &all);   // (its barriers order the clearing, too)
+  // stable rank within the warp's pairs (rows k, then lanes)
   const u32 lt = lanemask_lt();
+  u32 *wc = s_wc[warp];
 #pragma unroll
-  for (int k = 0; k < kItems; ++k) {
-    const int p = k & 1;
-    const long long i = base + k * kThreads + t;
-    const bool valid = i < n;
-    const u64 key = rk[k];
-    const u32 val = rv[k];
-    u32 d = valid ? (u32)((key >> shift) & (kBins - 1)) : (u32)(kBins + lane);
-    u32 peers = __match_any_sync(0xffffffffu, d);
-    u32 rank = __popc(peers & lt);
-    if (valid && rank == 0) s_cnt[p][warp][d] = __popc(peers);
-    __syncthreads();
+  for (int k = 0; k < kSItems; ++k) {
+    const bool valid = w0 + k * 32 + lane < left;
+    const u32 d = (u32)(rk[k] >> shift) & (u32)(bins - 1);
+    const u32 peers = digit_peers<kMaxDigit>(d, valid);
+    const u32 rank = __popc(peers & lt);
+    const u32 before = valid ? wc[d] : 0u;
+    __syncwarp();
+    if (valid && rank == 0) wc[d] = before + __popc(peers);
+    __syncwarp();
+    lr[k] = before + rank;
+  }
+  __syncthreads();
+  {   // digit t: offsets of the warps, then of the digit in the tile
+    u32 run = 0;
+    if (t < kSBins) {
 #pragma unroll
-    for (int j = 0; j < kBinsPerThread; ++j) {   // digit-owners: scan over warps
-      const int dgt = t + j * kThreads;
-      u32 run = s_run[dgt];
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) {
-        u32 c = s_cnt[p][w][dgt];
-        s_cnt[p][w][dgt] = run;
-        run += c;
-        s_cnt[p ^ 1][w][dgt] = 0;
+      for (int w = 0; w < kSW; ++w) {
+        const u32 x = s_wc[w][t];
+        s_wc[w][t] = run;
+        run += x;
       }
-      s_run[dgt] = run;
     }
-    __syncthreads();
-    if (valid) {
-      u32 pos = s_off[d] + s_cnt[p][warp][d] + rank;
+    const u32 loc = bscan512(run, ws, &all);
+    if (t < kSBins) {
+#pragma unroll
+      for (int w = 0; w < kSW; ++w) s_wc[w][t] += loc;
+      s_off[t] = off_d - loc;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kSItems; ++k) {
+    if (w0 + k * 32 + lane < left) {
+      const u32 d = (u32)(rk[k] >> shift) & (u32)(bins - 1);
+      const u32 lp = wc[d] + lr[k];
+      s_key[lp] = rk[k];
+      s_val[lp] = rv[k];
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kSItems; ++k) {
+    const u32 j = k * kST + t;
+    if (j < left) {
+      const u64 key = s_key[j];
+      const u32 pos = s_off[(u32)(key >> shift) & (u32)(bins - 1)] + j;
       keys_out[pos] = key;
-      vals_out[pos] = val;
-      if (next_counts) {
-        const u32 nd = (u32)((key >> next_shift) & (kBins - 1));
-        atomicAdd(next_counts + (long long)nd * tiles + pos / kTile, 1u);
-      }
+      vals_out[pos] = s_val[j];
     }
   }
 }
@@ -220,6 +258,7 @@ constexpr int kBItems = 8;
 constexpr int kBTile = kBT * kBItems;     // items per sub-tile
 constexpr int kBWarpItems = 32 * kBItems; // items per warp and sub-tile
 static_assert(kBT == kBins, "one digit per thread");
+static_assert(kBT == kST, "bscan512");
 // dynamic shared memory: staged keys and values, per-warp digit counters,
 // four per-digit arrays
 constexpr size_t kBSmem =
@@ -238,37 +277,6 @@ struct BatchSortArgs {
   u32 miss_site;         // test hook of the bounded waits (Limits::miss_site)
   u32 n_items, chunk;
 };
-
-// Block-wide exclusive scan over kBT threads.
-__device__ __forceinline__ u32 bscan512(u32 x, u32 *ws, u32 *total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const u32 incl = warp_incl_scan(x);
-  if (lane == 31) ws[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    u32 v = lane < kBW ? ws[lane] : 0u;
-    v = warp_incl_scan(v);
-    if (lane < kBW) ws[lane] = v;
-  }
-  __syncthreads();
-  const u32 r = (warp ? ws[warp - 1] : 0u) + incl - x;
-  *total = ws[kBW - 1];
-  __syncthreads();
-  return r;
-}
-
-// Lanes of the warp whose valid item has the same 9-bit digit (the answer of
-// a match_any, built from one ballot per digit bit).
-__device__ __forceinline__ u32 digit_peers(u32 d, bool valid) {
-  u32 peers = __ballot_sync(0xffffffffu, valid);
-#pragma unroll
-  for (int bb = 0; bb < kBits; ++bb) {
-    const bool on = (d >> bb) & 1;
-    const u32 bal = __ballot_sync(0xffffffffu, on);
-    peers &= on ? bal : ~bal;
-  }
-  return peers;
-}
 
 __device__ __forceinline__ u64 shfl64_up1(u64 x) {
   const u32 lo = __shfl_up_sync(0xffffffffu, (u32)x, 1);
@@ -429,7 +437,7 @@ __global__ void __launch_bounds__(kBT) k_batch_sort(BatchSortArgs a) {
       for (int k = 0; k < kBItems; ++k) {
         const bool valid = tb + sub_pos(k) < ce;
         const u32 d = (u32)((rk[k] >> shift) & (kBins - 1));
-        const u32 peers = digit_peers(d, valid);
+        const u32 peers = digit_peers<kBits>(d, valid);
         const u32 rank = __popc(peers & lt);
         const u32 before = valid ? wc[d] : 0u;
         __syncwarp();
@@ -596,9 +604,8 @@ __global__ void __launch_bounds__(kBT) k_batch_sort(BatchSortArgs a) {
 }  // namespace
 
 size_t sort_tmp_bytes(long long n) {
-  long long tiles = (n + kTile - 1) / kTile;
-  long long cnt = tiles * kBins;
-  return (size_t)(2 * cnt + kBins + 64) * sizeof(u32) + 256;
+  const long long tiles = (n + kSTile - 1) / kSTile;
+  return (size_t)(tiles * kSBins + kSBins + 64) * sizeof(u32) + 256;
 }
 
 int batch_sort_blocks(int num_sms) {
@@ -693,33 +700,30 @@ cudaError_t retarget_batch_sort(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t
   return cudaGraphExecKernelNodeSetParams(ex, node, &p);
 }
 
-void sort_pairs(u64 *keys, u32 *vals, u64 *keys_alt, u32 *vals_alt, long long n,
-                int key_bits, void *tmp, cudaStream_t st, int *launches) {
-  if (n <= 1 || key_bits <= 0) return;
-  const u32 tiles = (u32)((n + kTile - 1) / kTile);
-  const long long cnt = (long long)tiles * kBins;
-  u32 *counts[2] = {(u32 *)tmp, (u32 *)tmp + cnt};
-  u32 *totals = counts[1] + cnt;
+bool sort_pairs(u64 *keys, u32 *vals, u64 *keys_alt, u32 *vals_alt, long long n, int lo_bit,
+                int hi_bit, void *tmp, cudaStream_t st, int *launches) {
+  const int bits = hi_bit - lo_bit;
+  if (n <= 1 || bits <= 0) return false;
+  const u32 tiles = (u32)((n + kSTile - 1) / kSTile);
+  u32 *counts = (u32 *)tmp;
+  u32 *totals = counts + (long long)tiles * kSBins;
   u64 *kin = keys, *kout = keys_alt;
   u32 *vin = vals, *vout = vals_alt;
-  int passes = (key_bits + kBits - 1) / kBits;
-  k_hist<<<tiles, kThreads, 0, st>>>(kin, n, 0, counts[0], tiles);
-  if (launches) *launches += 1;
-  for (int pass = 0; pass < passes; ++pass) {
-    const int shift = pass * kBits;
-    const bool more = pass + 1 < passes;
-    u32 *cur = counts[pass & 1], *nxt = more ? counts[(pass + 1) & 1] : nullptr;
-    k_digit_scan<<<kBins, kThreads, 0, st>>>(cur, tiles, totals, nxt);
-    k_scatter<<<tiles, kThreads, 0, st>>>(kin, vin, n, shift, cur, totals, tiles, kout, vout, nxt,
-                                          shift + kBits);
-    if (launches) *launches += 2;
-    u64 *tk = kin; kin = kout; kout = tk;
-    u32 *tv = vin; vin = vout; vout = tv;
+  // as few passes as kMaxDigit allows, of equal digits
+  const int passes = (bits + kMaxDigit - 1) / kMaxDigit;
+  const int digit = (bits + passes - 1) / passes;
+  cudaFuncSetAttribute(k_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSSmem);
+  for (int shift = lo_bit; shift < hi_bit; shift += digit) {
+    const int bins = 1 << std::min(digit, hi_bit - shift);
+    k_hist<<<tiles, kST, 0, st>>>(kin, n, shift, bins, counts, tiles);
+    k_digit_scan<<<bins, kThreads, 0, st>>>(counts, tiles, totals);
+    k_scatter<<<tiles, kST, kSSmem, st>>>(kin, vin, n, shift, bins, counts, totals, tiles, kout,
+                                          vout);
+    if (launches) *launches += 3;
+    std::swap(kin, kout);
+    std::swap(vin, vout);
   }
-  if (kin != keys) {
-    cudaMemcpyAsync(keys, kin, (size_t)n * sizeof(u64), cudaMemcpyDeviceToDevice, st);
-    cudaMemcpyAsync(vals, vin, (size_t)n * sizeof(u32), cudaMemcpyDeviceToDevice, st);
-  }
+  return kin != keys;
 }
 
 }  // namespace sp
