@@ -235,7 +235,7 @@ bool find_input_nodes(sp_graph *g) {
     if (cudaGraphKernelNodeGetParams(nd, &p) != cudaSuccess) return false;
     if (p.func == sp::batch_sort_fn()) g->bg_sort = nd;
     else if (p.func == sp::inval_fn()) g->bg_inval = nd;
-    else if (p.func == sp::search_fn()) g->bg_search = nd;
+    else if (p.func == sp::search_fn(g)) g->bg_search = nd;
   }
   return g->bg_sort != nullptr && g->bg_search != nullptr;
 }

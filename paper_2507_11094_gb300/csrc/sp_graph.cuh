@@ -269,7 +269,7 @@ const void *batch_sort_fn();
 cudaError_t launch_search(sp_graph *g, const int *ds, const int *dd, long long nd,
                           const int *as, const int *ad, const int *aw, long long na,
                           int *launches, cudaStream_t stream);
-const void *search_fn();
+const void *search_fn(const sp_graph *g);
 cudaError_t retarget_search(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t node,
                             const int *ds, const int *dd, long long nd, const int *as,
                             const int *ad, const int *aw, long long na);

@@ -12,7 +12,7 @@
 #include <algorithm>
 #include <cstddef>
 
-#include "sp_graph.cuh"
+#include "sp_search.cuh"
 
 namespace sp {
 
@@ -693,11 +693,13 @@ struct SearchArgs {
 // edge is there), and its weight, into srch[i].  The stores do not change
 // before the merge, so this runs beside the sort; ids out of range (the sort
 // rejects the batch) get 0.  Each thread advances kCI searches in lockstep.
-__global__ void __launch_bounds__(kCT) k_search(SearchArgs a) {
+// kGuess: interpolating searches (row_search) in place of halving ones.
+template <bool kGuess>
+__global__ void __launch_bounds__(kCT, kGuess ? 3 : 4) k_search(SearchArgs a) {
   const long long nb = a.nd + a.na;
   const u32 ni = a.n_items;
   for (u32 tb = blockIdx.x * (u32)kCTile; tb < ni; tb += gridDim.x * (u32)kCTile) {
-    int col[kCI], lo[kCI], hi[kCI], deg[kCI];
+    int col[kCI], deg[kCI];
     u32 w[kCI];
     const int2 *old[kCI];
     bool val[kCI];
@@ -727,33 +729,47 @@ __global__ void __launch_bounds__(kCT) k_search(SearchArgs a) {
       rm.deg = 0;
       if (ok) rm = a.st[rev ? 1 : 0].row[row];
       old[k] = a.st[rev ? 1 : 0].adj + rm.start;
-      lo[k] = 0;
-      hi[k] = deg[k] = rm.deg;
+      deg[k] = rm.deg;
     }
-    for (;;) {   // binary searches in lockstep: every load of a step in flight together
-      bool act = false;
-      int mid[kCI], x[kCI];
+    u32 pos[kCI];
+    bool present[kCI];
+    if constexpr (kGuess) {
+      row_search<kCI>(old, deg, col, a.n, pos, present);
+    } else {   // halving, in lockstep: every load of a step in flight together
+      int lo[kCI], hi[kCI];
 #pragma unroll
       for (int k = 0; k < kCI; ++k) {
-        act |= lo[k] < hi[k];
-        mid[k] = (lo[k] + hi[k]) >> 1;
-        x[k] = lo[k] < hi[k] ? __ldg(&old[k][mid[k]].x) : 0;
+        lo[k] = 0;
+        hi[k] = deg[k];
       }
-      if (!act) break;
+      for (;;) {
+        bool act = false;
+        int mid[kCI], x[kCI];
 #pragma unroll
-      for (int k = 0; k < kCI; ++k)
-        if (lo[k] < hi[k]) {
-          if (x[k] < col[k]) lo[k] = mid[k] + 1; else hi[k] = mid[k];
+        for (int k = 0; k < kCI; ++k) {
+          act |= lo[k] < hi[k];
+          mid[k] = (lo[k] + hi[k]) >> 1;
+          x[k] = lo[k] < hi[k] ? __ldg(&old[k][mid[k]].x) : 0;
         }
+        if (!act) break;
+#pragma unroll
+        for (int k = 0; k < kCI; ++k)
+          if (lo[k] < hi[k]) {
+            if (x[k] < col[k]) lo[k] = mid[k] + 1; else hi[k] = mid[k];
+          }
+      }
+#pragma unroll
+      for (int k = 0; k < kCI; ++k) {
+        pos[k] = (u32)lo[k];
+        present[k] = (lo[k] < deg[k] ? __ldg(&old[k][lo[k]].x) : -1) == col[k];
+      }
     }
 #pragma unroll
-    for (int k = 0; k < kCI; ++k) {
-      const int cl = lo[k] < deg[k] ? __ldg(&old[k][lo[k]].x) : -1;
+    for (int k = 0; k < kCI; ++k)
       if (val[k]) {
         const u32 i = tb + (u32)(k * kCT) + threadIdx.x;
-        a.srch[i] = ((u64)w[k] << 32) | (cl == col[k] ? 0x80000000ull : 0ull) | (u32)lo[k];
+        a.srch[i] = ((u64)w[k] << 32) | (present[k] ? 0x80000000ull : 0ull) | pos[k];
       }
-    }
   }
 }
 
@@ -770,9 +786,21 @@ SearchArgs search_args(sp_graph *g, const int *ds, const int *dd, long long nd, 
   return a;
 }
 
+// The searches interpolate where the store is well beyond the L2: there they
+// are bound by random reads from DRAM (twice the threads made them slower),
+// and three rounds of reads take the place of ten.  A million updates on
+// R-MAT 22 (1.7 GB a store): search 355 -> 238 us, the batch 1.42 -> 1.25 ms.
+// In stores that the L2 half holds a halving step costs less than a guess:
+// R-MAT 20 (0.42 GB) 51 against 50 us, 32 small R-MATs (0.38 GB) 57 against
+// 71 us.
+bool search_guesses(const sp_graph *g) {
+  return std::max(g->fwd.slots, g->rev.slots) * (long long)sizeof(int2) >= (1LL << 30);
+}
+
 // One block of 256 threads per SM at most: beside it an SM still holds a
-// block of the batch sort (512 threads, 90-116 KB of shared memory, about
-// 45k registers), so the search never delays the sort's cooperative grid.
+// block of the batch sort (512 threads, 90-116 KB of shared memory, 45,056
+// registers; the search's 256 threads take 14,336 or 20,480), so the search
+// never delays the sort's cooperative grid.
 unsigned search_grid(const sp_graph *g, long long ni) {
   return blocks_for(ni, kCTile, std::max(1, g->num_sms));
 }
@@ -1481,12 +1509,16 @@ cudaError_t launch_search(sp_graph *g, const int *ds, const int *dd, long long n
                           int *launches, cudaStream_t stream) {
   const long long ni = 2 * (nd + na);
   if (ni == 0) return cudaSuccess;
-  k_search<<<search_grid(g, ni), kCT, 0, stream>>>(search_args(g, ds, dd, nd, as, ad, aw, na));
+  const SearchArgs a = search_args(g, ds, dd, nd, as, ad, aw, na);
+  if (search_guesses(g)) k_search<true><<<search_grid(g, ni), kCT, 0, stream>>>(a);
+  else k_search<false><<<search_grid(g, ni), kCT, 0, stream>>>(a);
   ++*launches;
   return cudaGetLastError();
 }
 
-const void *search_fn() { return (const void *)k_search; }
+const void *search_fn(const sp_graph *g) {
+  return search_guesses(g) ? (const void *)k_search<true> : (const void *)k_search<false>;
+}
 
 cudaError_t retarget_search(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t node,
                             const int *ds, const int *dd, long long nd, const int *as,
@@ -1494,7 +1526,7 @@ cudaError_t retarget_search(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t nod
   SearchArgs a = search_args(g, ds, dd, nd, as, ad, aw, na);
   void *args[1] = {&a};
   cudaKernelNodeParams p = {};
-  p.func = (void *)k_search;
+  p.func = const_cast<void *>(search_fn(g));
   p.gridDim = dim3(search_grid(g, 2 * (nd + na)));
   p.blockDim = dim3(kCT);
   p.sharedMemBytes = 0;
