@@ -210,7 +210,7 @@ void drop_batch_graphs(sp_graph *g) {
   if (g->bg_graph) cudaGraphDestroy(g->bg_graph);
   g->bg_exec = nullptr;
   g->bg_graph = nullptr;
-  g->bg_sort = g->bg_inval = g->bg_search = nullptr;
+  g->bg_sort = g->bg_inval = g->bg_search = g->bg_plan = g->bg_check = nullptr;
   g->bg_ready = false;
 }
 
@@ -220,10 +220,11 @@ void drop_batch_graphs(sp_graph *g) {
 bool inval_beside(const sp_graph *g) { return g->side && g->lim.jump_round == 0; }
 
 // The kernel nodes of the captured batch graph that read the batch inputs:
-// the batch sort and the old-row searches (every input array) and the
-// invalidation loop (the deletions).  Every other kernel reads the sorted items.
+// the batch sort and the old-row searches (every input array; a small batch's
+// check and plan in their place) and the invalidation loop (the deletions).  Every other
+// kernel reads the sorted items.
 bool find_input_nodes(sp_graph *g) {
-  g->bg_sort = g->bg_inval = g->bg_search = nullptr;
+  g->bg_sort = g->bg_inval = g->bg_search = g->bg_plan = g->bg_check = nullptr;
   size_t nn = 0;
   if (cudaGraphGetNodes(g->bg_graph, nullptr, &nn) != cudaSuccess) return false;
   std::vector<cudaGraphNode_t> nodes(nn);
@@ -236,14 +237,20 @@ bool find_input_nodes(sp_graph *g) {
     if (p.func == sp::batch_sort_fn()) g->bg_sort = nd;
     else if (p.func == sp::inval_fn()) g->bg_inval = nd;
     else if (p.func == sp::search_fn(g)) g->bg_search = nd;
+    else if (p.func == sp::plan_fn()) g->bg_plan = nd;
+    else if (p.func == sp::check_small_fn()) g->bg_check = nd;
   }
-  return g->bg_sort != nullptr && g->bg_search != nullptr;
+  return (g->bg_plan != nullptr && g->bg_check != nullptr) ||
+         (g->bg_sort != nullptr && g->bg_search != nullptr);
 }
 
 cudaError_t retarget_input_nodes(sp_graph *g, const int *ds, const int *dd, long long nd,
                                  const int *as, const int *ad, const int *aw, long long na) {
-  cudaError_t e = sp::retarget_batch_sort(g, g->bg_exec, g->bg_sort, ds, dd, nd, as, ad, aw, na);
-  if (e == cudaSuccess)
+  cudaError_t e =
+      g->bg_plan ? sp::retarget_plan(g, g->bg_exec, g->bg_check, g->bg_plan, ds, dd, nd, as, ad,
+                                     aw, na)
+                 : sp::retarget_batch_sort(g, g->bg_exec, g->bg_sort, ds, dd, nd, as, ad, aw, na);
+  if (e == cudaSuccess && !g->bg_plan)
     e = sp::retarget_search(g, g->bg_exec, g->bg_search, ds, dd, nd, as, ad, aw, na);
   if (e == cudaSuccess && g->bg_inval)
     e = sp::retarget_inval(g, g->bg_exec, g->bg_inval, ds, dd, nd, inval_beside(g) ? 1 : 0);
@@ -316,11 +323,16 @@ cudaError_t enqueue_batch(sp_graph *g, const int *ds, const int *dd, long long n
                           const int *as, const int *ad, const int *aw, long long n_add,
                           bool timed, int *launches, int mode = kInvalAfter) {
   const long long ni = 2 * (n_del + n_add);
-  sp::launch_ctl_reset(g, mode == kInvalKept ? 2 : 0, launches);
+  const bool small = ni > 0 && sp::plan_small(g, ni);   // one block plans the store update
+  const int reset = mode == kInvalKept ? 2 : 0;
+  if (small) sp::launch_check_small(g, ds, dd, n_del, as, ad, aw, n_add, reset, launches);
+  else sp::launch_ctl_reset(g, reset, launches);
   // the items' searches in their old rows run beside the batch sort (on the
   // SMs the sort leaves free; they read only the inputs and the old stores)
   cudaError_t e = cudaSuccess;
-  if (g->side) {
+  if (small) {
+    // (its plan does them, below, beside the invalidation)
+  } else if (g->side) {
     cudaEventRecord(g->fork0_ev, g->stream);
     cudaStreamWaitEvent(g->side, g->fork0_ev, 0);
     e = sp::launch_search(g, ds, dd, n_del, as, ad, aw, n_add, launches, g->side);
@@ -328,10 +340,12 @@ cudaError_t enqueue_batch(sp_graph *g, const int *ds, const int *dd, long long n
   } else {
     e = sp::launch_search(g, ds, dd, n_del, as, ad, aw, n_add, launches, g->stream);
   }
-  const cudaError_t es = sp::launch_batch_sort(g, ds, dd, n_del, as, ad, aw, n_add, launches);
-  if (e == cudaSuccess) e = es;
+  if (!small) {
+    const cudaError_t es = sp::launch_batch_sort(g, ds, dd, n_del, as, ad, aw, n_add, launches);
+    if (e == cudaSuccess) e = es;
+  }
   rec(g, timed, 1);
-  if (g->side) cudaStreamWaitEvent(g->stream, g->search_ev, 0);
+  if (!small && g->side) cudaStreamWaitEvent(g->stream, g->search_ev, 0);
   const bool beside = mode == kInvalBeside && n_del > 0;
   g->last_beside = beside && timed;
   // fork: the invalidation runs beside the count pass and the merge once the
@@ -351,10 +365,16 @@ cudaError_t enqueue_batch(sp_graph *g, const int *ds, const int *dd, long long n
     rec_side(g, timed, 1);
     cudaEventRecord(g->join_ev, g->side);
   };
-  if (beside && !share) fork();
-  sp::launch_count(g, ni, launches, beside && !share ? sp::inval_beside_blocks(g) : 0);
+  // (a small batch's plan and merge are ordinary grids: nothing waits for them)
+  if (beside && (small || !share)) fork();
+  if (small) {
+    const cudaError_t ep = sp::launch_plan(g, ds, dd, n_del, as, ad, aw, n_add, launches);
+    if (e == cudaSuccess) e = ep;
+  } else {
+    sp::launch_count(g, ni, launches, beside && !share ? sp::inval_beside_blocks(g) : 0);
+  }
   rec(g, timed, 2);
-  if (beside && share) fork();
+  if (beside && share && !small) fork();
   sp::launch_merge(g, ni, launches);
   rec(g, timed, 3);
   if (beside) cudaStreamWaitEvent(g->stream, g->join_ev, 0);   // join
@@ -1189,11 +1209,8 @@ sp_status pr_phase(sp_graph *g, const int *ds, const int *dd, long long nd, cons
     sp::launch_ctl_reset(g, 0, launches);
     cudaError_t e = cudaSuccess;
     if (n_flag > 0) e = sp::launch_flag(g, flag_dst, n_flag, launches);
-    const cudaError_t eq = sp::launch_search(g, ds, dd, nd, as, ad, aw, na, launches, g->stream);
-    if (e == cudaSuccess) e = eq;
-    const cudaError_t es = sp::launch_batch_sort(g, ds, dd, nd, as, ad, aw, na, launches);
+    const cudaError_t es = sp::launch_store_plan(g, ds, dd, nd, as, ad, aw, na, launches);
     if (e == cudaSuccess) e = es;
-    sp::launch_count(g, ni, launches);
     sp::launch_merge(g, ni, launches);
     sp::launch_finish(g, launches);
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -1443,12 +1460,9 @@ sp_status sp_tc_apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
   int launches = 0, regrows = 0;
   for (int attempt = 0;; ++attempt) {
     sp::launch_ctl_reset(g, 0, &launches);
-    const cudaError_t eq =
-        sp::launch_search(g, ds, dd, n_del, as, ad, aw, n_add, &launches, g->stream);
-    cudaError_t es = sp::launch_batch_sort(g, ds, dd, n_del, as, ad, aw, n_add, &launches);
-    if (es == cudaSuccess) es = eq;
+    const cudaError_t es =
+        sp::launch_store_plan(g, ds, dd, n_del, as, ad, aw, n_add, &launches);
     rec(g, true, 1);
-    sp::launch_count(g, ni, &launches);
     sp::launch_tc_batch_sym(g, nb, &launches);     // before anything changes
     sp::launch_tc_tasks(g, nb, &launches);
     rec(g, true, 2);

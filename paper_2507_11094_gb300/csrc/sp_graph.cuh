@@ -200,7 +200,7 @@ struct sp_graph {
   cudaGraph_t bg_graph = nullptr;
   cudaGraphExec_t bg_exec = nullptr;
   cudaGraphNode_t bg_sort = nullptr, bg_inval = nullptr,   // nodes that read the inputs
-                  bg_search = nullptr;
+                  bg_search = nullptr, bg_plan = nullptr, bg_check = nullptr;
   bool bg_ready = false;
   int capturing = -1;                    // >= 0 while the pipeline is captured
   unsigned long long bg_gen = 0;
@@ -279,6 +279,23 @@ cudaError_t retarget_batch_sort(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t
 const void *inval_fn();
 cudaError_t retarget_inval(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t node, const int *ds,
                            const int *dd, long long nd, int concurrent);
+// A small batch: its control reset and validation, and its searches, sort and
+// count, in one block each.
+bool plan_small(const sp_graph *g, long long ni);
+void launch_check_small(sp_graph *g, const int *ds, const int *dd, long long nd, const int *as,
+                        const int *ad, const int *aw, long long na, int reset, int *launches);
+cudaError_t launch_plan(sp_graph *g, const int *ds, const int *dd, long long nd, const int *as,
+                        const int *ad, const int *aw, long long na, int *launches);
+const void *plan_fn();
+const void *check_small_fn();
+cudaError_t retarget_plan(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t check,
+                          cudaGraphNode_t plan, const int *ds, const int *dd, long long nd,
+                          const int *as, const int *ad, const int *aw, long long na);
+// Everything before a batch's merge on the graph's stream, by either way
+// (after a control reset).
+cudaError_t launch_store_plan(sp_graph *g, const int *ds, const int *dd, long long nd,
+                              const int *as, const int *ad, const int *aw, long long na,
+                              int *launches);
 void launch_check_batch(sp_graph *g, const int *ds, const int *dd, long long nd, const int *as,
                         const int *ad, const int *aw, long long na, int *launches);
 

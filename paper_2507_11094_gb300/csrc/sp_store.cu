@@ -285,7 +285,7 @@ __global__ void k_copy_slots(const int2 *__restrict__ src, int2 *dst, long long 
 // full: 0 a new call, 1 a new graph, 2 a call rerun after a pool grow,
 // which keeps what the first attempt's invalidation found (it ran beside
 // the store update, changed the distances, and does not run again)
-__global__ void k_ctl_reset(Ctl *c, int full) {
+__device__ __forceinline__ void ctl_reset(Ctl *c, int full) {
   const bool keep = full == 2;
   c->status = 0;
   c->need_grow = 0;
@@ -349,6 +349,8 @@ __global__ void k_ctl_reset(Ctl *c, int full) {
     c->pool_need[0] = c->pool_need[1] = 0;
   }
 }
+
+__global__ void k_ctl_reset(Ctl *c, int full) { ctl_reset(c, full); }
 
 // Validation only (ids and weights), for callers that apply a batch in
 // several steps and must reject it before the first one.
@@ -440,6 +442,42 @@ __device__ __forceinline__ u64 block_excl_scan_u64(u64 x, u64 *ws, u64 *total) {
   *total = ws[nwarps - 1];
   __syncthreads();
   return r;
+}
+
+// Is a touched row merged in a group of small rows, and in how many strips
+// otherwise?
+__device__ __forceinline__ bool row_is_small(int old_deg, u32 items) {
+  return old_deg <= kSmallRow && items <= (u32)kSmallItems;
+}
+__device__ __forceinline__ u32 row_strips(int old_deg) {
+  return old_deg > kStrip ? (u32)((old_deg + kStrip - 1) / kStrip) : 1u;
+}
+
+// A touched row's new size and place: its alternate region, or a fresh pair of
+// regions in the spare pool when it outgrows its capacity.
+__device__ __forceinline__ void size_row(Ctl *c, const Store &st, const RowMeta &rm, int row,
+                                         int dir, int new_deg, float slack, Seg &sg,
+                                         u64 &relocated) {
+  sg.old_start = rm.start;
+  sg.old_deg = rm.deg;
+  sg.new_deg = new_deg;
+  sg.pad = 0;
+  if (new_deg > rm.cap) {
+    long long nc = row_capacity(new_deg, slack);
+    const long long dbl = round_up4(2LL * rm.cap);
+    if (dbl > nc) nc = dbl;
+    const u64 off = atomicAdd(&c->pool_need[dir], (u64)(2 * nc));
+    if ((long long)(off + 2 * nc) > st.slots - st.main_slots)
+      atomicOr(&c->need_grow, dir ? kGrowPoolRev : kGrowPoolFwd);
+    sg.dest = st.main_slots + (long long)off;
+    sg.new_alt = st.main_slots + (long long)off + nc;
+    sg.new_cap = (int)nc;
+    ++relocated;
+  } else {
+    sg.dest = st.alt[row];
+    sg.new_alt = rm.start;
+    sg.new_cap = rm.cap;
+  }
 }
 
 // The count pass in one cooperative launch; block b owns items
@@ -615,32 +653,11 @@ __global__ void __launch_bounds__(kCT, 3) k_count(CountArgs a) {
       const u64 p = pe[j] - pf[j];
       const int new_deg = rm[j].deg - (int)(u32)p + (int)(u32)(p >> 32);
       Seg &sg = a.seg[base + (u32)j * kCT + t];
-      sg.old_start = rm[j].start;
-      sg.old_deg = rm[j].deg;
-      sg.new_deg = new_deg;
-      sg.pad = 0;
+      size_row(c, st, rm[j], row[j], dir[j], new_deg, a.slack, sg, relocated);
       sg.prefix = key[j] & ~((2ull << a.bits) - 1);
       sg.base_pref = pf[j];
-      if (new_deg > rm[j].cap) {
-        long long nc = row_capacity(new_deg, a.slack);
-        const long long dbl = round_up4(2LL * rm[j].cap);
-        if (dbl > nc) nc = dbl;
-        const u64 off = atomicAdd(&c->pool_need[dir[j]], (u64)(2 * nc));
-        if ((long long)(off + 2 * nc) > st.slots - st.main_slots)
-          atomicOr(&c->need_grow, dir[j] ? kGrowPoolRev : kGrowPoolFwd);
-        sg.dest = st.main_slots + (long long)off;
-        sg.new_alt = st.main_slots + (long long)off + nc;
-        sg.new_cap = (int)nc;
-        ++relocated;
-      } else {
-        sg.dest = st.alt[row[j]];
-        sg.new_alt = rm[j].start;
-        sg.new_cap = rm[j].cap;
-      }
-      if (rm[j].deg <= kSmallRow && e[j] - f[j] <= (u32)kSmallItems)
-        nsmall[j] = 1;
-      else
-        nstr[j] = rm[j].deg > kStrip ? (u32)((rm[j].deg + kStrip - 1) / kStrip) : 1u;
+      if (row_is_small(rm[j].deg, e[j] - f[j])) nsmall[j] = 1;
+      else nstr[j] = row_strips(rm[j].deg);
       want += (u64)nstr[j] | ((u64)nsmall[j] << 32);
       ++touched;
       slots += (u64)rm[j].deg + (u64)new_deg;
@@ -803,6 +820,342 @@ bool search_guesses(const sp_graph *g) {
 // never delays the sort's cooperative grid.
 unsigned search_grid(const sp_graph *g, long long ni) {
   return blocks_for(ni, kCTile, std::max(1, g->num_sms));
+}
+
+// --------------------------------------------------------------------------
+// small batches: everything before the merge in one block
+// --------------------------------------------------------------------------
+//
+// A batch of at most kPlanItems items (1,024 updates) is all latency: the sort
+// and the count spend their time at barriers between passes over a few
+// hundred items.  One block does the work of k_search, k_batch_sort and
+// k_count with the items in shared memory, and writes what they write: a
+// bitonic sort of (key, item number) takes the place of the radix passes, block
+// scans that of the grid barriers.  Before it one more block resets the control
+// block and checks the batch, so that the invalidation runs beside all of it.
+// A call with 64 updates on 1,024 vertices: 136 -> 112 us; with 1,001 on
+// 100,003: 195 -> 172 us.  Above kPlanItems one block's searches and sort take
+// longer than the grid's.
+constexpr int kPlanT = 1024;             // threads at most: as many as the items need,
+constexpr int kPlanItems = 2 * kPlanT;   // two items each (a power of two of threads)
+
+struct PlanArgs {
+  SearchArgs in;
+  Ctl *ctl;
+  u64 *keys;
+  u32 *wts;
+  Seg *seg;
+  unsigned char *flags;
+  u64 *item_pref;
+  u32 *opos;
+  int2 *strips;
+  long long strips_cap;
+  int bits;
+  float slack;
+};
+
+constexpr size_t kPlanSmem = (size_t)kPlanItems * (2 * sizeof(u64) + sizeof(u32));
+static_assert(kPlanSmem <= 47 * 1024, "within what every launch may have");
+
+__global__ void __launch_bounds__(kPlanT, 1) k_plan(PlanArgs a) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  u64 *s_key = (u64 *)smraw;                  // sorted keys
+  u64 *s_srch = s_key + kPlanItems;           // search results by item number, then prefixes
+  u32 *s_idx = (u32 *)(s_srch + kPlanItems);  // item numbers in sorted order, then row heads
+  __shared__ u64 ws64[kPlanT / 32];
+  __shared__ u64 s_sum[3];
+  Ctl *c = a.ctl;
+  const int t = threadIdx.x, T = (int)blockDim.x;
+  const u32 P = 2u * (u32)T;   // slots, the last ones empty
+  const u32 ni = a.in.n_items;
+  const long long nb = a.in.nd + a.in.na;
+  const int bits = a.bits;
+  if (t < 3) s_sum[t] = 0;
+  bool bad = false;
+  // the items, as k_batch_sort numbers and checks them, and their searches in
+  // the old rows, as k_search makes them (both of a thread's in lockstep)
+  {
+    int u[2], v[2], w[2], col[2], deg[2];
+    bool val[2], rev[2];
+    const int2 *old[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const u32 i = (u32)(k * T + t);
+      val[k] = i < ni;
+      rev[k] = (long long)i >= nb;
+      const long long j = rev[k] ? (long long)i - nb : (long long)i;
+      u[k] = v[k] = w[k] = 0;
+      if (val[k]) {
+        if (j < a.in.nd) {
+          u[k] = __ldg(a.in.ds + j);
+          v[k] = __ldg(a.in.dd + j);
+        } else {
+          u[k] = __ldg(a.in.as + (j - a.in.nd));
+          v[k] = __ldg(a.in.ad + (j - a.in.nd));
+          w[k] = __ldg(a.in.aw + (j - a.in.nd));
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const u32 i = (u32)(k * T + t);
+      const long long j = rev[k] ? (long long)i - nb : (long long)i;
+      const u64 kind = j < a.in.nd ? 0 : 1;
+      const bool ok = u[k] >= 0 && u[k] < a.in.n && v[k] >= 0 && v[k] < a.in.n &&
+                      (kind == 0 || (w[k] >= 1 && w[k] <= SP_WMAX));
+      if (val[k] && !ok) {
+        bad = true;
+        u[k] = v[k] = 0;
+      }
+      s_key[i] = !val[k] ? ~0ull
+                 : rev[k] ? (1ull << (2 * bits + 1)) | ((u64)v[k] << (bits + 1)) |
+                                ((u64)u[k] << 1) | kind
+                          : ((u64)u[k] << (bits + 1)) | ((u64)v[k] << 1) | kind;
+      s_idx[i] = i;
+      RowMeta rm;
+      rm.start = 0;
+      rm.deg = 0;
+      const Store &st = a.in.st[rev[k] ? 1 : 0];
+      if (val[k] && ok) rm = st.row[rev[k] ? v[k] : u[k]];
+      col[k] = rev[k] ? u[k] : v[k];
+      old[k] = st.adj + rm.start;
+      deg[k] = rm.deg;
+    }
+    u32 at[2];
+    bool present[2];
+    row_search<2>(old, deg, col, a.in.n, at, present);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+      if (val[k])
+        s_srch[k * T + t] =
+            ((u64)(u32)w[k] << 32) | (present[k] ? 0x80000000ull : 0ull) | at[k];
+  }
+  if (__syncthreads_or(bad)) {   // nothing changes: every later kernel of the call sees the status
+    if (t == 0) set_status(c, SP_EINVAL);
+    return;
+  }
+  // bitonic sort by (key, item number): the order of a stable sort by key.  A
+  // thread holds two consecutive slots, so that distances below 64 stay in its
+  // warp's registers (in shared memory they took 25 of 45 us for 2,002 items)
+  u64 rk[2] = {s_key[2 * t], s_key[2 * t + 1]};
+  u32 ri[2] = {s_idx[2 * t], s_idx[2 * t + 1]};
+  for (u32 k = 2; k <= P; k <<= 1) {
+    u32 j = k >> 1;
+    if (j >= 64) {
+      s_key[2 * t] = rk[0];
+      s_key[2 * t + 1] = rk[1];
+      s_idx[2 * t] = ri[0];
+      s_idx[2 * t + 1] = ri[1];
+      for (; j >= 64; j >>= 1) {
+        __syncthreads();
+        const u32 x = 2 * ((u32)t & ~(j - 1)) + ((u32)t & (j - 1)), y = x + j;
+        const u64 kx = s_key[x], ky = s_key[y];
+        const u32 ix = s_idx[x], iy = s_idx[y];
+        const bool gt = kx > ky || (kx == ky && ix > iy);
+        if (gt == ((x & k) == 0)) {
+          s_key[x] = ky;
+          s_key[y] = kx;
+          s_idx[x] = iy;
+          s_idx[y] = ix;
+        }
+      }
+      __syncthreads();
+      rk[0] = s_key[2 * t];
+      rk[1] = s_key[2 * t + 1];
+      ri[0] = s_idx[2 * t];
+      ri[1] = s_idx[2 * t + 1];
+      __syncwarp();
+    }
+    const bool up = ((2u * (u32)t) & k) == 0;
+    for (; j >= 2; j >>= 1) {
+      const bool low = ((2u * (u32)t) & j) == 0;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const u64 ok = __shfl_xor_sync(kFull, rk[q], j >> 1);
+        const u32 oi = __shfl_xor_sync(kFull, ri[q], j >> 1);
+        const bool gt = rk[q] > ok || (rk[q] == ok && ri[q] > oi);
+        if (gt == (low == up)) {
+          rk[q] = ok;
+          ri[q] = oi;
+        }
+      }
+    }
+    const bool gt = rk[0] > rk[1] || (rk[0] == rk[1] && ri[0] > ri[1]);
+    if (gt == up) {
+      const u64 kk = rk[0];
+      const u32 ii = ri[0];
+      rk[0] = rk[1];
+      ri[0] = ri[1];
+      rk[1] = kk;
+      ri[1] = ii;
+    }
+  }
+  s_key[2 * t] = rk[0];
+  s_key[2 * t + 1] = rk[1];
+  s_idx[2 * t] = ri[0];
+  s_idx[2 * t + 1] = ri[1];
+  __syncthreads();
+  // which updates apply (k_count's first step), two consecutive items a thread
+  u64 iv[2] = {0, 0};
+  bool head[2] = {false, false};
+  u64 del_ok = 0, del_abs = 0, add_ok = 0, add_pres = 0;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const u32 i = 2 * (u32)t + q;
+    if (i >= ni) continue;
+    const u64 key = s_key[i], pk = i > 0 ? s_key[i - 1] : ~0ull, sr = s_srch[s_idx[i]];
+    const u64 nk = i + 1 < ni ? s_key[i + 1] : ~0ull;
+    const bool present = (sr >> 31) & 1;
+    const int dir = (int)(key >> (2 * bits + 1));
+    head[q] = i == 0 || (key >> (bits + 1)) != (pk >> (bits + 1));
+    bool applied;
+    if ((key & 1) == 0) {
+      applied = present && pk != key;
+      iv[q] = applied ? 1ull : 0ull;
+      if (dir == 0) { applied ? ++del_ok : ++del_abs; }
+    } else {
+      u32 first = i, last = i;
+      bool best = true;
+      if (pk == key || nk == key) {   // the run of insertions of this edge
+        while (first > 0 && s_key[first - 1] == key) --first;
+        while (last + 1 < ni && s_key[last + 1] == key) ++last;
+        u32 bi = first, bw = (u32)(s_srch[s_idx[first]] >> 32);
+        for (u32 r = first + 1; r <= last; ++r) {
+          const u32 w2 = (u32)(s_srch[s_idx[r]] >> 32);
+          if (w2 < bw) { bw = w2; bi = r; }
+        }
+        best = bi == i;
+      }
+      const bool del_exists = first > 0 && s_key[first - 1] == (key ^ 1ull);
+      const bool run_applies = !present || del_exists;
+      applied = best && run_applies;
+      iv[q] = applied ? (1ull << 32) : 0ull;
+      if (dir == 0 && i == first) {
+        add_ok += run_applies;
+        add_pres += (u64)(last - first + 1) - (run_applies ? 1 : 0);
+      }
+    }
+    a.keys[i] = key;
+    a.opos[i] = (u32)sr & 0x7FFFFFFFu;
+    a.wts[i] = (u32)(sr >> 32);
+    a.flags[i] = (applied ? 1 : 0) | (present ? 2 : 0);
+  }
+  // prefixes of the applied, and the heads of the touched rows
+  u64 total, nheads;
+  const u64 pre = block_excl_scan_u64(iv[0] + iv[1], ws64, &total);
+  const u32 h0 = (u32)block_excl_scan_u64((u64)head[0] + (u64)head[1], ws64, &nheads);
+  // (the scans' barriers: every use of the search results and item numbers is over)
+  const u32 nseg = (u32)nheads;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const u32 i = 2 * (u32)t + q;
+    if (i >= ni) continue;
+    const u64 x = pre + (q ? iv[0] : 0ull);
+    s_srch[i] = x;
+    a.item_pref[i] = x;
+    if (head[q]) s_idx[h0 + (q ? (u32)head[0] : 0u)] = i;
+  }
+  if (t == 0) a.item_pref[ni] = total;
+  __syncthreads();
+  // the touched rows (k_count's third step)
+  u64 touched = 0, relocated = 0, slots = 0, want[2] = {0, 0};
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const u32 si = (u32)(q * T + t);
+    if (si >= nseg) continue;
+    const u32 f = s_idx[si], e = si + 1 < nseg ? s_idx[si + 1] : ni;
+    const u64 pfx = s_key[f] >> (bits + 1);
+    const int row = (int)(pfx & ((1ull << bits) - 1)), dir = (int)(pfx >> bits);
+    const Store &st = a.in.st[dir];
+    const RowMeta rm = st.row[row];
+    const u64 pf = s_srch[f], p = (e < ni ? s_srch[e] : total) - pf;
+    Seg sg;
+    sg.first = f;
+    sg.end = e;
+    sg.row = row;
+    sg.dir = dir;
+    size_row(c, st, rm, row, dir, rm.deg - (int)(u32)p + (int)(u32)(p >> 32), a.slack, sg,
+             relocated);
+    sg.prefix = pfx << (bits + 1);
+    sg.base_pref = pf;
+    a.seg[si] = sg;
+    if (row_is_small(rm.deg, e - f)) want[q] = 1ull << 32;
+    else want[q] = (u64)row_strips(rm.deg);
+    ++touched;
+    slots += (u64)rm.deg + (u64)sg.new_deg;
+  }
+  u64 all;
+  u64 at = block_excl_scan_u64(want[0] + want[1], ws64, &all);
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int si = q * T + t;
+    for (u32 k = 0; k < (u32)want[q]; ++k)
+      a.strips[(u32)at + k] = make_int2(si, (int)(k * kStrip));
+    if (want[q] >> 32) a.strips[a.strips_cap - 1 - (long long)(at >> 32)] = make_int2(si, 0);
+    at += want[q];
+  }
+  if (t == 0) {
+    c->n_seg = nseg;
+    c->bstrips = (u32)all;
+    c->sstrips = (u32)(all >> 32);
+  }
+  // the counters (at most kPlanItems each: 16 bits of a word)
+  u64 sum[3] = {del_ok | (del_abs << 16) | (add_ok << 32) | (add_pres << 48),
+                touched | (relocated << 16), slots};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum[k] += __shfl_xor_sync(kFull, sum[k], o);
+    if ((t & 31) == 0 && sum[k]) atomicAdd(&s_sum[k], sum[k]);
+  }
+  __syncthreads();
+  if (t == 0) {
+    c->del_applied = s_sum[0] & 0xFFFF;
+    c->del_absent = (s_sum[0] >> 16) & 0xFFFF;
+    c->add_applied = (s_sum[0] >> 32) & 0xFFFF;
+    c->add_present = s_sum[0] >> 48;
+    c->rows_touched = s_sum[1] & 0xFFFF;
+    c->rows_relocated = s_sum[1] >> 16;
+    c->merge_slots = s_sum[2];
+  }
+}
+
+// A small batch's control reset and validation (k_check_batch in one block),
+// after which the invalidation may run beside the plan.
+__global__ void __launch_bounds__(kPlanT) k_check_small(SearchArgs in, Ctl *c, int reset) {
+  const int t = threadIdx.x;
+  if (t == (int)blockDim.x - 1) {
+    ctl_reset(c, reset);
+    __threadfence();
+  }
+  bool bad = false;
+  for (long long i = t; i < in.nd + in.na; i += blockDim.x) {
+    const bool del = i < in.nd;
+    const long long j = del ? i : i - in.nd;
+    const int u = del ? in.ds[j] : in.as[j], v = del ? in.dd[j] : in.ad[j];
+    const int w = del ? 1 : in.aw[j];
+    bad |= u < 0 || u >= in.n || v < 0 || v >= in.n || w < 1 || w > SP_WMAX;
+  }
+  if (__syncthreads_or(bad) && t == 0) set_status(c, SP_EINVAL);
+}
+
+PlanArgs plan_args(sp_graph *g, const int *ds, const int *dd, long long nd, const int *as,
+                   const int *ad, const int *aw, long long na) {
+  BatchBufs &b = g->bb;
+  PlanArgs a;
+  a.in = search_args(g, ds, dd, nd, as, ad, aw, na);
+  a.ctl = g->ctl;
+  a.keys = b.keys;
+  a.wts = b.vals_alt;
+  a.seg = b.seg;
+  a.flags = b.flags;
+  a.item_pref = b.item_pref;
+  a.opos = b.opos;
+  a.strips = b.strips;
+  a.strips_cap = b.strips_cap;
+  a.bits = g->bits;
+  a.slack = g->slack;
+  return a;
 }
 
 // --------------------------------------------------------------------------
@@ -1433,14 +1786,15 @@ void launch_merge(sp_graph *g, long long ni, int *launches) {
   a.bits = g->bits;
   a.n_items = (u32)ni;
   // exactly the resident blocks: every warp starts at once and the strips
-  // spread evenly over them
+  // spread evenly over them (a small batch: a block per item at most)
   static int per_sm = 0;
   if (per_sm == 0 &&
       (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_merge, kThreads, 0) !=
            cudaSuccess ||
        per_sm < 1))
     per_sm = 4;
-  k_merge<<<(unsigned)std::max(1, g->num_sms * per_sm), kThreads, 0, g->stream>>>(a);
+  const long long full = std::max(1, g->num_sms * per_sm);
+  k_merge<<<(unsigned)std::min(full, ni), kThreads, 0, g->stream>>>(a);
   *launches += 1;
 }
 
@@ -1532,6 +1886,68 @@ cudaError_t retarget_search(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t nod
   p.sharedMemBytes = 0;
   p.kernelParams = args;
   return cudaGraphExecKernelNodeSetParams(ex, node, &p);
+}
+
+static unsigned plan_threads(long long ni) {
+  unsigned t = 32;
+  while (2 * (long long)t < ni) t <<= 1;
+  return t;
+}
+
+// (the barrier test hooks of the sort and the count need those kernels)
+bool plan_small(const sp_graph *g, long long ni) {
+  return ni <= kPlanItems && g->lim.miss_site != 4u && g->lim.miss_site != 5u;
+}
+
+cudaError_t launch_plan(sp_graph *g, const int *ds, const int *dd, long long nd, const int *as,
+                        const int *ad, const int *aw, long long na, int *launches) {
+  k_plan<<<1, plan_threads(2 * (nd + na)), kPlanSmem, g->stream>>>(
+      plan_args(g, ds, dd, nd, as, ad, aw, na));
+  ++*launches;
+  return cudaGetLastError();
+}
+
+void launch_check_small(sp_graph *g, const int *ds, const int *dd, long long nd, const int *as,
+                        const int *ad, const int *aw, long long na, int reset, int *launches) {
+  k_check_small<<<1, plan_threads(2 * (nd + na)), 0, g->stream>>>(
+      search_args(g, ds, dd, nd, as, ad, aw, na), g->ctl, reset);
+  ++*launches;
+}
+
+const void *plan_fn() { return (const void *)k_plan; }
+const void *check_small_fn() { return (const void *)k_check_small; }
+
+cudaError_t retarget_plan(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t check,
+                          cudaGraphNode_t plan, const int *ds, const int *dd, long long nd,
+                          const int *as, const int *ad, const int *aw, long long na) {
+  PlanArgs a = plan_args(g, ds, dd, nd, as, ad, aw, na);
+  int reset = 0;
+  void *cargs[3] = {&a.in, &a.ctl, &reset};
+  void *args[1] = {&a};
+  cudaKernelNodeParams p = {};
+  p.func = (void *)k_check_small;
+  p.gridDim = dim3(1);
+  p.blockDim = dim3(plan_threads(2 * (nd + na)));
+  p.sharedMemBytes = 0;
+  p.kernelParams = cargs;
+  const cudaError_t e = cudaGraphExecKernelNodeSetParams(ex, check, &p);
+  if (e != cudaSuccess) return e;
+  p.func = (void *)k_plan;
+  p.sharedMemBytes = (unsigned)kPlanSmem;
+  p.kernelParams = args;
+  return cudaGraphExecKernelNodeSetParams(ex, plan, &p);
+}
+
+cudaError_t launch_store_plan(sp_graph *g, const int *ds, const int *dd, long long nd,
+                              const int *as, const int *ad, const int *aw, long long na,
+                              int *launches) {
+  const long long ni = 2 * (nd + na);
+  if (ni == 0) return cudaSuccess;
+  if (plan_small(g, ni)) return launch_plan(g, ds, dd, nd, as, ad, aw, na, launches);
+  const cudaError_t e = launch_search(g, ds, dd, nd, as, ad, aw, na, launches, g->stream);
+  const cudaError_t es = launch_batch_sort(g, ds, dd, nd, as, ad, aw, na, launches);
+  launch_count(g, ni, launches);
+  return e != cudaSuccess ? e : es;
 }
 
 void launch_finish(sp_graph *g, int *launches) {

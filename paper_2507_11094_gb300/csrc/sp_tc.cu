@@ -535,6 +535,8 @@ __global__ void __launch_bounds__(kThreads) k_tc_delta(DeltaArgs a, int kind) {
         lo[k] = 0;
         hi[k] = e < wdeg ? sdeg : 0;
       }
+      // (halving: the rows of a batch's pairs are in L2, where the extra
+      // arithmetic of an interpolating search costs more than its reads save)
       for (;;) {
         int y[kDK], mid[kDK];
         bool act = false;

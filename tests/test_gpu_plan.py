@@ -1,0 +1,97 @@
+"""GPU tests of small batches, whose store update one block plans, around the
+largest one (1,024 updates, above which the grid's sort and count take over)
+and at odd and tiny sizes: counters, both stores and distances against the
+oracle, with repeated updates, no-ops and delete-then-insert among them."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2507_11094_gb300 import sp
+from paper_2507_11094_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    from paper_2507_11094_gb300 import build
+    build.build()
+    oracle.build()
+    sp.load()
+
+
+def messy(rng, n, keys, k):
+    """k updates: deletions of present and absent edges and insertions of new
+    and present ones, a third of them repeated (insertions with other weights)
+    or naming an edge that the batch deletes too."""
+    nd = int(rng.integers(0, k + 1)) if k > 1 else int(rng.integers(0, 2))
+    na = k - nd
+
+    def some(count):
+        pick = rng.choice(keys, size=count)
+        rnd = rng.integers(0, n * n, size=count)
+        return np.where(rng.random(count) < 0.6, pick, rnd)
+    d, a = some(nd), some(na)
+    for x in (d, a):
+        if x.size > 2:
+            again = rng.random(x.size) < 0.3
+            x[again] = rng.choice(x, size=int(again.sum()))
+    if nd and na:
+        both = rng.random(na) < 0.2
+        a[both] = rng.choice(d, size=int(both.sum()))
+    w = rng.integers(1, 101, size=na)
+    i32 = lambda x: np.ascontiguousarray(x, np.int32)
+    return wl.Batch(i32(d // n), i32(d % n), i32(a // n), i32(a % n), i32(w))
+
+
+@pytest.mark.parametrize("n,m", [(40, 300), (5000, 40000)])
+@pytest.mark.parametrize("sizes", [(1, 1, 1, 2, 3), (31, 32, 33, 64, 65), (511, 512, 513, 700, 700),
+                                   (1022, 1023, 1024, 1025, 1026), (1024, 1024, 1024, 1100, 1)])
+@pytest.mark.parametrize("own_stream", [False, True])
+def test_small_batches(n, m, sizes, own_stream):
+    import torch
+    ro, col, w = wl.er_digraph(n, m, 1, 100, seed=n)
+    ref = oracle.OracleGraph(n, ro, col, w)
+    rng = np.random.default_rng(n + sizes[0])
+    st = torch.cuda.Stream() if own_stream else None
+    with sp.Graph(n, ro, col, w, slack=0.05, stream=st) as g:
+        g.sssp_init(0)
+        for k in sizes:
+            ro, col, _ = ref.csr()
+            b = messy(rng, n, wl.csr_keys(n, ro, col), k)
+            want = ref.apply(b)
+            got = g.apply(b, stats=True)
+            assert (got.n_del_applied, got.n_del_absent, got.n_add_applied,
+                    got.n_add_present) == want
+            np.testing.assert_array_equal(g.get_dist(), ref.dijkstra(0))
+            for x, y in zip(g.export_csr(), ref.csr()):
+                np.testing.assert_array_equal(x, y)
+        ro, col, w = ref.csr()
+        u = np.repeat(np.arange(n), np.diff(ro))
+        order = np.lexsort((u, col))
+        rro, rcol, rw = g.export_csr(reverse=True)
+        np.testing.assert_array_equal(np.diff(rro), np.bincount(col, minlength=n))
+        np.testing.assert_array_equal(rcol, u[order])
+        np.testing.assert_array_equal(rw, w[order])
+
+
+@pytest.mark.parametrize("k", [1, 7, 1024])
+def test_an_invalid_update_changes_nothing(k):
+    n = 300
+    ro, col, w = wl.er_digraph(n, 2000, 1, 100, seed=3)
+    with sp.Graph(n, ro, col, w) as g:
+        g.sssp_init(0)
+        before = g.get_dist()
+        z = np.zeros(0, np.int32)
+        for bad in ((k - 1, n, 1), (0, -1, 1), (k // 2, 5, 0), (k // 2, 5, sp.SP_WMAX + 1)):
+            d = np.full(k, 7, np.int32)
+            ww = np.ones(k, np.int32)
+            d[bad[0]], ww[bad[0]] = bad[1], bad[2]
+            with pytest.raises(sp.SpError) as e:
+                g.apply_batch(z, z, np.arange(k, dtype=np.int32) % n, d, ww)
+            assert e.value.code == sp.SP_EINVAL
+        np.testing.assert_array_equal(g.get_dist(), before)
+        for x, y in zip(g.export_csr(), (ro, col, w)):
+            np.testing.assert_array_equal(x, y)
