@@ -257,8 +257,8 @@ cudaError_t retarget_input_nodes(sp_graph *g, const int *ds, const int *dd, long
   return e;
 }
 
-// The control block of the call, on the host.  mirrored: the call ended
-// with k_finish, which wrote it into the pinned copy already.
+// The control block of the call, on the host.  mirrored: the call's last
+// kernel wrote it into the pinned copy already.
 sp_status read_ctl(sp_graph *g, bool mirrored = false) {
   if (!mirrored)
     cudaMemcpyAsync(g->ctl_host, g->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, g->stream);
@@ -384,11 +384,15 @@ cudaError_t enqueue_batch(sp_graph *g, const int *ds, const int *dd, long long n
   // the pull and OnAdd run as the first stage of the push loop's launch: the
   // push phase spans events 4..7 (fill_stats with `fold`), and events 5 and 6
   // are not recorded (each timing event is one more node of a captured graph)
-  if (e == cudaSuccess) e = sp::launch_push(g, launches, n_del > 0 ? 1 : 0, ni);
+  // (and ends the call, unless the degree count follows it)
+  const bool pool = g->lim.pool_rounds > 0;
+  if (e == cudaSuccess) e = sp::launch_push(g, launches, n_del > 0 ? 1 : 0, ni, !pool);
   rec(g, timed, 7);
   // the degree share that picks the pool kernel of the next call
-  if (g->lim.pool_rounds > 0) sp::launch_deg_mid(g, launches);
-  sp::launch_finish(g, launches);
+  if (pool) {
+    sp::launch_deg_mid(g, launches);
+    sp::launch_finish(g, launches);
+  }
   rec(g, timed, 8);
   if (e == cudaSuccess) e = cudaGetLastError();
   return e;
@@ -410,7 +414,6 @@ sp_status restore_after(sp_graph *g, bool touched, sp_status rc) {
     return rc;
   }
   cudaError_t e = sp::launch_push(g, &launches);
-  sp::launch_finish(g, &launches);
   if (e != cudaSuccess || read_ctl(g, true) != SP_OK ||
       status_of_repair(g, *g->ctl_host) != SP_OK) {
     cudaGetLastError();
@@ -749,7 +752,6 @@ sp_status sp_sssp_init(sp_graph *g, int32_t source, sp_batch_stats *stats) {
   sp::launch_init(g, source, &launches);
   cudaError_t e = sp::launch_push(g, &launches);
   rec(g, timed, SP_NPHASE - 1);
-  sp::launch_finish(g, &launches);
   rec(g, timed, SP_NPHASE);
   if (e != cudaSuccess) {
     g->last_err = (int)e;
@@ -990,7 +992,7 @@ sp_status apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
     }
     // the read-out follows the batch on the stream (a rerun repeats it)
     enqueue_out(g, out, &launches);
-    rc = read_ctl(g, true);   // the batch ends with k_finish, replayed or not
+    rc = read_ctl(g, true);   // the batch's last kernel mirrors it, replayed or not
     if (rc != SP_OK) {
       g->state = 2;
       return rc;
@@ -1068,7 +1070,6 @@ sp_status sp_sssp_init_multi(sp_graph *g, const int32_t *sources, int32_t k,
   sp::launch_init_multi(g, src_d, k, &launches);
   cudaError_t e = sp::launch_push(g, &launches);
   rec(g, timed, SP_NPHASE - 1);
-  sp::launch_finish(g, &launches);
   rec(g, timed, SP_NPHASE);
   sp_status rc = read_ctl(g, true);
   // the list stays with the handle (a failed batch restores from it)

@@ -1412,6 +1412,7 @@ __global__ void __launch_bounds__(is_pool(OP) ? kPoolThreads : kPersistThreads, 
   if (OP == kOpInval && a.concurrent) {
     if (!batch_valid_block(c)) return;
   } else if (!repair_enabled_block(c)) {
+    if (kPushOp && a.finish) finish_call(c, a.finish);
     return;
   }
   if (threadIdx.x == 0) {
@@ -1745,6 +1746,7 @@ __global__ void __launch_bounds__(is_pool(OP) ? kPoolThreads : kPersistThreads, 
     }
     if (capped) raise_timeout(c, 1, 1, round + jumps);
   }
+  if (kPushOp && a.finish) finish_call(c, a.finish);
 }
 
 // --- pull (one pass over A) -----------------------------------------------
@@ -2048,6 +2050,7 @@ LoopArgs make_args(sp_graph *g) {
   a.ptag = g->prtag;
   a.cut = g->cut;
   a.concurrent = 0;
+  a.finish = nullptr;
   a.seed_pull = 0;
   a.keys = g->bb.keys;
   a.vals = g->bb.vals_alt;   // the batch's weights in sorted order (the count pass's)
@@ -2155,8 +2158,9 @@ cudaError_t launch_inval(sp_graph *g, const int *ds, const int *dd, long long nd
   return launch_loop(g, kOpInval, a, launches, concurrent && stream ? stream : g->stream);
 }
 
-cudaError_t launch_push(sp_graph *g, int *launches, int pull, long long n_items) {
+cudaError_t launch_push(sp_graph *g, int *launches, int pull, long long n_items, bool last) {
   LoopArgs a = make_args(g);
+  if (last) a.finish = g->ctl_host;
   a.seed_pull = pull;
   a.n_items = n_items;
   // pool entries carry a row's start / 4 in 32 bits

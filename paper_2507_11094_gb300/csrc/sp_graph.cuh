@@ -132,6 +132,7 @@ struct LoopArgs {
   // beside the store update, so it reads neither store (no frontier rounds)
   u32 *cut;
   int concurrent;
+  Ctl *finish;           // the push loop ends the call: the host's copy (or null)
   // first stage of the push loop of a batch (before its first barrier): the
   // pull over the affected list A, and OnAdd over the sorted batch items
   int seed_pull;
@@ -307,7 +308,10 @@ cudaError_t launch_inval(sp_graph *g, const int *ds, const int *dd, long long nd
                          int *launches, int concurrent = 0, cudaStream_t stream = nullptr);
 // push fixedPoint; for a batch (pull != 0 or n_items > 0) its first stage
 // pulls over A and relaxes the applied insertions
-cudaError_t launch_push(sp_graph *g, int *launches, int pull = 0, long long n_items = 0);
+// and, unless more kernels of the call follow, its last block ends the call
+// as launch_finish does (`last`)
+cudaError_t launch_push(sp_graph *g, int *launches, int pull = 0, long long n_items = 0,
+                        bool last = true);
 // blocks (one per SM) of an invalidation beside the store update
 int inval_beside_blocks(const sp_graph *g);
 void launch_unpack(sp_graph *g, int *dist_d, int *parent_d, int *launches);

@@ -71,6 +71,7 @@ struct Ctl {
   u32 to_site;           // the wait that raised timeout: 1 round cap, 2 loop barrier,
                          // 3 single-block episode, 4 batch-sort barrier
   u32 to_info;           // its round, barrier index or episode
+  alignas(128) u32 done;           // blocks of the call's last kernel that have ended
   // grid barriers of the two persistent loops (monotone arrival counts)
   alignas(128) u64 bar_inval;
   alignas(128) u64 bar_push;

@@ -301,6 +301,7 @@ __device__ __forceinline__ void ctl_reset(Ctl *c, int full) {
   }
   c->cmin = 0xFFFFFFFFu;
   c->bad = 0;
+  c->done = 0;
   c->bar_inval = 0;
   c->bar_push = 0;
   c->bar_sort = 0;
@@ -1178,8 +1179,8 @@ struct MergeArgs {
 };
 
 __device__ __forceinline__ bool merge_enabled(Ctl *c) {
-  return ld_cg_i32(&c->status) == 0 && ld_cg_i32(&c->need_grow) == 0 &&
-         ld_cg_i32(&c->bad) == 0;
+  const int4 f = __ldcg((const int4 *)&c->status);   // status, need_grow (one read for both)
+  return (f.x | f.y | ld_cg_i32(&c->bad)) == 0;
 }
 
 // The merged row holds the kept old entries and the applied insertions in
