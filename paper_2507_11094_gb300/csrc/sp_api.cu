@@ -97,23 +97,16 @@ sp_status ensure_batch_buffers(sp_graph *g, long long ni, long long nb_host) {
     ++g->gen;
   }
   if (nb_host > b.cap_in) {
-    const long long c = std::max(nb_host, b.cap_in * 2);
-    int *p[5];
-    bool ok = true;
-    for (int i = 0; i < 5; ++i) {
-      p[i] = ok ? (int *)al.get((size_t)c * 4) : nullptr;
-      ok = ok && p[i];
-    }
-    if (!ok) {
-      for (int i = 0; i < 5; ++i) al.put(p[i], (size_t)c * 4);
-      return SP_ENOMEM;
-    }
-    const long long old = b.cap_in;
-    al.put(b.in_del_src, old * 4); al.put(b.in_del_dst, old * 4);
-    al.put(b.in_add_src, old * 4); al.put(b.in_add_dst, old * 4); al.put(b.in_add_w, old * 4);
-    b.in_del_src = p[0]; b.in_del_dst = p[1];
-    b.in_add_src = p[2]; b.in_add_dst = p[3];
-    b.in_add_w = p[4];
+    // one allocation for the five arrays, each on a 256-byte boundary
+    const long long c = (std::max(nb_host, b.cap_in * 2) + 63) / 64 * 64;
+    int *p = (int *)al.get((size_t)c * 20);
+    if (!p) return SP_ENOMEM;
+    al.put(b.in_del_src, (size_t)b.cap_in * 20);
+    b.in_del_src = p;
+    b.in_del_dst = p + c;
+    b.in_add_src = p + 2 * c;
+    b.in_add_dst = p + 3 * c;
+    b.in_add_w = p + 4 * c;
     b.cap_in = c;
     ++g->gen;
   }
@@ -496,9 +489,7 @@ sp_status sp_graph_destroy(sp_graph *g) {
   al.put(b.strips, (size_t)b.strips_cap * 8);
   al.put(b.tmp, b.tmp_bytes);
   al.put(b.srch, c * 8);
-  c = b.cap_in;
-  al.put(b.in_del_src, c * 4); al.put(b.in_del_dst, c * 4);
-  al.put(b.in_add_src, c * 4); al.put(b.in_add_dst, c * 4); al.put(b.in_add_w, c * 4);
+  al.put(b.in_del_src, (size_t)b.cap_in * 20);
   al.put(g->fwd.row, n * sizeof(sp::RowMeta));
   al.put(g->fwd.alt, n * sizeof(long long));
   al.put(g->rev.alt, n * sizeof(long long));
@@ -600,12 +591,16 @@ sp_status sp_graph_create(int32_t n, int64_t m, const int64_t *row_off, const in
     sp_graph_destroy(g);
     return SP_ECUDA;
   }
-  if (cudaMallocHost(&g->ctl_host, sizeof(Ctl)) != cudaSuccess) {
+  // the control block's mirror and the block for small host batches and outputs
+  constexpr size_t kCtlBytes = (sizeof(Ctl) + 255) / 256 * 256;
+  if (cudaMallocHost(&g->ctl_host, kCtlBytes + (5 * sp::kSmallUpdates + 2 * sp::kSmallOut) * 4) !=
+      cudaSuccess) {
     cudaGetLastError();
     g->ctl_host = nullptr;
     sp_graph_destroy(g);
     return SP_ENOMEM;
   }
+  g->small_host = (int *)((char *)g->ctl_host + kCtlBytes);
   g->ctl = (Ctl *)g->al.get(sizeof(Ctl));
   const size_t nn = (size_t)n;
   g->s = (u64 *)g->al.get(nn * 8);
@@ -793,6 +788,7 @@ struct DistOut {
   bool want = false;
   int32_t *dist_d = nullptr, *parent_d = nullptr;   // unpack targets
   int32_t *dist_h = nullptr, *parent_h = nullptr;   // pageable host copies (or null)
+  bool from_block = false;   // they are filled from the page-locked block, by the host
 };
 
 sp_status resolve_out(sp_graph *g, int32_t *dist, int32_t *parent, int out_on_device,
@@ -811,16 +807,31 @@ sp_status resolve_out(sp_graph *g, int32_t *dist, int32_t *parent, int out_on_de
     o->parent_d = mp;
     return SP_OK;
   }
-  o->dist_d = g->out_dist;
-  o->parent_d = parent ? g->out_parent : nullptr;
   o->dist_h = dist;
   o->parent_h = parent;
+  if (g->n <= sp::kSmallOut) {   // through the handle's page-locked block
+    o->dist_d = g->small_host + 5 * sp::kSmallUpdates;
+    o->parent_d = parent ? o->dist_d + sp::kSmallOut : nullptr;
+    o->from_block = true;
+    return SP_OK;
+  }
+  o->dist_d = g->out_dist;
+  o->parent_d = parent ? g->out_parent : nullptr;
   return SP_OK;
+}
+
+// After the call's synchronisation: what the unpack kernel left in the
+// handle's page-locked block.
+void take_out(const sp_graph *g, const DistOut &o) {
+  if (!o.from_block) return;
+  std::memcpy(o.dist_h, o.dist_d, (size_t)g->n * 4);
+  if (o.parent_h) std::memcpy(o.parent_h, o.parent_d, (size_t)g->n * 4);
 }
 
 void enqueue_out(sp_graph *g, const DistOut &o, int *launches) {
   if (!o.want) return;
   sp::launch_unpack(g, o.dist_d, o.parent_d, launches);
+  if (o.from_block) return;
   if (o.dist_h)
     cudaMemcpyAsync(o.dist_h, o.dist_d, (size_t)g->n * 4, cudaMemcpyDeviceToHost, g->stream);
   if (o.parent_h)
@@ -875,6 +886,10 @@ sp_status apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
   if (g->state != 1) return SP_ESTATE;
   const long long nb = n_del + n_add, ni = 2 * nb;
   const bool timed = stats != nullptr;
+  // a small batch in host memory is read in place by the few kernels that need
+  // it (pageable arrays from the handle's page-locked block, into which they
+  // are copied here), with no staging kernel or copy in front
+  const bool in_place = !inputs_on_device && nb > 0 && sp::plan_small(g, ni);
   // the same batch shape twice in a row: the pipeline runs as a cached CUDA
   // graph (one launch instead of seven), its input-reading nodes pointed at
   // this call's arrays
@@ -903,12 +918,23 @@ sp_status apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
       mapped = m[2] && m[3] && m[4];
     }
   }
-  sp_status rc = ensure_batch_buffers(g, ni, inputs_on_device ? 0 : std::max(n_del, n_add));
+  sp_status rc =
+      ensure_batch_buffers(g, ni, inputs_on_device || in_place ? 0 : std::max(n_del, n_add));
   if (rc != SP_OK) return rc;
   auto &b = g->bb;
   rec(g, timed, 0);
   int staged = 0;
-  if (mapped) {
+  if (in_place) {
+    const int32_t *src[5] = {del_src, del_dst, add_src, add_dst, add_w};
+    const int *in[5];
+    for (int q = 0; q < 5; ++q) {
+      const long long k = q < 2 ? n_del : n_add;
+      int *h = g->small_host + q * sp::kSmallUpdates;
+      if (!mapped && k) std::memcpy(h, src[q], (size_t)k * 4);
+      in[q] = mapped ? (const int *)m[q] : h;
+    }
+    ds = in[0]; dd = in[1]; as = in[2]; ad = in[3]; aw = in[4];
+  } else if (mapped) {
     const int *src[5] = {(const int *)m[0], (const int *)m[1], (const int *)m[2],
                          (const int *)m[3], (const int *)m[4]};
     int *const dst[5] = {b.in_del_src, b.in_del_dst, b.in_add_src, b.in_add_dst, b.in_add_w};
@@ -1026,6 +1052,7 @@ sp_status apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
 
   }
   const Ctl &c = *g->ctl_host;
+  take_out(g, out);
   g->m += (long long)c.add_applied - (long long)c.del_applied;
   if (c.add_applied + c.del_applied > 0) {
     g->pr_state = 0;   // ranks no longer hold
@@ -1597,25 +1624,15 @@ sp_status sp_get_dist(sp_graph *g, int32_t *dist, int32_t *parent, int out_on_de
   if (!g || !dist) return SP_EINVAL;
   if (g->state != 1) return SP_ESTATE;
   int launches = 0;
-  if (out_on_device && (!device_out(g, dist) || (parent && !device_out(g, parent))))
-    return SP_EINVAL;
-  // a page-locked, mapped host destination is written in place
-  int32_t *mdist = out_on_device ? nullptr : (int32_t *)mapped_host(dist);
-  int32_t *mparent = out_on_device || !parent ? nullptr : (int32_t *)mapped_host(parent);
-  if (out_on_device) {
-    sp::launch_unpack(g, dist, parent, &launches);
-  } else if (mdist && (!parent || mparent)) {
-    sp::launch_unpack(g, mdist, mparent, &launches);
-  } else {
-    sp::launch_unpack(g, g->out_dist, parent ? g->out_parent : nullptr, &launches);
-    cudaMemcpyAsync(dist, g->out_dist, (size_t)g->n * 4, cudaMemcpyDeviceToHost, g->stream);
-    if (parent)
-      cudaMemcpyAsync(parent, g->out_parent, (size_t)g->n * 4, cudaMemcpyDeviceToHost, g->stream);
-  }
+  DistOut o;
+  const sp_status rc = resolve_out(g, dist, parent, out_on_device, &o);
+  if (rc != SP_OK) return rc;
+  enqueue_out(g, o, &launches);
   if (cudaStreamSynchronize(g->stream) != cudaSuccess) {
     cudaGetLastError();
     return SP_ECUDA;
   }
+  take_out(g, o);
   return SP_OK;
 }
 

@@ -99,7 +99,7 @@ struct BatchBufs {
   long long strips_cap = 0;
   void *tmp = nullptr;
   size_t tmp_bytes = 0;
-  long long cap_in = 0;             // staging for host inputs
+  long long cap_in = 0;             // staging for host inputs (one allocation, at in_del_src)
   int *in_del_src = nullptr, *in_del_dst = nullptr;
   int *in_add_src = nullptr, *in_add_dst = nullptr, *in_add_w = nullptr;
 };
@@ -143,6 +143,14 @@ struct LoopArgs {
   int bits;
 };
 
+}  // namespace sp
+
+namespace sp {
+// Batches of at most this many updates are planned by one block, and read from
+// host memory in place; distances of at most kSmallOut vertices reach pageable
+// arrays through the handle's page-locked block (5 x 4 KB + 2 x 64 KB).
+constexpr int kSmallUpdates = 1024;
+constexpr int kSmallOut = 16384;
 }  // namespace sp
 
 struct sp_graph {
@@ -221,6 +229,7 @@ struct sp_graph {
   long long own_cap = 0;        // entries of each chunk-owner table
   sp::Ctl *ctl = nullptr;       // device
   sp::Ctl *ctl_host = nullptr;  // pinned
+  int *small_host = nullptr;    // behind it: small host batches, then small outputs
   int *out_dist = nullptr, *out_parent = nullptr;
   sp::BatchBufs bb;
   int source = -1;

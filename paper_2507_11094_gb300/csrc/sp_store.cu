@@ -839,6 +839,7 @@ unsigned search_grid(const sp_graph *g, long long ni) {
 // longer than the grid's.
 constexpr int kPlanT = 1024;             // threads at most: as many as the items need,
 constexpr int kPlanItems = 2 * kPlanT;   // two items each (a power of two of threads)
+static_assert(kPlanItems == 2 * kSmallUpdates, "two items an update");
 
 struct PlanArgs {
   SearchArgs in;

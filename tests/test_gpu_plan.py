@@ -95,3 +95,43 @@ def test_an_invalid_update_changes_nothing(k):
         np.testing.assert_array_equal(g.get_dist(), before)
         for x, y in zip(g.export_csr(), (ro, col, w)):
             np.testing.assert_array_equal(x, y)
+
+
+# distances through the handle's page-locked block and, above 16,384 vertices,
+# through a device buffer; batches read in place from pageable and page-locked
+# arrays, and one update more
+@pytest.mark.parametrize("n", [1, 3, 16383, 16384, 16385])
+@pytest.mark.parametrize("pinned", [False, True])
+def test_small_host_arrays(n, pinned):
+    import torch
+
+    def host(x):
+        if not pinned or not x.size:
+            return x
+        t = torch.empty(x.size, dtype=torch.int32, pin_memory=True)
+        t.numpy()[:] = x
+        return t.numpy()
+    m = min(4 * n, n * (n - 1))
+    ro, col, w = wl.er_digraph(n, m, 1, 100, seed=n) if m else (np.zeros(n + 1, np.int64),
+                                                                 np.zeros(0, np.int32),
+                                                                 np.zeros(0, np.int32))
+    ref = oracle.OracleGraph(n, ro, col, w)
+    rng = np.random.default_rng(n)
+    from oracle.invariants import check_sssp
+    with sp.Graph(n, ro, col, w, stream=torch.cuda.Stream()) as g:
+        g.sssp_init(0)
+        for k in (5, 5, 5, 1024, 1025):
+            if n == 1:
+                break
+            ro, col, _ = ref.csr()
+            keys = wl.csr_keys(n, ro, col) if col.size else np.array([1])
+            b = messy(rng, n, keys, k)
+            ref.apply(b)
+            d, p = np.full(n, -7, np.int32), np.full(n, -7, np.int32)
+            a = [host(x) for x in (b.del_src, b.del_dst, b.add_src, b.add_dst, b.add_w)]
+            g.apply_batch_get(*a, dist=d, parent=p)
+            np.testing.assert_array_equal(d, ref.dijkstra(0))
+            check_sssp(n, *ref.csr(), 0, d, p)
+        d, p = g.get_dist(parent=True)
+        np.testing.assert_array_equal(d, ref.dijkstra(0))
+        check_sssp(n, *ref.csr(), 0, d, p)
