@@ -117,7 +117,7 @@ struct Ctl {
   // insertions' corrections by number of updated edges (1, 2, 3)
   alignas(128) u64 tc_static;
   u64 tc_del[3], tc_ins[3];
-  u32 tc_ngiant, tc_nbig;          // staticTC: rows oriented by the whole grid, long lists
+  u32 tc_ngiant, tc_nbig, tc_nmid;        // staticTC: rows oriented by the whole grid, long lists
   alignas(128) u32 tc_bpos;        // ... long lists and short-list groups handed out so far
   alignas(128) u32 tc_spos;
   u64 tc_ntask[2];                 // corrections: tasks listed (deletions, insertions)

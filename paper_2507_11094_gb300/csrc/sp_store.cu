@@ -315,7 +315,7 @@ __device__ __forceinline__ void ctl_reset(Ctl *c, int full) {
   c->prd0 = c->prd1 = c->prd2 = 0.0;
   c->pr_iters = 0;
   c->tc_static = 0;
-  c->tc_ngiant = c->tc_nbig = c->tc_bpos = c->tc_spos = 0;
+  c->tc_ngiant = c->tc_nbig = c->tc_nmid = c->tc_bpos = c->tc_spos = 0;
   c->tc_ntask[0] = c->tc_ntask[1] = c->tc_tpos[0] = c->tc_tpos[1] = 0;
   c->tc_del[0] = c->tc_del[1] = c->tc_del[2] = 0;
   c->tc_ins[0] = c->tc_ins[1] = c->tc_ins[2] = 0;

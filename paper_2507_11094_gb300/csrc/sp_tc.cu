@@ -213,9 +213,11 @@ __global__ void __launch_bounds__(kThreads) k_tc_orient_giant(OrientArgs a) {
   if (bad) atomicCAS(&a.c->status, 0, SP_EINVAL);
 }
 
-// The lists longer than kWarpList, one block each, in a list of their own;
+// The lists longer than kWarpList, one block each, in a list of their own
+// (those longer than kLongList from its front, the others from its end: a
+// block that starts on a long one last would keep the rest of the GPU waiting);
 // the shorter ones are taken from the vertices in order, a warp each.
-constexpr u32 kWarpList = 32;
+constexpr u32 kWarpList = 32, kLongList = 256;
 
 __global__ void __launch_bounds__(kThreads) k_tc_lists(const u32 *__restrict__ cnt, int n, u32 *big,
                                                        Ctl *c) {
@@ -223,19 +225,23 @@ __global__ void __launch_bounds__(kThreads) k_tc_lists(const u32 *__restrict__ c
   const long long step = (long long)gridDim.x * kThreads;
   for (long long b = blockIdx.x * (long long)kThreads + (threadIdx.x & ~31); b < n; b += step) {
     const long long v = b + lane;
-    const bool is = v < n && cnt[v] > kWarpList;
-    const u32 m = __ballot_sync(kFull, is);
-    if (!m) continue;
-    u32 base = 0;
-    if (lane == 0) base = atomicAdd(&c->tc_nbig, (u32)__popc(m));
-    base = __shfl_sync(kFull, base, 0);
-    if (is) big[base + __popc(m & lanemask_lt())] = (u32)v;
+    const u32 d = v < n ? cnt[v] : 0u;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const bool is = k == 0 ? d > kLongList : d > kWarpList && d <= kLongList;
+      const u32 m = __ballot_sync(kFull, is);
+      if (!m) continue;
+      u32 base = 0;
+      if (lane == 0) base = atomicAdd(k == 0 ? &c->tc_nbig : &c->tc_nmid, (u32)__popc(m));
+      base = __shfl_sync(kFull, base, 0) + __popc(m & lanemask_lt());
+      if (is) big[k == 0 ? base : (u32)n - 1u - base] = (u32)v;
+    }
   }
 }
 
 constexpr u32 kEmpty = 0xFFFFFFFFu;       // no vertex has this id (n < 2^31)
-constexpr u32 kTabMax = 8192;             // slots of a block's table: half of them used
-constexpr u32 kWarpTab = 64;
+constexpr u32 kTabMax = 8192;             // slots of a block's table: half of them used at most
+constexpr u32 kWarpTab = 128, kWarpTabBits = 7;
 constexpr u32 kWK = 4;                    // probes per lane in flight
 
 __device__ __forceinline__ u32 hash_slot(u32 x, u32 bits) { return (x * 0x9E3779B1u) >> (32 - bits); }
@@ -311,14 +317,14 @@ __global__ void __launch_bounds__(kThreads) k_tc_count(Store st, int n, const u3
   __shared__ u32 s_u, s_pos;
   if (ld_cg_i32(&c->status) != 0) return;   // not symmetric (the same answer in every block)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const u32 nbig = ld_cg_u32(&c->tc_nbig);
+  const u32 nlong = ld_cg_u32(&c->tc_nbig), nbig = nlong + ld_cg_u32(&c->tc_nmid);
   u64 sum = 0;
   for (;;) {
     __syncthreads();
     if (threadIdx.x == 0) s_u = atomicAdd(&c->tc_bpos, 1u);
     __syncthreads();
     if (s_u >= nbig) break;
-    const u32 u = big[s_u];
+    const u32 u = big[s_u < nlong ? s_u : (u32)n - 1u - (s_u - nlong)];
     const u32 d = cnt[u];
     const u32 *out = (const u32 *)(st.adj + st.alt[u]);
     // members per grab: every warp gets some, a lane each
@@ -326,7 +332,7 @@ __global__ void __launch_bounds__(kThreads) k_tc_count(Store st, int n, const u3
     for (u32 part = 0; part < d; part += kTabMax / 2) {
       const u32 np = min(d - part, kTabMax / 2);
       u32 bits = 7;
-      while ((1u << bits) < 2 * np) ++bits;
+      while ((1u << bits) < 4 * np && (1u << bits) < kTabMax) ++bits;
       __syncthreads();
       for (u32 i = threadIdx.x; i < (1u << bits); i += kThreads) tab[i] = kEmpty;
       if (threadIdx.x == 0) s_pos = 0;
@@ -366,8 +372,8 @@ __global__ void __launch_bounds__(kThreads) k_tc_count(Store st, int n, const u3
       todo &= todo - 1;
       const u32 d = __shfl_sync(kFull, dl, o);
       const u32 *out = (const u32 *)(st.adj + __shfl_sync(kFull, al, o));
-      wtab[lane] = kEmpty;
-      wtab[lane + 32] = kEmpty;
+#pragma unroll
+      for (u32 k = 0; k < kWarpTab; k += 32) wtab[lane + k] = kEmpty;
       u32 len = 0;
       const u32 *p = nullptr;
       u32 v = 0;
@@ -377,9 +383,9 @@ __global__ void __launch_bounds__(kThreads) k_tc_count(Store st, int n, const u3
         p = (const u32 *)(st.adj + st.alt[v]);
       }
       __syncwarp();
-      if ((u32)lane < d) tab_put(wtab, 6, v);
+      if ((u32)lane < d) tab_put(wtab, kWarpTabBits, v);
       __syncwarp();
-      sum += count_lists(p, len, wtab, 6);
+      sum += count_lists(p, len, wtab, kWarpTabBits);
       __syncwarp();
     }
   }
