@@ -131,7 +131,7 @@ typedef struct {
     int64_t device_bytes;    /* device memory held by the handle            */
     int32_t state;           /* 0 = no distances, 1 = valid, 2 = SP_ESTATE  */
     int32_t num_sms;
-    int32_t pool_step;       /* edges a lane relaxes per step in the pool
+    int32_t pool_step;       /* edges of an entry relaxed per step in the pool
                                 schedule: 5 once at least 1/64 of the
                                 vertices have 5..8 out-edges, else 4 (an
                                 extension: speed only, never a distance) */

@@ -33,7 +33,7 @@ namespace {
 
 // kOpPool: the push fixedPoint with block-local relaxation (pool schedule)
 constexpr int kOpPush = 0, kOpInval = 1, kOpFlag = 2, kOpPool = 3, kOpPoolWide = 4;
-// the two pool kernels differ only in the edges a lane relaxes per step
+// the two pool kernels differ only in the edges of an entry relaxed per step
 __host__ __device__ constexpr bool is_pool(int op) { return op == kOpPool || op == kOpPoolWide; }
 constexpr int K = kEdgesPerLane;
 // block stages of the persistent loops (dynamic shared memory)
@@ -321,11 +321,11 @@ __device__ __forceinline__ void flush_far(Stage *st, u32 *pile, u32 *cnt, u32 *f
 // there.
 
 constexpr u32 kPoolUnknown = 0xFFFFFFFFu;   // entry degree not read yet
-// Pool edges per lane and step: four (kOpPool) or five (kOpPoolWide).  A warp
-// takes as many steps as its largest entry needs, and each step is one more
-// dependent round trip, so on a grid where batches gave many vertices a fifth
-// edge the wide steps win; where almost every vertex has at most four, the
-// narrow steps issue fewer instructions per sub-round and win.
+// Edges of a pool entry per step, a lane each: four (kOpPool) or five
+// (kOpPoolWide).  A warp takes as many steps as its largest entry needs, and
+// each step is one more dependent round trip, so on a grid where batches gave
+// many vertices a fifth edge the wide steps win; where almost every vertex has
+// at most four, the narrow steps serve eight entries per warp, not six.
 constexpr int kPoolWideShare = 64;   // wide when >= 1/64 of the vertices have 5..8 out-edges
 
 // Fetch a line toward L2 without waiting for it: a pool entry's next use is
@@ -400,140 +400,149 @@ struct PoolCounters {
 // block), starting from list 0, until the pool is empty or lim.pool_rounds
 // sub-rounds have run; then the entries left go to the global frontier qn.
 // An entry whose vertex holds a smaller distance by now is skipped (the
-// improvement that lowered it appended its own entry).  Each lane expands
-// one entry, kPU edges per step, with every edge's load, packed atomicMin and
-// (speculative) read of the target's row in flight together, so that a
-// target it improves enters the other list with its row already known.
-// Improved targets at or above thresh go to the far pile (pile != nullptr).
+// improvement that lowered it appended its own entry).  kPU lanes share an
+// entry and take one edge each per step, the edge's packed atomicMin and the
+// (speculative) read of its target's row in flight together, so that a target
+// it improves enters the other list with its row already known.  Improved
+// targets at or above thresh go to the far pile (pile != nullptr).
+//
+// A sub-round expands about 80 entries in 24 warps: it is one pass through
+// this code, bound by the latency of its instructions as much as by its three
+// dependent reads (L2 about 300 cycles, DRAM 720).  With a lane per entry and
+// kPU edges per lane, three warps walked kPU times the instructions while the
+// others waited (2047 x 1531 grid, 1%, two batches: 35.9 -> 24.5 ms; a sub-
+// round 3.9 -> 2.4 us).
 template <int kPU>
 __device__ __forceinline__ void pool_drain(const LoopArgs &a, Pool *pl, u32 thresh, u32 tag,
                                            u32 phase, const Queue &qn, u32 *pile, u32 *pcnt,
                                            u32 *pmin, Stage *sf, PoolCounters &pc) {
+  constexpr u32 kPer = 32 / kPU;    // entries per warp (lanes beyond them idle)
   const int lane = threadIdx.x & 31;
-  const u32 bs = blockDim.x;
+  const u32 sub_e = (u32)lane / kPU, sub_k = (u32)lane % kPU;
+  const u32 step = (blockDim.x >> 5) * kPer;
   const RowMeta *row = a.fwd.row;
   const u64 t_in = globaltimer_ns();
-  u32 p = 0, sub = 0;
+  // list p holds cn[c] entries; the counts rotate over three words, so that one
+  // barrier ends a sub-round (the third is cleared while nobody uses it)
+  u32 p = 0, c = 0, sub = 0;
   for (;;) {
     __syncthreads();
-    const u32 nraw = *(volatile u32 *)&pl->n[p];
+    const u32 nraw = *(volatile u32 *)&pl->n[c];
     const u32 n = nraw < kPoolCap ? nraw : kPoolCap;
     if (n == 0 || sub >= a.lim.pool_rounds) break;   // block-uniform
-    const u32 q = p ^ 1;
+    const u32 q = p ^ 1, cq = next3(c);
+    if (threadIdx.x == 0) pl->n[next3(cq)] = 0u;
     const uint4 *E = pl->e[p];
-    for (u32 base = threadIdx.x & ~31u; base < n; base += bs) {
-      const u32 i = base + lane;
+    uint4 *N = pl->e[q];
+    for (u32 base = (threadIdx.x >> 5) * kPer; base < n; base += step) {
+      const u32 i = base + sub_e;
       uint4 en = make_uint4(0u, 0u, 0u, 0u);
-      if (i < n) en = E[i];
+      if (sub_e < kPer && i < n) en = E[i];
       const u32 v = en.x, d = en.y;
       u32 deg = en.w;
       long long start = (long long)en.z << 2;
-      u64 sv = 0ull;
       if (deg != 0 && (v >= (u32)a.n ||
                        (deg != kPoolUnknown && start + (long long)deg > a.fwd.slots))) {
         atomicExch(&a.ctl->bad, 1);   // never expected: record and skip
         deg = 0;
       }
+      u64 sv = 0ull;
+      if (deg) sv = ld_cg_u64(a.s + v);
       if (deg == kPoolUnknown) {     // appended by the round's frontier expansion
         const int4 r = __ldg((const int4 *)(row + v));
-        sv = ld_cg_u64(a.s + v);
         start = (long long)(((u64)(u32)r.y << 32) | (u32)r.x);
         deg = (u32)r.z;
-      } else if (deg) {
-        sv = ld_cg_u64(a.s + v);
       }
-      // the first step's edges load together with the state word, before
+      const bool is_big = deg > (u32)kPoolDeg;
+      if (__any_sync(kFull, is_big)) {
+        // a vertex with more out-edges than an entry takes goes to the frontier
+        bool big[K] = {};
+        u32 bx[K] = {};
+        big[0] = is_big && sub_k == 0 && dist_of(sv) == d;
+        bx[0] = v;
+        if (big[0]) big[0] = atomicExch(a.qflag + v, tag) != tag;
+        enqueue(qn, row, bx, big, 1, pc.n_enq);
+        if (is_big) deg = 0;
+      }
+      // the first step's edge loads together with the state word, before
       // anything waits for either
-      int2 ed0[kPU];
-#pragma unroll
-      for (int k = 0; k < kPU; ++k)
-        ed0[k] = (u32)k < deg && deg <= (u32)kPoolDeg ? __ldg(a.fwd.adj + start + k)
-                                                       : make_int2(0, 0);
-      // a vertex with more out-edges than a lane takes goes to the frontier
-      bool big[K] = {};
-      u32 bx[K] = {};
-      big[0] = deg > (u32)kPoolDeg && dist_of(sv) == d;
-      bx[0] = v;
-      if (big[0]) big[0] = atomicExch(a.qflag + v, tag) != tag;
-      enqueue(qn, row, bx, big, 1, pc.n_enq);
-      if (deg > (u32)kPoolDeg) deg = 0;
+      int2 ed = sub_k < deg ? __ldg(a.fwd.adj + start + sub_k) : make_int2(0, 0);
       u32 steps = (deg + kPU - 1) / kPU;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const u32 y = __shfl_xor_sync(kFull, steps, o);
-        steps = y > steps ? y : steps;
-      }
-      bool live = false;
+      steps = __reduce_max_sync(kFull, steps);
+      const bool live = deg > 0 && dist_of(sv) == d;
       for (u32 t = 0; t < steps; ++t) {
-        int2 ed[kPU];
-#pragma unroll
-        for (int k = 0; k < kPU; ++k) {
-          const u32 e = t * kPU + (u32)k;
-          ed[k] = t == 0 ? ed0[k] : (e < deg ? __ldg(a.fwd.adj + start + e) : make_int2(0, 0));
-        }
-        if (t == 0) live = deg > 0 && dist_of(sv) == d;
-        // per edge: target, candidate distance, the target's old state (from
-        // the atomicMin) and its row (start / 4, degree), read together
-        u32 tx[K], nd[K], ms4[K];
-        int mdg[K];
-        u64 old[K];
-        bool act[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-          const u32 e = t * kPU + (u32)k;
-          act[k] = k < kPU && live && e < deg;
-          tx[k] = k < kPU ? (u32)ed[k < kPU ? k : 0].x : 0u;
-          nd[k] = k < kPU ? d + (u32)ed[k < kPU ? k : 0].y : kInf;
-          if (act[k]) {
-            ++pc.n_edges;
-            if (nd[k] >= kInf) {
-              pc.range_err = 1;
-              act[k] = false;
-            }
-          }
-          old[k] = act[k] ? atomicMin((unsigned long long *)(a.s + tx[k]), pack(nd[k], v)) : 0ull;
-          ms4[k] = 0;
-          mdg[k] = 0;
-          if (act[k]) {
-            const int4 r = __ldg((const int4 *)(row + tx[k]));
-            ms4[k] = (u32)((((u64)(u32)r.y << 32) | (u32)r.x) >> 2);
-            mdg[k] = r.z;
+        const u32 e = t * kPU + sub_k;
+        if (t > 0) ed = e < deg ? __ldg(a.fwd.adj + start + e) : make_int2(0, 0);
+        const u32 x = (u32)ed.x, nd = d + (u32)ed.y;
+        bool act = live && e < deg;
+        if (act) {
+          ++pc.n_edges;
+          if (nd >= kInf) {
+            pc.range_err = 1;
+            act = false;
           }
         }
-        bool near[K], far[K];
-        u32 fmin = 0xFFFFFFFFu;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-          near[k] = far[k] = false;
-          if (act[k] && pack(nd[k], v) < old[k]) {
-            ++pc.n_imp;
-            if (nd[k] < thresh) {
-              near[k] = true;
-            } else if (pile) {
-              far[k] = atomicExch(a.ftag + tx[k], phase) != phase;
-              if (far[k] && nd[k] < fmin) fmin = nd[k];
+        u64 old = 0ull;
+        int4 r = make_int4(0, 0, 0, 0);
+        if (act) {
+          old = atomicMin((unsigned long long *)(a.s + x), pack(nd, v));
+          r = __ldg((const int4 *)(row + x));
+        }
+        const bool better = act && pack(nd, v) < old;
+        pc.n_imp += better;
+        const bool near = better && nd < thresh;
+        const int xd = r.z;
+        // near targets of 1..kPoolDeg out-edges: entries of the other list
+        bool rest = near && xd > kPoolDeg;
+        const bool take = near && xd > 0 && !rest;
+        const u32 m = __ballot_sync(kFull, take);
+        if (m) {
+          u32 at = 0;
+          if (lane == 0) at = atomicAdd(&pl->n[cq], (u32)__popc(m));
+          at = __shfl_sync(kFull, at, 0) + __popc(m & lanemask_lt());
+          if (take) {
+            if (at < kPoolCap) {
+              const u32 xs4 = (u32)((((u64)(u32)r.y << 32) | (u32)r.x) >> 2);
+              N[at] = make_uint4(x, nd, xs4, (u32)xd);
+              // what the entry's expansion reads first: its edges
+              const int2 *e0 = a.fwd.adj + ((long long)xs4 << 2);
+              prefetch_l2(e0);
+              if (xd > 4) prefetch_l2(e0 + xd - 1);
+              ++pc.n_in;
+            } else {
+              rest = true;
             }
           }
         }
-        bool rest[K], want[K];
-        pool_push<true>(pl, q, tx, nd, near, kPU, ms4, mdg, rest, pc.n_in, row, a.fwd.adj);
-#pragma unroll
-        for (int k = 0; k < K; ++k)
-          want[k] = k < kPU && rest[k] && atomicExch(a.qflag + tx[k], tag) != tag;
-        enqueue(qn, row, tx, want, kPU, pc.n_enq);
-        if (pile) far_append(pile, pcnt, pmin, sf, tx, far, kPU, fmin);
+        if (__any_sync(kFull, rest)) {
+          bool want[K] = {};
+          u32 tx[K] = {};
+          want[0] = rest && atomicExch(a.qflag + x, tag) != tag;
+          tx[0] = x;
+          enqueue(qn, row, tx, want, 1, pc.n_enq);
+        }
+        if (pile) {
+          bool far[K] = {};
+          u32 tx[K] = {};
+          far[0] = better && !near;
+          if (__any_sync(kFull, far[0])) {
+            far[0] = far[0] && atomicExch(a.ftag + x, phase) != phase;
+            tx[0] = x;
+            far_append(pile, pcnt, pmin, sf, tx, far, 1, far[0] ? nd : 0xFFFFFFFFu);
+          }
+        }
       }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) pl->n[p] = 0u;
     p = q;
+    c = cq;
     ++sub;
   }
   pc.subs += sub;
   if (sub) pc.ns += globaltimer_ns() - t_in;
   // entries left when the budget ran out: to the global frontier
   {
-    const u32 nraw = *(volatile u32 *)&pl->n[p];
+    const u32 bs = blockDim.x;
+    const u32 nraw = *(volatile u32 *)&pl->n[c];
     const u32 n = nraw < kPoolCap ? nraw : kPoolCap;
     const uint4 *E = pl->e[p];
     for (u32 base = threadIdx.x & ~31u; base < n; base += bs) {
@@ -548,7 +557,7 @@ __device__ __forceinline__ void pool_drain(const LoopArgs &a, Pool *pl, u32 thre
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) pl->n[0] = pl->n[1] = 0u;
+  if (threadIdx.x == 0) pl->n[0] = pl->n[1] = pl->n[2] = 0u;
 }
 
 // --- edge operations ------------------------------------------------------
@@ -1425,7 +1434,7 @@ __global__ void __launch_bounds__(is_pool(OP) ? kPoolThreads : kPersistThreads, 
     if (is_pool(OP)) {
       pool.e[0] = (uint4 *)(dsm + kLoopSmem / sizeof(u32));
       pool.e[1] = pool.e[0] + kPoolCap;
-      pool.n[0] = pool.n[1] = 0u;
+      pool.n[0] = pool.n[1] = pool.n[2] = 0u;
     }
   }
   __syncthreads();

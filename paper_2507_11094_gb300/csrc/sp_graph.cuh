@@ -16,10 +16,10 @@ constexpr int kEdgesPerLane = kChunk / 32;
 constexpr int kSmallDeg = 8;
 constexpr int kLocalRoundCap = 4096;   // frontier edges of a single-block round
 constexpr int kPersistThreads = 768;    // persistent fixedPoint loops: 80 registers a thread
-// the push loop with block-local relaxation: a sub-round expands about a
-// hundred pool entries per block, so fewer threads with more registers each
-// (128) serve it better than 768 that spill
-constexpr int kPoolThreads = 512;
+// the push loop with block-local relaxation: a sub-round expands about 80 pool
+// entries per block, four or five lanes each (2047 x 1531 grid, 1%: 25.8 ms
+// with 512 threads, 24.4 with 768, 24.3 with 1,024)
+constexpr int kPoolThreads = 768;
 // Co-residency of cooperative launches from several handles at once (the
 // serving runtime's slots): a handle with a block share (sp_set_loop_blocks)
 // launches every cooperative kernel with at most that many blocks, each with
@@ -64,7 +64,7 @@ constexpr int kPoolDeg = 16;            // largest out-degree a pool entry may h
 constexpr u32 kPoolCap = 2048;          // entries per list
 struct Pool {
   uint4 *e[2];
-  u32 n[2];                             // appended so far (may pass kPoolCap)
+  u32 n[3];                             // appended so far (may pass kPoolCap), rotating
 };
 
 // One touched (store, row) pair of a batch, after sorting.
