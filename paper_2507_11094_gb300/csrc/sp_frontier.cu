@@ -1138,7 +1138,7 @@ __device__ __forceinline__ LocalState local_rounds(const LoopArgs &a, u32 cur, u
   LocalState out{};
   Ctl *c = a.ctl;
   const int lane = threadIdx.x & 31;
-  const u32 tid = threadIdx.x, bs = blockDim.x;
+  const u32 tid = threadIdx.x, bs = blockDim.x, round0 = round;
   u32 *lx[2] = {smem, smem + kLocalCap};
   u32 *ldeg[2] = {smem + 2 * kLocalCap, smem + 3 * kLocalCap};
   u32 *ld[2] = {smem + 4 * kLocalCap, smem + 5 * kLocalCap};
@@ -1284,21 +1284,25 @@ __device__ __forceinline__ LocalState local_rounds(const LoopArgs &a, u32 cur, u
       break;
     }
   }
-  // hand the frontier back through the global queue (duplicates are fine:
-  // the distributed rounds read each vertex's distance when they expand it)
+  // hand the frontier back through the global queue, every vertex once: the
+  // list may hold a vertex several times, and so more entries than the graph
+  // has vertices, which is what the queue has room for.  (No other round uses
+  // this one's tag; without a round the list is the queue's, which has none
+  // twice.)
   const u32 nxt = next3(cur);
   const Queue qn =
       make_queue(a.qent[nxt], a.qown[nxt], qcnt_ptr(c, nxt), a.qsv[nxt], scnt_ptr(c, nxt));
   u64 dummy = 0;
   const u32 nl = s_n[p];
   const u32 *Lx = lx[p];
+  const u32 tag = ld_cg_u32(&c->epoch) + round;
   for (u32 base = (threadIdx.x >> 5) * 32; base < nl; base += bs) {
     const u32 i = base + lane;
     bool want[K] = {};
     u32 xx[K] = {};
     if (i < nl) {
       xx[0] = Lx[i];
-      want[0] = true;
+      want[0] = round == round0 || atomicExch(a.qflag + xx[0], tag) != tag;
     }
     enqueue(qn, a.fwd.row, xx, want, 1, dummy);
   }

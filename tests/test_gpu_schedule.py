@@ -190,3 +190,23 @@ def test_pool_step_widens_as_batches_add_fifth_edges():
             d = check_all(g, ref, W.source, store=False)
             steps.append(g.info().pool_step)
     assert steps[0] == 4 and steps[-1] == 5, steps
+
+
+@pytest.mark.parametrize("n,deg", [(40, 30), (300, 40), (700, 20), (1499, 12), (3000, 10)])
+def test_single_block_rounds_hand_back_each_vertex_once(n, deg):
+    """Frontiers of single-block rounds hold a vertex once per improvement, on
+    small graphs with wide weights more often than there are vertices; handed
+    back to the grid they fit its queues, which have room for each vertex once."""
+    rng = np.random.default_rng(n)
+    key = np.unique(rng.integers(0, n, n * deg) * n + rng.integers(0, n, n * deg))
+    u, v = key // n, key % n
+    ro = np.zeros(n + 1, np.int64)
+    np.cumsum(np.bincount(u, minlength=n), out=ro[1:])
+    w = rng.integers(1, 100000, key.size).astype(np.int32)
+    ref = oracle.OracleGraph(n, ro, v.astype(np.int32), w)
+    with sp.Graph(n, ro, v.astype(np.int32), w) as g:
+        for edges in (256, 1024, 4096):
+            g.set_local_rounds(edges)
+            for src in rng.integers(0, n, 12):
+                g.sssp_init(int(src))
+                np.testing.assert_array_equal(g.get_dist(), ref.dijkstra(int(src)))
