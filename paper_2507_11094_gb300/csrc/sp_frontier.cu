@@ -861,68 +861,86 @@ __device__ __forceinline__ void process_chunk(Op &op, const int2 *ent, const u32
       web = kNoEdge;
     }
   }
-  const u32 l31 = __shfl_sync(kFull, web == kNoEdge ? kNoEdge : web + wdeg, 31);
-  const u32 wend = l31 == kNoEdge ? n_edges : l31;
-  const u32 ebeg = e0 + (u32)(KK * lane);
-  // owner of ebeg inside the window: last lane whose first edge <= ebeg
-  int o = 0;
-#pragma unroll
-  for (int step = 16; step > 0; step >>= 1) {
-    const u32 ebc = __shfl_sync(kFull, web, (o + step) & 31);
-    if (o + step < 32 && ebc <= ebeg) o += step;
-  }
-  u32 slot = jw + (u32)o;
-  u32 v = __shfl_sync(kFull, wv, o), eb = __shfl_sync(kFull, web, o);
-  u32 deg = __shfl_sync(kFull, wdeg, o), dv = __shfl_sync(kFull, wd, o);
-  long long start = (long long)shfl64((u64)wstart, o);
-  if (ebeg < e_end && ebeg >= wend) {
-    // beyond the window (many tiny rows in one chunk): search the queue
-    u32 lo = jw, hi = n_ent - 1;
-    while (lo < hi) {
-      const u32 mid = (lo + hi + 1) >> 1;
-      if ((u32)__ldcg(&ent[mid].y) <= ebeg) lo = mid; else hi = mid - 1;
-    }
-    slot = lo;
-    const int2 en = __ldcg(ent + slot);
-    v = (u32)en.x;
-    eb = (u32)en.y;
-    const RowMeta rm = st.row[v];
-    deg = (u32)rm.deg;
-    start = rm.start;
-    dv = op.vdata(v);
-    o = 32;
-  }
   bool act[KK];
   u32 ov[KK], od[KK];
   int2 ed[KK];
   u64 sx[KK];
+  if (__shfl_sync(kFull, web, 1) >= e_end) {
+    // one row holds all of these edges (a hub's chunks): lanes take consecutive
+    // ones, two lines a load instead of sixteen, and nothing is searched.  The
+    // L1 looks up a line per clock, and half of a static solve's lookups were
+    // its edges (R-MAT 20: 556 -> 531 us).
+    const u32 v = __shfl_sync(kFull, wv, 0), eb = __shfl_sync(kFull, web, 0);
+    const u32 dv = __shfl_sync(kFull, wd, 0);
+    const long long start = (long long)shfl64((u64)wstart, 0);
 #pragma unroll
-  for (int k = 0; k < KK; ++k) {
-    const u32 e = ebeg + (u32)k;
-    act[k] = e < e_end;
-    const int nl = (o + 1) & 31;
-    const u32 nv = __shfl_sync(kFull, wv, nl), neb = __shfl_sync(kFull, web, nl);
-    const u32 ndeg = __shfl_sync(kFull, wdeg, nl), nd = __shfl_sync(kFull, wd, nl);
-    const long long nstart = (long long)shfl64((u64)wstart, nl);
-    if (act[k] && e >= eb + deg) {  // next entry (entries are contiguous in edge space)
-      ++slot;
-      if (o + 1 < 32) {
-        ++o;
-        v = nv; eb = neb; deg = ndeg; dv = nd; start = nstart;
-      } else {
-        const int2 en = __ldcg(ent + slot);
-        v = (u32)en.x;
-        eb = (u32)en.y;
-        const RowMeta rm = st.row[v];
-        deg = (u32)rm.deg;
-        start = rm.start;
-        dv = op.vdata(v);
-        o = 32;
-      }
+    for (int k = 0; k < KK; ++k) {
+      const u32 e = e0 + (u32)(32 * k + lane);
+      act[k] = e < e_end;
+      ov[k] = v;
+      od[k] = dv;
+      ed[k] = act[k] ? __ldg(st.adj + start + (e - eb)) : make_int2(0, 0);
     }
-    ov[k] = v;
-    od[k] = dv;
-    ed[k] = act[k] ? __ldg(st.adj + start + (e - eb)) : make_int2(0, 0);
+  } else {
+    const u32 l31 = __shfl_sync(kFull, web == kNoEdge ? kNoEdge : web + wdeg, 31);
+    const u32 wend = l31 == kNoEdge ? n_edges : l31;
+    const u32 ebeg = e0 + (u32)(KK * lane);
+    // owner of ebeg inside the window: last lane whose first edge <= ebeg
+    int o = 0;
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1) {
+      const u32 ebc = __shfl_sync(kFull, web, (o + step) & 31);
+      if (o + step < 32 && ebc <= ebeg) o += step;
+    }
+    u32 slot = jw + (u32)o;
+    u32 v = __shfl_sync(kFull, wv, o), eb = __shfl_sync(kFull, web, o);
+    u32 deg = __shfl_sync(kFull, wdeg, o), dv = __shfl_sync(kFull, wd, o);
+    long long start = (long long)shfl64((u64)wstart, o);
+    if (ebeg < e_end && ebeg >= wend) {
+      // beyond the window (many tiny rows in one chunk): search the queue
+      u32 lo = jw, hi = n_ent - 1;
+      while (lo < hi) {
+        const u32 mid = (lo + hi + 1) >> 1;
+        if ((u32)__ldcg(&ent[mid].y) <= ebeg) lo = mid; else hi = mid - 1;
+      }
+      slot = lo;
+      const int2 en = __ldcg(ent + slot);
+      v = (u32)en.x;
+      eb = (u32)en.y;
+      const RowMeta rm = st.row[v];
+      deg = (u32)rm.deg;
+      start = rm.start;
+      dv = op.vdata(v);
+      o = 32;
+    }
+#pragma unroll
+    for (int k = 0; k < KK; ++k) {
+      const u32 e = ebeg + (u32)k;
+      act[k] = e < e_end;
+      const int nl = (o + 1) & 31;
+      const u32 nv = __shfl_sync(kFull, wv, nl), neb = __shfl_sync(kFull, web, nl);
+      const u32 ndeg = __shfl_sync(kFull, wdeg, nl), nd = __shfl_sync(kFull, wd, nl);
+      const long long nstart = (long long)shfl64((u64)wstart, nl);
+      if (act[k] && e >= eb + deg) {  // next entry (entries are contiguous in edge space)
+        ++slot;
+        if (o + 1 < 32) {
+          ++o;
+          v = nv; eb = neb; deg = ndeg; dv = nd; start = nstart;
+        } else {
+          const int2 en = __ldcg(ent + slot);
+          v = (u32)en.x;
+          eb = (u32)en.y;
+          const RowMeta rm = st.row[v];
+          deg = (u32)rm.deg;
+          start = rm.start;
+          dv = op.vdata(v);
+          o = 32;
+        }
+      }
+      ov[k] = v;
+      od[k] = dv;
+      ed[k] = act[k] ? __ldg(st.adj + start + (e - eb)) : make_int2(0, 0);
+    }
   }
 #pragma unroll
   for (int k = 0; k < KK; ++k) sx[k] = act[k] ? op.load(ed[k]) : 0ull;
