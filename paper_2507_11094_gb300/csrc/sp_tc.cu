@@ -241,7 +241,8 @@ __global__ void __launch_bounds__(kThreads) k_tc_lists(const u32 *__restrict__ c
 
 constexpr u32 kEmpty = 0xFFFFFFFFu;       // no vertex has this id (n < 2^31)
 constexpr u32 kTabMax = 8192;             // slots of a block's table: half of them used at most
-constexpr u32 kWarpTab = 128, kWarpTabBits = 7;
+constexpr u32 kWarpTab = 1024, kWarpTabBits = 10;   // a warp's, for lists of up to kWarpList
+static_assert(kWarpTab * (kThreads / 32) <= kTabMax, "the warps' tables share the block's");
 constexpr u32 kWK = 4;                    // probes per lane in flight
 
 __device__ __forceinline__ u32 hash_slot(u32 x, u32 bits) { return (x * 0x9E3779B1u) >> (32 - bits); }
@@ -310,10 +311,12 @@ __device__ __forceinline__ u32 count_lists(const u32 *ptr, u32 len, const u32 *t
 // than half a block's table is taken in parts (a triangle's w lies in exactly
 // one of them).  What bounds it is the walk: sum over the oriented edges
 // u -> v of |out(v)| list words through L2, one or two shared-memory probes
-// each.
+// each; a warp waits for its lane with the longest chain of them, so tables are
+// as sparse as the memory allows (an eighth or less filled up to 1,024 members;
+// symmetric R-MAT 18: 710 us at a quarter, 544 so).
 __global__ void __launch_bounds__(kThreads) k_tc_count(Store st, int n, const u32 *__restrict__ cnt,
                                                        const u32 *__restrict__ big, Ctl *c) {
-  __shared__ u32 tab[kTabMax];
+  __shared__ __align__(16) u32 tab[kTabMax];
   __shared__ u32 s_u, s_pos;
   if (ld_cg_i32(&c->status) != 0) return;   // not symmetric (the same answer in every block)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -332,7 +335,7 @@ __global__ void __launch_bounds__(kThreads) k_tc_count(Store st, int n, const u3
     for (u32 part = 0; part < d; part += kTabMax / 2) {
       const u32 np = min(d - part, kTabMax / 2);
       u32 bits = 7;
-      while ((1u << bits) < 4 * np && (1u << bits) < kTabMax) ++bits;
+      while ((1u << bits) < 8 * np && (1u << bits) < kTabMax) ++bits;
       __syncthreads();
       for (u32 i = threadIdx.x; i < (1u << bits); i += kThreads) tab[i] = kEmpty;
       if (threadIdx.x == 0) s_pos = 0;
@@ -373,7 +376,8 @@ __global__ void __launch_bounds__(kThreads) k_tc_count(Store st, int n, const u3
       const u32 d = __shfl_sync(kFull, dl, o);
       const u32 *out = (const u32 *)(st.adj + __shfl_sync(kFull, al, o));
 #pragma unroll
-      for (u32 k = 0; k < kWarpTab; k += 32) wtab[lane + k] = kEmpty;
+      for (u32 k = 0; k < kWarpTab / 4; k += 32)
+        ((uint4 *)wtab)[lane + k] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
       u32 len = 0;
       const u32 *p = nullptr;
       u32 v = 0;
