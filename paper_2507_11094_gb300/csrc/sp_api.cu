@@ -227,7 +227,7 @@ bool find_input_nodes(sp_graph *g) {
     if (cudaGraphNodeGetType(nd, &t) != cudaSuccess || t != cudaGraphNodeTypeKernel) continue;
     cudaKernelNodeParams p = {};
     if (cudaGraphKernelNodeGetParams(nd, &p) != cudaSuccess) return false;
-    if (p.func == sp::batch_sort_fn()) g->bg_sort = nd;
+    if (sp::is_batch_sort(p.func)) g->bg_sort = nd;
     else if (p.func == sp::inval_fn()) g->bg_inval = nd;
     else if (p.func == sp::search_fn(g)) g->bg_search = nd;
     else if (p.func == sp::plan_fn()) g->bg_plan = nd;

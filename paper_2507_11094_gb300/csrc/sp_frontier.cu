@@ -868,8 +868,8 @@ __device__ __forceinline__ void process_chunk(Op &op, const int2 *ent, const u32
   if (__shfl_sync(kFull, web, 1) >= e_end) {
     // one row holds all of these edges (a hub's chunks): lanes take consecutive
     // ones, two lines a load instead of sixteen, and nothing is searched.  The
-    // L1 looks up a line per clock, and half of a static solve's lookups were
-    // its edges (R-MAT 20: 556 -> 531 us).
+    // L1 looks up a line per clock, and a quarter of a static solve's lookups
+    // were for these edges (R-MAT 20: 556 -> 531 us).
     const u32 v = __shfl_sync(kFull, wv, 0), eb = __shfl_sync(kFull, web, 0);
     const u32 dv = __shfl_sync(kFull, wd, 0);
     const long long start = (long long)shfl64((u64)wstart, 0);

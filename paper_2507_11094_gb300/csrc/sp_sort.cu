@@ -22,13 +22,13 @@
 #include "sp_graph.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace sp {
 
 namespace {
 
-constexpr int kBits = 9;               // digits of the batch sort
-constexpr int kBins = 1 << kBits;
+constexpr int kBinsMax = 1 << 10;       // digits of the batch sort: 9 or 10 bits
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxDigit = 8;           // digits of the edge sort
@@ -235,12 +235,24 @@ k_scatter(const u64 *__restrict__ keys, const u32 *__restrict__ vals, long long 
 // (store, row) -- the grouping that lets every touched row be merged once
 // (updateCSRDel + updateCSRAdd of the DynSSSP driver as one sort-merge).
 //
-// Block b owns the contiguous chunk [b*C, (b+1)*C) of item positions.  Per
-// 9-bit digit pass:
+// Block b owns a contiguous chunk of item positions.  Items arrive forward
+// store first and, within a store, deletions first, and every pass is stable:
+// so the kind bit is never sorted on, and where the grid has two blocks or
+// more, half of them sorts the forward items and half the reverse ones, each
+// within its own half of the positions, and the store's bit is not sorted on
+// either.  That leaves 2 * bits key bits, in digits of ten bits where this
+// saves a pass over nine (19, 20 and 23 to 25 bits an id): on R-MAT 20 four
+// passes instead of five, on R-MAT 22 five (nine bits) instead of six.  A pass
+// is two grid barriers, a scatter and a read back.  A batch and its undo of
+// 1,000,000 updates on R-MAT 22: 2,398 -> 2,369 us, of 161,000 on 32 graphs
+// together: 1,070 -> 1,058 us, of 20,971 pairs in the triangle count: 1,012 ->
+// 987 us; R-MAT 20 and 167,772 updates: 816 us either way (the searches beside
+// the sort take as long).  A batch within one tile is sorted by one block with
+// the store's bit.  Per pass:
 //   1. the block counts the digit over its chunk and writes the counts as
 //      row b of a table (chunk-major);                     -- grid barrier
-//   2. thread d reads column d (coalesced across the warp): the digit's
-//      total and its count in earlier chunks; a block scan of the totals
+//   2. the threads read the table's columns (coalesced across the warp): a
+//      digit's total and its count in earlier chunks of its half; a block scan of the totals
 //      gives the digit bases;
 //   3. per sub-tile of kBTile items (warp w holds items w*256 .. w*256+255,
 //      eight per lane): each warp ranks its items with match_any against
@@ -252,17 +264,17 @@ k_scatter(const u64 *__restrict__ keys, const u32 *__restrict__ vals, long long 
 // the scatter.  Data other blocks wrote is read through L2 (.cg), and
 // loads are issued in unrolled batches so that their latencies overlap.
 // ---------------------------------------------------------------------------
-constexpr int kBT = 512;                  // threads per block (one digit each)
+constexpr int kBT = 512;                  // threads per block (one or two digits each)
 constexpr int kBW = kBT / 32;
 constexpr int kBItems = 8;
 constexpr int kBTile = kBT * kBItems;     // items per sub-tile
 constexpr int kBWarpItems = 32 * kBItems; // items per warp and sub-tile
-static_assert(kBT == kBins, "one digit per thread");
 static_assert(kBT == kST, "bscan512");
 // dynamic shared memory: staged keys and values, per-warp digit counters,
 // four per-digit arrays
-constexpr size_t kBSmem =
-    (size_t)kBTile * (sizeof(u64) + sizeof(u32)) + (size_t)(kBW * kBins + 4 * kBins) * 4;
+template <int KB>
+constexpr size_t kBSmem = (size_t)kBTile * (sizeof(u64) + sizeof(u32)) +
+                          (size_t)(kBW * kBT + 4 * (1 << KB)) * 4;
 
 struct BatchSortArgs {
   const int *ds, *dd, *as, *ad, *aw;
@@ -270,12 +282,13 @@ struct BatchSortArgs {
   int n, bits, passes;
   u64 *kbuf[2];
   u32 *vbuf[2];
-  u32 *tab;          // [G][kBins] digit counts per chunk
+  u32 *tab;          // [G][1 << KB] digit counts per chunk
   Seg *seg;
   Ctl *ctl;
   unsigned long long wait_ns;
   u32 miss_site;         // test hook of the bounded waits (Limits::miss_site)
   u32 n_items, chunk;
+  u32 halves;        // 2: half of the grid per store
 };
 
 __device__ __forceinline__ u64 shfl64_up1(u64 x) {
@@ -289,12 +302,18 @@ __device__ __forceinline__ u32 sub_pos(int k) {
   return (threadIdx.x >> 5) * kBWarpItems + k * 32 + (threadIdx.x & 31);
 }
 
+// KB bits a digit.  Per-warp digit counters: 32-bit at nine bits, pairs of 16
+// bits at ten (a sub-tile has 4,096 items), so 512 words a warp either way.
+template <int KB>
 __global__ void __launch_bounds__(kBT) k_batch_sort(BatchSortArgs a) {
+  constexpr int kBins = 1 << KB, kDT = kBins / kBT;   // digits, and digits per thread
+  static_assert(kDT == 1 || kDT == 2, "counter words");
+  using Cnt = std::conditional_t<kDT == 1, u32, unsigned short>;
   extern __shared__ __align__(16) unsigned char smraw[];
   u64 *s_key = (u64 *)smraw;                         // [kBTile]
   u32 *s_val = (u32 *)(s_key + kBTile);              // [kBTile]
-  u32 *s_wc = s_val + kBTile;                        // [kBW][kBins] per-warp digit counts
-  u32 *s_off = s_wc + kBW * kBins;                   // global start of digit (next sub-tile)
+  u32 *s_wc = s_val + kBTile;                        // [kBW][kBT] words of per-warp digit counts
+  u32 *s_off = s_wc + kBW * kBT;                   // global start of digit (next sub-tile)
   u32 *s_run = s_off + kBins;
   u32 *s_loc = s_run + kBins;                        // sub-tile start of digit
   u32 *s_hist = s_loc + kBins;                       // digit counts
@@ -302,7 +321,10 @@ __global__ void __launch_bounds__(kBT) k_batch_sort(BatchSortArgs a) {
   Ctl *c = a.ctl;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const u32 G = gridDim.x, b = blockIdx.x;
-  const u32 cb = min(b * a.chunk, a.n_items), ce = min(cb + a.chunk, a.n_items);
+  // this block's half of the grid and of the positions, and its chunk there
+  const u32 Gh = G / a.halves, half = b / Gh, bh = b - half * Gh;
+  const u32 nh0 = half * (a.n_items / a.halves), nh1 = nh0 + a.n_items / a.halves;
+  const u32 cb = min(nh0 + bh * a.chunk, nh1), ce = min(cb + a.chunk, nh1);
   const bool one = ce - cb <= (u32)kBTile;           // the chunk is one sub-tile
   u64 *bar = &c->bar_sort;
   u64 nbar = 0;
@@ -316,7 +338,8 @@ __global__ void __launch_bounds__(kBT) k_batch_sort(BatchSortArgs a) {
   // low key bit is 0 for a deletion and 1 for an insertion, so a deletion
   // sorts before an insertion of the same edge) with the first digit's
   // counts; an invalid id or weight raises SP_EINVAL (nothing will change)
-  s_hist[t] = 0;
+#pragma unroll
+  for (int e = 0; e < kDT; ++e) s_hist[e * kBT + t] = 0;
   __syncthreads();
   for (u32 tb = cb; tb < ce; tb += kBTile) {
     int u[kBItems], v[kBItems], w[kBItems];
@@ -360,49 +383,61 @@ __global__ void __launch_bounds__(kBT) k_batch_sort(BatchSortArgs a) {
       if (i < ce) {
         a.kbuf[0][i] = rk[k];
         a.vbuf[0][i] = rv[k];
-        atomicAdd(&s_hist[rk[k] & (kBins - 1)], 1u);
+        atomicAdd(&s_hist[(rk[k] >> 1) & (kBins - 1)], 1u);
       }
     }
   }
   __syncthreads();
-  a.tab[(size_t)b * kBins + t] = s_hist[t];
+#pragma unroll
+  for (int e = 0; e < kDT; ++e) a.tab[(size_t)b * kBins + e * kBT + t] = s_hist[e * kBT + t];
 
   for (int p = 0; p < a.passes; ++p) {
     if (coop_barrier(bar, ++nbar * G, c, a.wait_ns, 4, a.miss_site)) return;
-    const int shift = p * kBits;
-    // digit bases of this chunk: thread t sums digits 4*(t % 128) .. +3 over
-    // the rows q = t / 128 (mod 4) with 16-byte loads; the four partial sums
-    // of each digit meet in shared memory (s_loc holds the totals, s_run the
-    // counts of earlier chunks)
+    const int shift = 1 + p * KB;   // above the kind bit
+    // digit bases of this chunk: thread t sums digits 4*(t % kPer) .. +3 over
+    // its half's rows q = t / kPer (mod kRows) with 16-byte loads; the partial
+    // sums of each digit meet in shared memory (s_loc holds the totals, s_run
+    // the counts of earlier chunks)
     {
-      const u32 dq = (u32)(t & 127) * 4, rg = (u32)t >> 7;
+      constexpr u32 kPer = kBins / 4, kRows = kBT / kPer;
+      const u32 *tab = a.tab + (size_t)half * Gh * kBins;
+      const u32 dq = ((u32)t & (kPer - 1)) * 4, rg = (u32)t / kPer;
       uint4 tot = make_uint4(0u, 0u, 0u, 0u), pre = tot;
-      for (u32 q0 = rg; q0 < G; q0 += 4 * 8) {
+      for (u32 q0 = rg; q0 < Gh; q0 += kRows * 8) {
         uint4 x[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const u32 q = q0 + 4 * u;
-          x[u] = q < G ? __ldcg((const uint4 *)(a.tab + (size_t)q * kBins + dq))
-                       : make_uint4(0u, 0u, 0u, 0u);
+          const u32 q = q0 + kRows * u;
+          x[u] = q < Gh ? __ldcg((const uint4 *)(tab + (size_t)q * kBins + dq))
+                        : make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const bool before = q0 + 4 * u < b;
+          const bool before = q0 + kRows * u < bh;
           tot.x += x[u].x; tot.y += x[u].y; tot.z += x[u].z; tot.w += x[u].w;
           if (before) { pre.x += x[u].x; pre.y += x[u].y; pre.z += x[u].z; pre.w += x[u].w; }
         }
       }
-      s_loc[t] = 0;
-      s_run[t] = 0;
+#pragma unroll
+      for (int e = 0; e < kDT; ++e) {
+        s_loc[e * kBT + t] = 0;
+        s_run[e * kBT + t] = 0;
+      }
       __syncthreads();
       atomicAdd(&s_loc[dq], tot.x); atomicAdd(&s_loc[dq + 1], tot.y);
       atomicAdd(&s_loc[dq + 2], tot.z); atomicAdd(&s_loc[dq + 3], tot.w);
       atomicAdd(&s_run[dq], pre.x); atomicAdd(&s_run[dq + 1], pre.y);
       atomicAdd(&s_run[dq + 2], pre.z); atomicAdd(&s_run[dq + 3], pre.w);
       __syncthreads();
-      u32 all;
-      const u32 base = bscan512(s_loc[t], ws, &all);
-      s_off[t] = base + s_run[t];
+      u32 all, mine = 0;
+#pragma unroll
+      for (int e = 0; e < kDT; ++e) mine += s_loc[t * kDT + e];
+      u32 base = nh0 + bscan512(mine, ws, &all);
+#pragma unroll
+      for (int e = 0; e < kDT; ++e) {
+        s_off[t * kDT + e] = base + s_run[t * kDT + e];
+        base += s_loc[t * kDT + e];
+      }
     }
     const u64 *kin = a.kbuf[p & 1];
     const u32 *vin = a.vbuf[p & 1];
@@ -416,7 +451,8 @@ __global__ void __launch_bounds__(kBT) k_batch_sort(BatchSortArgs a) {
           rk[k] = i < ce ? __ldcg(kin + i) : 0ull;
           rv[k] = i < ce ? __ldcg(vin + i) : 0u;
         }
-        s_hist[t] = 0;
+#pragma unroll
+        for (int e = 0; e < kDT; ++e) s_hist[e * kBT + t] = 0;
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < kBItems; ++k)
@@ -424,34 +460,41 @@ __global__ void __launch_bounds__(kBT) k_batch_sort(BatchSortArgs a) {
         __syncthreads();
       }
       {
-        u32 all;
-        s_loc[t] = bscan512(s_hist[t], ws, &all);
+        u32 all, mine = 0;
 #pragma unroll
-        for (int w = 0; w < kBW; ++w) s_wc[w * kBins + t] = 0;
+        for (int e = 0; e < kDT; ++e) mine += s_hist[t * kDT + e];
+        u32 base = bscan512(mine, ws, &all);
+#pragma unroll
+        for (int e = 0; e < kDT; ++e) {
+          s_loc[t * kDT + e] = base;
+          base += s_hist[t * kDT + e];
+        }
+#pragma unroll
+        for (int w = 0; w < kBW; ++w) s_wc[w * kBT + t] = 0;
       }
       __syncthreads();
       // stable rank within the warp's items (rows k, then lanes)
       u32 lr[kBItems];
-      u32 *wc = s_wc + warp * kBins;
+      Cnt *wc = (Cnt *)(s_wc + warp * kBT);
 #pragma unroll
       for (int k = 0; k < kBItems; ++k) {
         const bool valid = tb + sub_pos(k) < ce;
         const u32 d = (u32)((rk[k] >> shift) & (kBins - 1));
-        const u32 peers = digit_peers<kBits>(d, valid);
+        const u32 peers = digit_peers<KB>(d, valid);
         const u32 rank = __popc(peers & lt);
-        const u32 before = valid ? wc[d] : 0u;
+        const u32 before = valid ? (u32)wc[d] : 0u;
         __syncwarp();
-        if (valid && rank == 0) wc[d] = before + __popc(peers);
+        if (valid && rank == 0) wc[d] = (Cnt)(before + __popc(peers));
         __syncwarp();
         lr[k] = before + rank;
       }
       __syncthreads();
-      {   // digit t: offsets of the warps
+      {   // word t (a digit, or two of 16 bits): offsets of the warps
         u32 run = 0;
 #pragma unroll
         for (int w = 0; w < kBW; ++w) {
-          const u32 x = s_wc[w * kBins + t];
-          s_wc[w * kBins + t] = run;
+          const u32 x = s_wc[w * kBT + t];
+          s_wc[w * kBT + t] = run;
           run += x;
         }
       }
@@ -479,13 +522,15 @@ __global__ void __launch_bounds__(kBT) k_batch_sort(BatchSortArgs a) {
         }
       }
       __syncthreads();
-      s_off[t] += s_hist[t];
+#pragma unroll
+      for (int e = 0; e < kDT; ++e) s_off[e * kBT + t] += s_hist[e * kBT + t];
       __syncthreads();
     }
     if (coop_barrier(bar, ++nbar * G, c, a.wait_ns, 4, a.miss_site)) return;
     if (p + 1 < a.passes) {   // the next digit's counts over this chunk
-      const int nshift = shift + kBits;
-      s_hist[t] = 0;
+      const int nshift = shift + KB;
+#pragma unroll
+      for (int e = 0; e < kDT; ++e) s_hist[e * kBT + t] = 0;
       __syncthreads();
       for (u32 tb = cb; tb < ce; tb += kBTile) {
 #pragma unroll
@@ -499,7 +544,8 @@ __global__ void __launch_bounds__(kBT) k_batch_sort(BatchSortArgs a) {
           if (tb + sub_pos(k) < ce) atomicAdd(&s_hist[(rk[k] >> nshift) & (kBins - 1)], 1u);
       }
       __syncthreads();
-      a.tab[(size_t)b * kBins + t] = s_hist[t];
+#pragma unroll
+      for (int e = 0; e < kDT; ++e) a.tab[(size_t)b * kBins + e * kBT + t] = s_hist[e * kBT + t];
     }
   }
 
@@ -608,43 +654,57 @@ size_t sort_tmp_bytes(long long n) {
   return (size_t)(tiles * kSBins + kSBins + 64) * sizeof(u32) + 256;
 }
 
-int batch_sort_blocks(int num_sms) {
+// Co-resident blocks per SM of one digit width; 0 if it cannot run.
+template <int KB>
+static int sort_per_sm() {
   int per_sm = 0;
-  if (cudaFuncSetAttribute(k_batch_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)std::max(kBSmem, kExclusiveSmem)) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_sort, kBT, kBSmem) !=
-          cudaSuccess ||
-      per_sm < 1)
+  if (cudaFuncSetAttribute(k_batch_sort<KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)std::max(kBSmem<KB>, kExclusiveSmem)) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_sort<KB>, kBT, kBSmem<KB>) !=
+          cudaSuccess)
     return 0;
-  return per_sm * num_sms;
+  return per_sm;
+}
+
+int batch_sort_blocks(int num_sms) {
+  return std::max(0, std::min(sort_per_sm<9>(), sort_per_sm<10>())) * num_sms;
 }
 
 size_t batch_sort_tmp_bytes(int max_blocks) {
-  return (size_t)kBins * std::max(max_blocks, 1) * sizeof(u32) + 256;
+  return (size_t)kBinsMax * std::max(max_blocks, 1) * sizeof(u32) + 256;
 }
 
 namespace {
 
-// Dynamic shared memory of a launch: a handle with a block share gives each
-// block an SM of its own (kExclusiveSmem).
-size_t sort_smem(const sp_graph *g) {
-  return g->loop_blocks_user > 0 ? std::max(kBSmem, kExclusiveSmem) : kBSmem;
-}
+// One launch of the batch sort: its kernel and dynamic shared memory.
+struct SortLaunch {
+  void (*fn)(BatchSortArgs);
+  size_t smem;
+  int G;
+};
 
 // Arguments and grid of the batch sort for these inputs.
-int batch_sort_args(sp_graph *g, const int *ds, const int *dd, long long nd, const int *as,
-                    const int *ad, const int *aw, long long na, BatchSortArgs &a) {
+SortLaunch batch_sort_args(sp_graph *g, const int *ds, const int *dd, long long nd,
+                           const int *as, const int *ad, const int *aw, long long na,
+                           BatchSortArgs &a) {
   const long long ni = 2 * (nd + na);
   BatchBufs &bb = g->bb;
-  int G = (int)std::min<long long>((ni + kBTile - 1) / kBTile, g->sort_blocks);
-  if (g->loop_blocks_user > 0 && g->loop_blocks_user < G) G = g->loop_blocks_user;
-  if (G < 1) G = 1;
+  int cap = g->sort_blocks;
+  if (g->loop_blocks_user > 0 && g->loop_blocks_user < cap) cap = g->loop_blocks_user;
+  // two blocks or more: as many for either store
+  a.halves = ni > kBTile && cap >= 2 ? 2 : 1;
+  const long long nh = ni / (int)a.halves;
+  const int Gh = (int)std::max(1ll, std::min<long long>((nh + kBTile - 1) / kBTile,
+                                                        cap / (int)a.halves));
+  const int G = Gh * (int)a.halves;
   a.ds = ds; a.dd = dd; a.as = as; a.ad = ad; a.aw = aw;
   a.nd = nd; a.na = na;
   a.n = g->n;
   a.bits = g->bits;
-  const int key_bits = 2 * g->bits + 2;
-  a.passes = (key_bits + kBits - 1) / kBits;
+  const int key_bits = 2 * g->bits + (a.halves == 1 ? 1 : 0);
+  const int p9 = std::max((key_bits + 8) / 9, 1), p10 = std::max((key_bits + 9) / 10, 1);
+  const bool wide = p10 < p9;
+  a.passes = wide ? p10 : p9;
   // the last pass writes keys/vals
   const int odd = a.passes & 1;
   a.kbuf[0] = odd ? bb.keys_alt : bb.keys;
@@ -657,24 +717,29 @@ int batch_sort_args(sp_graph *g, const int *ds, const int *dd, long long nd, con
   a.wait_ns = g->lim.wait_ns;
   a.miss_site = g->lim.miss_site;
   a.n_items = (u32)ni;
-  a.chunk = (u32)((ni + G - 1) / G);
-  return G;
+  a.chunk = (u32)((nh + Gh - 1) / Gh);
+  // a handle with a block share gives each block an SM of its own
+  const size_t least = g->loop_blocks_user > 0 ? kExclusiveSmem : 0;
+  if (wide) return {k_batch_sort<10>, std::max(kBSmem<10>, least), G};
+  return {k_batch_sort<9>, std::max(kBSmem<9>, least), G};
 }
 
 }  // namespace
 
-const void *batch_sort_fn() { return (const void *)k_batch_sort; }
+bool is_batch_sort(const void *fn) {
+  return fn == (const void *)k_batch_sort<9> || fn == (const void *)k_batch_sort<10>;
+}
 
 cudaError_t launch_batch_sort(sp_graph *g, const int *ds, const int *dd, long long nd,
                               const int *as, const int *ad, const int *aw, long long na,
                               int *launches) {
   if (nd + na == 0) return cudaSuccess;
   BatchSortArgs a;
-  const int G = batch_sort_args(g, ds, dd, nd, as, ad, aw, na, a);
+  const SortLaunch l = batch_sort_args(g, ds, dd, nd, as, ad, aw, na, a);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)G);
+  cfg.gridDim = dim3((unsigned)l.G);
   cfg.blockDim = dim3(kBT);
-  cfg.dynamicSmemBytes = sort_smem(g);
+  cfg.dynamicSmemBytes = l.smem;
   cfg.stream = g->stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;   // all blocks co-resident
@@ -682,20 +747,20 @@ cudaError_t launch_batch_sort(sp_graph *g, const int *ds, const int *dd, long lo
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   ++*launches;
-  return cudaLaunchKernelEx(&cfg, k_batch_sort, a);
+  return cudaLaunchKernelEx(&cfg, l.fn, a);
 }
 
 cudaError_t retarget_batch_sort(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t node,
                                 const int *ds, const int *dd, long long nd, const int *as,
                                 const int *ad, const int *aw, long long na) {
   BatchSortArgs a;
-  const int G = batch_sort_args(g, ds, dd, nd, as, ad, aw, na, a);
+  const SortLaunch l = batch_sort_args(g, ds, dd, nd, as, ad, aw, na, a);
   void *args[1] = {&a};
   cudaKernelNodeParams p = {};
-  p.func = (void *)k_batch_sort;
-  p.gridDim = dim3((unsigned)G);
+  p.func = (void *)l.fn;
+  p.gridDim = dim3((unsigned)l.G);
   p.blockDim = dim3(kBT);
-  p.sharedMemBytes = (unsigned)sort_smem(g);
+  p.sharedMemBytes = (unsigned)l.smem;
   p.kernelParams = args;
   return cudaGraphExecKernelNodeSetParams(ex, node, &p);
 }

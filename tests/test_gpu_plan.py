@@ -135,3 +135,35 @@ def test_small_host_arrays(n, pinned):
         d, p = g.get_dist(parent=True)
         np.testing.assert_array_equal(d, ref.dijkstra(0))
         check_sssp(n, *ref.csr(), 0, d, p)
+
+
+@pytest.mark.parametrize("n,m", [(600, 5000), (5000, 40000), (300000, 500000)])
+@pytest.mark.parametrize("blocks", [0, 1, 3])
+def test_grid_sorted_batches(n, m, blocks):
+    """Batches just above what one block plans and around whole tiles of the
+    grid's sort, either store in half of its blocks (or both in one block),
+    with the ids that take digits of ten bits and of nine."""
+    ro, col, w = wl.er_digraph(n, m, 1, 100, seed=n)
+    ref = oracle.OracleGraph(n, ro, col, w)
+    rng = np.random.default_rng(n + blocks)
+    with sp.Graph(n, ro, col, w, slack=0.05) as g:
+        if blocks:
+            g.set_loop_blocks(blocks)
+        g.sssp_init(0)
+        for k in (1025, 2048, 2049, 4096, 4097, 8193, 20001):
+            ro, col, _ = ref.csr()
+            b = messy(rng, n, wl.csr_keys(n, ro, col), k)
+            want = ref.apply(b)
+            got = g.apply(b, stats=True)
+            assert (got.n_del_applied, got.n_del_absent, got.n_add_applied,
+                    got.n_add_present) == want
+            for x, y in zip(g.export_csr(), ref.csr()):
+                np.testing.assert_array_equal(x, y)
+        np.testing.assert_array_equal(g.get_dist(), ref.dijkstra(0))
+        ro, col, w = ref.csr()
+        u = np.repeat(np.arange(n), np.diff(ro))
+        order = np.lexsort((u, col))
+        rro, rcol, rw = g.export_csr(reverse=True)
+        np.testing.assert_array_equal(np.diff(rro), np.bincount(col, minlength=n))
+        np.testing.assert_array_equal(rcol, u[order])
+        np.testing.assert_array_equal(rw, w[order])
