@@ -695,6 +695,9 @@ __global__ void __launch_bounds__(kCT, 3) k_count(CountArgs a) {
 // batch: the old-row searches, beside the batch sort
 // --------------------------------------------------------------------------
 
+// Searches per thread in lockstep at most: interpolating and halving ones.
+constexpr int kGuessWidth = 4, kHalveWidth = 6;
+
 struct SearchArgs {
   const int *ds, *dd, *as, *ad, *aw;
   long long nd, na;
@@ -702,6 +705,7 @@ struct SearchArgs {
   u64 *srch;
   int n;
   u32 n_items;
+  u32 per;   // searches that a thread advances together (k_search)
 };
 
 // Item i of the batch in the batch sort's own numbering (update j < nd is
@@ -710,13 +714,20 @@ struct SearchArgs {
 // pass needs it (position = old entries with a smaller col, and whether the
 // edge is there), and its weight, into srch[i].  The stores do not change
 // before the merge, so this runs beside the sort; ids out of range (the sort
-// rejects the batch) get 0.  Each thread advances kCI searches in lockstep.
-// kGuess: interpolating searches (row_search) in place of halving ones.
+// rejects the batch) get 0.  Each thread advances searches in lockstep: halving
+// ones as many (a.per) as spread the items evenly over whole rounds of the grid,
+// since a round is one chain of dependent reads whatever its width (against
+// always four, a batch and its undo: 32 graphs together, 660,000 items in three
+// rounds instead of five, 1,053 -> 1,029 us; R-MAT 20, two rounds of five, within
+// 1% either way in two runs).  kGuess: interpolating ones (row_search), always four: they are
+// bound by their reads from DRAM (evened out: 2,335 -> 2,351 us on R-MAT 22).
+// (80 registers a thread at most: the sort's block has its place on the SM.)
 template <bool kGuess>
-__global__ void __launch_bounds__(kCT, kGuess ? 3 : 4) k_search(SearchArgs a) {
+__global__ void __launch_bounds__(kCT, 3) k_search(SearchArgs a) {
+  constexpr int kCI = kGuess ? kGuessWidth : kHalveWidth;
   const long long nb = a.nd + a.na;
-  const u32 ni = a.n_items;
-  for (u32 tb = blockIdx.x * (u32)kCTile; tb < ni; tb += gridDim.x * (u32)kCTile) {
+  const u32 ni = a.n_items, per = kGuess ? (u32)kCI : a.per, tile = per * (u32)kCT;
+  for (u32 tb = blockIdx.x * tile; tb < ni; tb += gridDim.x * tile) {
     int col[kCI], deg[kCI];
     u32 w[kCI];
     const int2 *old[kCI];
@@ -724,7 +735,7 @@ __global__ void __launch_bounds__(kCT, kGuess ? 3 : 4) k_search(SearchArgs a) {
 #pragma unroll
     for (int k = 0; k < kCI; ++k) {   // every input load first
       const u32 i = tb + (u32)(k * kCT) + threadIdx.x;
-      val[k] = i < ni;
+      val[k] = (u32)k < per && i < ni;
       int u = 0, v = 0;
       w[k] = 0;
       const bool rev = (long long)i >= nb;
@@ -791,19 +802,6 @@ __global__ void __launch_bounds__(kCT, kGuess ? 3 : 4) k_search(SearchArgs a) {
   }
 }
 
-SearchArgs search_args(sp_graph *g, const int *ds, const int *dd, long long nd, const int *as,
-                       const int *ad, const int *aw, long long na) {
-  SearchArgs a;
-  a.ds = ds; a.dd = dd; a.as = as; a.ad = ad; a.aw = aw;
-  a.nd = nd; a.na = na;
-  a.st[0] = g->fwd;
-  a.st[1] = g->rev;
-  a.srch = g->bb.srch;
-  a.n = g->n;
-  a.n_items = (u32)(2 * (nd + na));
-  return a;
-}
-
 // The searches interpolate where the store is well beyond the L2: there they
 // are bound by random reads from DRAM (twice the threads made them slower),
 // and three rounds of reads take the place of ten.  A million updates on
@@ -815,12 +813,29 @@ bool search_guesses(const sp_graph *g) {
   return std::max(g->fwd.slots, g->rev.slots) * (long long)sizeof(int2) >= (1LL << 30);
 }
 
+SearchArgs search_args(sp_graph *g, const int *ds, const int *dd, long long nd, const int *as,
+                       const int *ad, const int *aw, long long na) {
+  SearchArgs a;
+  a.ds = ds; a.dd = dd; a.as = as; a.ad = ad; a.aw = aw;
+  a.nd = nd; a.na = na;
+  a.st[0] = g->fwd;
+  a.st[1] = g->rev;
+  a.srch = g->bb.srch;
+  a.n = g->n;
+  a.n_items = (u32)(2 * (nd + na));
+  const long long wave = (long long)std::max(1, g->num_sms) * kCT;
+  const long long each = (a.n_items + wave - 1) / wave;
+  const long long rounds = std::max(1ll, (each + kHalveWidth - 1) / kHalveWidth);
+  a.per = (u32)(search_guesses(g) ? kGuessWidth : std::max(1ll, (each + rounds - 1) / rounds));
+  return a;
+}
+
 // One block of 256 threads per SM at most: beside it an SM still holds a
 // block of the batch sort (512 threads, 90-116 KB of shared memory, 45,056
-// registers; the search's 256 threads take 14,336 or 20,480), so the search
+// registers; the search's 256 threads take 20,480 at most), so the search
 // never delays the sort's cooperative grid.
-unsigned search_grid(const sp_graph *g, long long ni) {
-  return blocks_for(ni, kCTile, std::max(1, g->num_sms));
+unsigned search_grid(const sp_graph *g, const SearchArgs &a) {
+  return blocks_for(a.n_items, (long long)a.per * kCT, std::max(1, g->num_sms));
 }
 
 // --------------------------------------------------------------------------
@@ -1866,8 +1881,8 @@ cudaError_t launch_search(sp_graph *g, const int *ds, const int *dd, long long n
   const long long ni = 2 * (nd + na);
   if (ni == 0) return cudaSuccess;
   const SearchArgs a = search_args(g, ds, dd, nd, as, ad, aw, na);
-  if (search_guesses(g)) k_search<true><<<search_grid(g, ni), kCT, 0, stream>>>(a);
-  else k_search<false><<<search_grid(g, ni), kCT, 0, stream>>>(a);
+  if (search_guesses(g)) k_search<true><<<search_grid(g, a), kCT, 0, stream>>>(a);
+  else k_search<false><<<search_grid(g, a), kCT, 0, stream>>>(a);
   ++*launches;
   return cudaGetLastError();
 }
@@ -1883,7 +1898,7 @@ cudaError_t retarget_search(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t nod
   void *args[1] = {&a};
   cudaKernelNodeParams p = {};
   p.func = const_cast<void *>(search_fn(g));
-  p.gridDim = dim3(search_grid(g, 2 * (nd + na)));
+  p.gridDim = dim3(search_grid(g, a));
   p.blockDim = dim3(kCT);
   p.sharedMemBytes = 0;
   p.kernelParams = args;
