@@ -186,7 +186,9 @@ sp_status sp_sssp_init(sp_graph *g, int32_t source, sp_batch_stats *stats);
  * buffers first: page-locked arrays that are mapped into the device's
  * address space (cudaHostAlloc, pinned tensors) by one kernel that reads
  * them across the host link, any other host array by the copy engine.  The
- * call is synchronous, so the arrays may be reused once it returns.
+ * call is synchronous, so the arrays may be reused once it returns.  A batch of
+ * at most 1,024 updates in host memory is not staged: its kernels read it in
+ * place, pageable arrays through a page-locked block of the handle.
  */
 sp_status sp_apply_batch(sp_graph *g,
                          int64_t n_del, const int32_t *del_src, const int32_t *del_dst,
@@ -221,7 +223,8 @@ sp_status sp_apply_batch_get(sp_graph *g,
  * program).  out_on_device: dist/parent are device arrays of the graph's
  * device, else SP_EINVAL before anything runs (out_on_device = 0: host
  * memory; page-locked, mapped host arrays are written in place by the
- * kernel, others through a device buffer and a copy).  The call is
+ * kernel, others through a device buffer and a copy, or, up to 16,384
+ * vertices, through a page-locked block of the handle).  The call is
  * synchronous.  SP_ESTATE if no valid distances exist.
  */
 sp_status sp_get_dist(sp_graph *g, int32_t *dist, int32_t *parent,
@@ -594,7 +597,7 @@ sp_status sp_tc_apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
                             int inputs_on_device, int64_t *count, sp_batch_stats *stats);
 
 /*
- * sp_apply_batch runs its kernels (eight per batch) as a cached CUDA graph
+ * sp_apply_batch runs its kernels (seven per batch) as a cached CUDA graph
  * when a batch has the same shape (deletion and insertion counts, stats or
  * not) as the one before it: one graph launch replaces the kernel launches.
  * Device inputs are read where they are (the three kernels that read them
