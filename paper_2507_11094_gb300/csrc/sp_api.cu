@@ -320,23 +320,9 @@ cudaError_t enqueue_batch(sp_graph *g, const int *ds, const int *dd, long long n
   const int reset = mode == kInvalKept ? 2 : 0;
   if (small) sp::launch_check_small(g, ds, dd, n_del, as, ad, aw, n_add, reset, launches);
   else sp::launch_ctl_reset(g, reset, launches);
-  // the items' searches in their old rows run beside the batch sort (on the
-  // SMs the sort leaves free; they read only the inputs and the old stores)
   cudaError_t e = cudaSuccess;
-  if (small) {
-    // (its plan does them, below, beside the invalidation)
-  } else if (g->side) {
-    cudaEventRecord(g->fork0_ev, g->stream);
-    cudaStreamWaitEvent(g->side, g->fork0_ev, 0);
-    e = sp::launch_search(g, ds, dd, n_del, as, ad, aw, n_add, launches, g->side);
-    cudaEventRecord(g->search_ev, g->side);
-  } else {
-    e = sp::launch_search(g, ds, dd, n_del, as, ad, aw, n_add, launches, g->stream);
-  }
-  if (!small) {
-    const cudaError_t es = sp::launch_batch_sort(g, ds, dd, n_del, as, ad, aw, n_add, launches);
-    if (e == cudaSuccess) e = es;
-  }
+  // (a small batch's plan does its searches and sort, below, beside the invalidation)
+  if (!small) e = sp::launch_search_sort(g, ds, dd, n_del, as, ad, aw, n_add, launches);
   rec(g, timed, 1);
   if (!small && g->side) cudaStreamWaitEvent(g->stream, g->search_ev, 0);
   const bool beside = mode == kInvalBeside && n_del > 0;

@@ -301,6 +301,11 @@ const void *check_small_fn();
 cudaError_t retarget_plan(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t check,
                           cudaGraphNode_t plan, const int *ds, const int *dd, long long nd,
                           const int *as, const int *ad, const int *aw, long long na);
+// The searches beside the batch sort; the graph's stream has to wait for
+// search_ev (with a side stream) before their results are read.
+cudaError_t launch_search_sort(sp_graph *g, const int *ds, const int *dd, long long nd,
+                               const int *as, const int *ad, const int *aw, long long na,
+                               int *launches);
 // Everything before a batch's merge on the graph's stream, by either way
 // (after a control reset).
 cudaError_t launch_store_plan(sp_graph *g, const int *ds, const int *dd, long long nd,

@@ -167,3 +167,36 @@ def test_grid_sorted_batches(n, m, blocks):
         np.testing.assert_array_equal(np.diff(rro), np.bincount(col, minlength=n))
         np.testing.assert_array_equal(rcol, u[order])
         np.testing.assert_array_equal(rw, w[order])
+
+
+# above one block's batches the old-row searches run beside the sort, on the
+# handle's side stream (none on the legacy stream); only then are they read
+@pytest.mark.parametrize("own_stream", [False, True])
+def test_searches_beside_the_sort_of_triangle_and_rank_batches(own_stream):
+    import torch
+    st = torch.cuda.Stream() if own_stream else None
+    W = wl.sym_er(4096, 40000, 700, 3)       # 2,800 updates a batch
+    ref = oracle.OracleGraph(W.n, W.row_off, W.col, W.w)
+    with sp.Graph(W.n, W.row_off, W.col, W.w, stream=st) as g:
+        assert g.tc_init() == ref.triangles()
+        for k in range(4):
+            b = W.batch(k)
+            cnt = ref.apply(b)
+            c, s = g.tc_apply(b, stats=True)
+            assert (s.n_del_applied, s.n_del_absent, s.n_add_applied, s.n_add_present) == cnt
+            assert c == ref.triangles()
+    W = wl.rmat(13, batch_frac=0.04, seed=3)   # two phases of 2,600 updates
+    ref = oracle.OracleGraph(W.n, W.row_off, W.col, W.w)
+    want, _ = ref.pagerank(0.85, 1e-6, 100)
+    with sp.Graph(W.n, W.row_off, W.col, W.w, stream=st) as g:
+        g.pr_init(0.85, 1e-6, 100)
+        for k in range(4):
+            b = W.batch(k)
+            assert min(b.del_src.size, b.add_src.size) > 1024
+            cnt = ref.pagerank_batch(b, want, 0.85, 1e-6, 100)
+            s = g.pr_apply(b, stats=True)
+            assert (s.n_del_applied, s.n_del_absent, s.n_add_applied, s.n_add_present) == cnt[:4]
+            # (the bounds of the ranks' own parity tests)
+            np.testing.assert_allclose(g.pr_get(), want, rtol=2e-5, atol=1e-9)
+            for x, y in zip(g.export_csr(), ref.csr()):
+                np.testing.assert_array_equal(x, y)
