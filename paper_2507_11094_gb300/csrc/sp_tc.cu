@@ -65,7 +65,7 @@ __device__ __forceinline__ int owner_lane(u32 incl, u32 t) {
 // same pass every row is compared with the same row of the reverse store:
 // equal rows everywhere mean that every edge has its reverse, which is the
 // symmetry check without a search per edge.  R-MAT 18, edge factor 8: check and
-// count 0.69 ms; a warp per vertex v walking its lower neighbours one by one,
+// count 0.54 ms; a warp per vertex v walking its lower neighbours one by one,
 // behind a binary search per edge, took 29.3 ms (1.14 ms of it the check):
 // the hubs' rows were serial.
 constexpr int kOrientRow = 256;      // longer rows are taken by a whole block
