@@ -17,8 +17,8 @@
 //     one list after the other, padded to whole 16-byte loads with a place
 //     that holds zero: half the bytes of the (col, w) pairs without the
 //     store's slack, so that most of them stay in L2 from step to step (left
-//     in the rows' alternate regions, which is where they go when no memory
-//     can be had for them, R-MAT 20's 67 MB cost 149 MB of HBM reads a step);
+//     in the rows' alternate regions, which is where they go when there is no
+//     room for them, R-MAT 20's 67 MB cost 149 MB of HBM reads a step);
 //   * the vertices are listed by in-degree class, with everything a step
 //     needs of one in arrays over its position in that list; a term's place,
 //     where it is not hot, follows its vertex's position.
@@ -76,8 +76,8 @@ struct PrArgs {
   Limits lim;
   Store fwd, rev;
   PrScratch *sc;
-  u32 *lists;            // the in-neighbour lists: packed, or (null) in the
-                         // alternate regions of the reverse store
+  u32 *lists;            // room for the packed in-neighbour lists, or null
+  u64 list_words;        // ... in 16-byte words
   float *pr;             // ranks by vertex
   float *term[2];        // pr / outdeg by place (kHot, the zero place, then by vertex)
   u32 *place;            // a vertex's place
@@ -245,7 +245,6 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
   if (!repair_enabled_block(c)) return;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const u32 n = (u32)a.n, G = gridDim.x;
-  u32 *lists = a.lists ? a.lists : (u32 *)a.rev.adj;
   const u32 chunk = (n + G - 1) / G;
   const u32 cb = min(blockIdx.x * chunk, n), ce = min(cb + chunk, n);
   u64 *bar = &c->bar_push;
@@ -293,6 +292,7 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
   // term, and the selected vertices by position
   u32 first[kClasses], cnt[kClasses];
   const u32 nsegs = __ldcg(&a.sc->segs);
+  bool packed;
   {
     u64 at = 0;
 #pragma unroll
@@ -303,6 +303,10 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
       if (t == k) s_cls[k] += at;
       at += x;
     }
+    // packed, if the rows as they are now fit: the room follows the host's edge
+    // count, which an asynchronous batch that nobody finished leaves behind (the
+    // same answer in every block: the counts are final since the barrier)
+    packed = a.lists && (u64)(u32)at <= a.list_words;
     if (t == 0) {
       s_T = kPrBins;
       s_hot = 0;
@@ -321,6 +325,7 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
     if (t == 0) s_hot = total ? atomicAdd(&a.sc->hot, total) : 0u;
     __syncthreads();
   }
+  u32 *lists = packed ? a.lists : (u32 *)a.rev.adj;
   const u32 T = s_T, nhot = s_nhot;
   for (u32 b = cb + (t & ~31); b < ce && !stop; b += kPrThreads) {
     const u32 v = b + lane;
@@ -361,7 +366,7 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
       a.term[1][p] = f;
     }
     if (sel) {
-      a.list[pos] = a.lists ? 4ull * wpos : 2ull * (u64)a.rev.alt[v];
+      a.list[pos] = packed ? 4ull * wpos : 2ull * (u64)a.rev.alt[v];
       a.lenp[pos] = make_int2(in.deg, (int)p);
       a.degv[pos] = make_int2(od, (int)v);
       a.rank[pos] = r;
@@ -386,7 +391,7 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
     const int k = kClsWarp + t % 3;
     const u32 b = blockIdx.x + t / 3;
     u32 r = (u32)((u64)cnt[k] * b / G);
-    if (a.lists && b > 0 && b < G && cnt[k] > 0) {
+    if (packed && b > 0 && b < G && cnt[k] > 0) {
       const u64 w0 = __ldcg(a.list + first[k]);
       const u64 want = w0 + 4 * ((u64)(u32)ld_cg_u64(&a.sc->cls[k]) * b / G);
       u32 lo = 0, hi = cnt[k];
@@ -682,6 +687,7 @@ cudaError_t launch_pr(sp_graph *g, int all, float init, int *launches) {
   pr_lists(g);
   PrArgs p;
   p.lists = g->prlist;
+  p.list_words = g->prlist_bytes / 16;
   p.ctl = g->ctl;
   p.lim = g->lim;
   p.fwd = g->fwd;

@@ -1,0 +1,64 @@
+"""GPU tests of calls on a handle whose edge count on the host lags behind the
+stores (an asynchronous batch that nobody has finished, a phase that ran into
+a bound): results follow the stores' rows, whatever the host believes."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2507_11094_gb300 import sp
+from paper_2507_11094_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    from paper_2507_11094_gb300 import build
+    build.build()
+    oracle.build()
+    sp.load()
+
+
+def insertions(n, keys, w):
+    i32 = lambda x: np.ascontiguousarray(x, np.int32)
+    z = np.zeros(0, np.int32)
+    return wl.Batch(z, z, i32(keys // n), i32(keys % n), i32(w))
+
+
+def launch_unfinished(g, b):
+    """Apply b asynchronously; the host is never told the outcome."""
+    import torch
+    x = g.capture(*[torch.from_numpy(a).cuda() for a in
+                    (b.del_src, b.del_dst, b.add_src, b.add_dst, b.add_w)])
+    x.launch()
+    g.sync()
+    return x
+
+
+# new edges whose in-neighbour lists take several times the room that the
+# host's count asks for, and just more than it
+@pytest.mark.parametrize("n,m,k", [(120, 1000, 6000), (1000, 4000, 12000), (100, 5000, 2500),
+                                   (3000, 20000, 9000)])
+def test_ranks_of_a_graph_with_more_edges_than_the_host_knows(n, m, k):
+    import torch
+    ro, col, w = wl.er_digraph(n, m, 1, 100, seed=n)
+    ref = oracle.OracleGraph(n, ro, col, w)
+    rng = np.random.default_rng(m)
+    free = np.setdiff1d(np.arange(n * n), wl.csr_keys(n, ro, col))
+    b = insertions(n, rng.choice(free, size=k, replace=False), rng.integers(1, 101, k))
+    with sp.Graph(n, ro, col, w, stream=torch.cuda.Stream()) as g:
+        g.sssp_init(0)
+        g.reserve(k)
+        x = launch_unfinished(g, b)
+        ref.apply(b)
+        np.testing.assert_array_equal(g.get_dist(), ref.dijkstra(0))   # it applied
+        assert g.m == m
+        st = g.pr_init(0.85, 1e-6, 100, stats=True)
+        want, it = ref.pagerank(0.85, 1e-6, 100)
+        # (the bounds of the ranks' own parity tests)
+        np.testing.assert_allclose(g.pr_get(), want, rtol=2e-5, atol=1e-9)
+        assert abs(st.rounds_push - it) <= 1
+        assert st.relaxed_edges == (m + k) * st.rounds_push
+        x.close()
