@@ -615,15 +615,14 @@ void launch_tc_static(sp_graph *g, int *launches) {
   k_tc_orient<<<grid_for(g->n, a.rpw * (kThreads / 32), g->num_sms * 16), kThreads, 0, g->stream>>>(
       a);
   ++*launches;
-  if (g->m > kOrientGiant) {   // such a row can be there
-    k_tc_orient_giant<<<(unsigned)g->num_sms * 4, kThreads, 0, g->stream>>>(a);
-    ++*launches;
-  }
+  // (whether there is such a row is known on the device only: the host's edge
+  // count may lag behind the stores)
+  k_tc_orient_giant<<<(unsigned)g->num_sms * 4, kThreads, 0, g->stream>>>(a);
   k_tc_lists<<<grid_for(g->n, kThreads, g->num_sms * 8), kThreads, 0, g->stream>>>(a.cnt, g->n,
                                                                                    g->cut, g->ctl);
   k_tc_count<<<(unsigned)g->num_sms * 6, kThreads, 0, g->stream>>>(g->fwd, g->n, a.cnt, g->cut,
                                                                    g->ctl);
-  *launches += 2;
+  *launches += 3;
 }
 
 void launch_tc_batch_sym(sp_graph *g, long long nb, int *launches) {

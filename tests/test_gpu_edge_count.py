@@ -62,3 +62,28 @@ def test_ranks_of_a_graph_with_more_edges_than_the_host_knows(n, m, k):
         assert abs(st.rounds_push - it) <= 1
         assert st.relaxed_edges == (m + k) * st.rounds_push
         x.close()
+
+
+def test_triangles_of_hubs_that_the_host_does_not_know():
+    # an empty graph becomes three hubs, joined to each other and to every vertex
+    # of a rim: rows that the whole grid orients (more than 65,536 entries), and
+    # the hubs' own triangle is counted from such a row.  Nobody finishes the batch
+    import torch
+    k = 66000
+    hubs = np.array([7, 30000, 66002], np.int64)
+    rim = np.setdiff1d(np.arange(k + 3), hubs)
+    n = 200000                       # (with room in the spare pool for the hubs' rows)
+    u = np.concatenate([np.repeat(hubs, k), [7, 7, 30000]])
+    v = np.concatenate([np.tile(rim, 3), [30000, 66002, 66002]])
+    u, v = np.concatenate([u, v]), np.concatenate([v, u])
+    b = insertions(n, u * n + v, np.ones(u.size, np.int64))
+    z = np.zeros(0, np.int32)
+    with sp.Graph(n, np.zeros(n + 1, np.int64), z, z, slack=0.0,
+                  stream=torch.cuda.Stream()) as g:
+        g.sssp_init(0)
+        g.reserve(u.size)
+        x = launch_unfinished(g, b)
+        assert g.m == 0
+        assert g.get_dist()[:k + 3].max() == 2   # it applied: all are two steps apart at most
+        assert g.tc_init() == 3 * k + 1
+        x.close()
