@@ -1239,8 +1239,8 @@ sp_status pr_phase(sp_graph *g, const int *ds, const int *dd, long long nd, cons
     const Ctl &c = *g->ctl_host;
     if (c.status != 0) return (sp_status)c.status;
     if (c.bad) return SP_ECUDA;
-    if (c.timeout) return SP_ETIMEOUT;
     if (c.need_grow == 0) break;
+    if (c.timeout) return SP_ETIMEOUT;   // nothing changed
     if (attempt >= 6) return SP_ENOMEM;
     ++*regrows;
     if (c.need_grow & sp::kGrowPoolFwd) {
@@ -1254,7 +1254,7 @@ sp_status pr_phase(sp_graph *g, const int *ds, const int *dd, long long nd, cons
     rc = sp::ensure_owner_tables(g);
     if (rc != SP_OK) return rc;
   }
-  {
+  {   // the edges are merged, also where a bound was hit in the flag propagation
     const Ctl &c = *g->ctl_host;
     g->m += (long long)c.add_applied - (long long)c.del_applied;
     acc.del_applied += c.del_applied;
@@ -1267,6 +1267,7 @@ sp_status pr_phase(sp_graph *g, const int *ds, const int *dd, long long nd, cons
     acc.inval_edges += c.inval_edges;
     acc.merge_slots += c.merge_slots;
     acc.rounds_inval += c.rounds_inval;
+    if (c.timeout) return SP_ETIMEOUT;
   }
   if (n_flag == 0) return SP_OK;   // nothing flagged: every rank stays
   cudaError_t e = sp::launch_pr(g, 0, 0.0f, launches);

@@ -87,3 +87,54 @@ def test_triangles_of_hubs_that_the_host_does_not_know():
         assert g.get_dist()[:k + 3].max() == 2   # it applied: all are two steps apart at most
         assert g.tc_init() == 3 * k + 1
         x.close()
+
+
+# a rank batch of which a phase's flags run into a round cap: the phase's edges
+# are merged, so the edge count follows, what held on the old edges no longer
+# does, and the ranks can be computed again (also through one block's plan)
+@pytest.mark.parametrize("nd,na", [(0, 2500), (0, 700), (1500, 0), (600, 2500)])
+def test_a_rank_batch_that_hits_a_bound_leaves_the_edge_count_right(nd, na):
+    n, m = 100, 5000
+    ro, col, w = wl.er_digraph(n, m, 1, 100, seed=7)
+    keys = wl.csr_keys(n, ro, col)
+    rng = np.random.default_rng(nd + na)
+    gone = rng.choice(keys, size=nd, replace=False)
+    new = rng.choice(np.setdiff1d(np.arange(n * n), keys), size=na, replace=False)
+    i32 = lambda x: np.ascontiguousarray(x, np.int32)
+    b = wl.Batch(i32(gone // n), i32(gone % n), i32(new // n), i32(new % n),
+                 i32(rng.integers(1, 101, na)))
+    # the first phase that has updates hits the bound, and the call ends there
+    z = np.zeros(0, np.int32)
+    done = b if not nd else wl.Batch(b.del_src, b.del_dst, z, z, z)
+    ref = oracle.OracleGraph(n, ro, col, w)
+    with sp.Graph(n, ro, col, w) as g:
+        g.sssp_init(0)
+        g.pr_init(0.85, 1e-6, 100)
+        g.set_limits(1)
+        with pytest.raises(sp.SpError) as e:
+            g.pr_apply(b)
+        assert e.value.code == sp.SP_ETIMEOUT
+        g.set_limits(0)
+        ref.apply(done)
+        assert g.m == m - done.del_src.size + done.add_src.size
+        for call in (g.get_dist, g.pr_get):
+            with pytest.raises(sp.SpError) as e:
+                call()
+            assert e.value.code == sp.SP_ESTATE
+        for rev in (False, True):
+            got = g.export_csr(reverse=rev)
+            rro, rcol, rw = ref.csr()
+            u = np.repeat(np.arange(n), np.diff(rro))
+            if rev:
+                order = np.lexsort((u, rcol))
+                want = (np.concatenate([[0], np.cumsum(np.bincount(rcol, minlength=n))]),
+                        u[order], rw[order])
+            else:
+                want = (rro, rcol, rw)
+            for x, y in zip(got, want):
+                np.testing.assert_array_equal(x, y)
+        g.pr_init(0.85, 1e-6, 100)
+        np.testing.assert_allclose(g.pr_get(), ref.pagerank(0.85, 1e-6, 100)[0], rtol=2e-5,
+                                   atol=1e-9)
+        g.sssp_init(0)
+        np.testing.assert_array_equal(g.get_dist(), ref.dijkstra(0))
