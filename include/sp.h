@@ -186,9 +186,12 @@ sp_status sp_sssp_init(sp_graph *g, int32_t source, sp_batch_stats *stats);
  * buffers first: page-locked arrays that are mapped into the device's
  * address space (cudaHostAlloc, pinned tensors) by one kernel that reads
  * them across the host link, any other host array by the copy engine.  The
- * call is synchronous, so the arrays may be reused once it returns.  A batch of
- * at most 1,024 updates in host memory is not staged: its kernels read it in
- * place, pageable arrays through a page-locked block of the handle.
+ * call is synchronous, so the arrays may be reused once it returns.  Arrays of
+ * registered, managed or page-locked memory are read in stream order (work
+ * queued on the graph's stream may still be filling them).  A batch of at most
+ * 1,024 updates is not staged if its arrays are all page-locked and mapped (its
+ * kernels read them in place) or all ordinary host memory and the graph's stream
+ * is idle (they are copied into a page-locked block of the handle).
  */
 sp_status sp_apply_batch(sp_graph *g,
                          int64_t n_del, const int32_t *del_src, const int32_t *del_dst,

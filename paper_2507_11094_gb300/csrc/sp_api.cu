@@ -414,6 +414,24 @@ const void *mapped_host(const void *p) {
   return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
 }
 
+// Ordinary host memory that CUDA does not know of: only the host writes it, so
+// the host may read it as soon as the graph's stream is idle.  Registered, managed
+// or device memory may still be written by work that the caller has queued there.
+bool unregistered_host(const void *p) {
+  cudaPointerAttributes at;
+  if (!p || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeUnregistered;
+}
+
+bool stream_idle(const sp_graph *g) {
+  const bool idle = cudaStreamQuery(g->stream) == cudaSuccess;
+  if (!idle) cudaGetLastError();
+  return idle;
+}
+
 // A device array the graph's kernels may write: memory of the graph's device
 // (or managed memory).  Host pointers passed as device outputs are refused
 // before anything is launched.
@@ -872,10 +890,6 @@ sp_status apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
   if (g->state != 1) return SP_ESTATE;
   const long long nb = n_del + n_add, ni = 2 * nb;
   const bool timed = stats != nullptr;
-  // a small batch in host memory is read in place by the few kernels that need
-  // it (pageable arrays from the handle's page-locked block, into which they
-  // are copied here), with no staging kernel or copy in front
-  const bool in_place = !inputs_on_device && nb > 0 && sp::plan_small(g, ni);
   // the same batch shape twice in a row: the pipeline runs as a cached CUDA
   // graph (one launch instead of seven), its input-reading nodes pointed at
   // this call's arrays
@@ -903,6 +917,19 @@ sp_status apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
       m[4] = mapped_host(add_w);
       mapped = m[2] && m[3] && m[4];
     }
+  }
+  // a small batch in page-locked or in ordinary host memory is read in place by
+  // the few kernels that need it, with no staging kernel or copy in front.
+  // Ordinary arrays go through the handle's page-locked block, into which they
+  // are copied here: not in stream order, so only if nothing is queued on the
+  // graph's stream, and not where one of the arrays is memory that queued work
+  // may write (a mix with page-locked or managed arrays takes the staged copies)
+  bool in_place = !inputs_on_device && nb > 0 && sp::plan_small(g, ni);
+  if (in_place && !mapped) {
+    const void *in[5] = {del_src, del_dst, add_src, add_dst, add_w};
+    for (int q = 0; q < 5; ++q)
+      if ((q < 2 ? n_del : n_add) > 0) in_place = in_place && unregistered_host(in[q]);
+    in_place = in_place && stream_idle(g);
   }
   sp_status rc =
       ensure_batch_buffers(g, ni, inputs_on_device || in_place ? 0 : std::max(n_del, n_add));
