@@ -189,9 +189,10 @@ sp_status sp_sssp_init(sp_graph *g, int32_t source, sp_batch_stats *stats);
  * call is synchronous, so the arrays may be reused once it returns.  Arrays of
  * registered, managed or page-locked memory are read in stream order (work
  * queued on the graph's stream may still be filling them).  A batch of at most
- * 1,024 updates is not staged if its arrays are all page-locked and mapped (its
- * kernels read them in place) or all ordinary host memory and the graph's stream
- * is idle (they are copied into a page-locked block of the handle).
+ * 1,024 updates needs no staging copy if its arrays are all page-locked and
+ * mapped (its first kernel reads them) or all ordinary host memory and the
+ * graph's stream is idle (they are copied into a page-locked block of the
+ * handle).  Either way every host array is read once.
  */
 sp_status sp_apply_batch(sp_graph *g,
                          int64_t n_del, const int32_t *del_src, const int32_t *del_dst,

@@ -237,13 +237,28 @@ bool find_input_nodes(sp_graph *g) {
          (g->bg_sort != nullptr && g->bg_search != nullptr);
 }
 
+// host: the arrays that a small batch's check reads (null: ds .. aw, as the
+// other nodes).  Nodes that read what the graph has them read already, as the
+// staging buffers call after call, are left alone.
 cudaError_t retarget_input_nodes(sp_graph *g, const int *ds, const int *dd, long long nd,
-                                 const int *as, const int *ad, const int *aw, long long na) {
-  cudaError_t e =
-      g->bg_plan ? sp::retarget_plan(g, g->bg_exec, g->bg_check, g->bg_plan, ds, dd, nd, as, ad,
-                                     aw, na)
-                 : sp::retarget_batch_sort(g, g->bg_exec, g->bg_sort, ds, dd, nd, as, ad, aw, na);
-  if (e == cudaSuccess && !g->bg_plan)
+                                 const int *as, const int *ad, const int *aw, long long na,
+                                 const int *const *host) {
+  const int *const dev[5] = {ds, dd, as, ad, aw};
+  const int *const *in = host ? host : dev;
+  cudaError_t e = cudaSuccess;
+  if (g->bg_check && (!std::equal(in, in + 5, g->bg_in) || g->bg_host != (host != nullptr))) {
+    e = sp::retarget_check_small(g, g->bg_exec, g->bg_check, in[0], in[1], nd, in[2], in[3], in[4],
+                                 na, host != nullptr);
+    std::copy(in, in + 5, g->bg_in);
+    g->bg_host = host != nullptr;
+  }
+  if (std::equal(dev, dev + 5, g->bg_dev)) return e;
+  std::copy(dev, dev + 5, g->bg_dev);
+  if (e == cudaSuccess && g->bg_plan)
+    e = sp::retarget_plan(g, g->bg_exec, g->bg_plan, ds, dd, nd, as, ad, aw, na);
+  if (e == cudaSuccess && g->bg_sort)
+    e = sp::retarget_batch_sort(g, g->bg_exec, g->bg_sort, ds, dd, nd, as, ad, aw, na);
+  if (e == cudaSuccess && g->bg_search)
     e = sp::retarget_search(g, g->bg_exec, g->bg_search, ds, dd, nd, as, ad, aw, na);
   if (e == cudaSuccess && g->bg_inval)
     e = sp::retarget_inval(g, g->bg_exec, g->bg_inval, ds, dd, nd, inval_beside(g) ? 1 : 0);
@@ -311,15 +326,24 @@ enum InvalMode {
   kInvalKept = 2,     // a rerun after a pool grow: the first attempt's stands
 };
 
-// The kernel sequence of one batch (no host synchronisation).
+// The kernel sequence of one batch (no host synchronisation).  host: the five
+// arrays of a small batch in host memory, which its check copies to ds .. aw (the
+// staging buffers).
 cudaError_t enqueue_batch(sp_graph *g, const int *ds, const int *dd, long long n_del,
                           const int *as, const int *ad, const int *aw, long long n_add,
-                          bool timed, int *launches, int mode = kInvalAfter) {
+                          bool timed, int *launches, int mode = kInvalAfter,
+                          const int *const *host = nullptr) {
   const long long ni = 2 * (n_del + n_add);
   const bool small = ni > 0 && sp::plan_small(g, ni);   // one block plans the store update
   const int reset = mode == kInvalKept ? 2 : 0;
-  if (small) sp::launch_check_small(g, ds, dd, n_del, as, ad, aw, n_add, reset, launches);
-  else sp::launch_ctl_reset(g, reset, launches);
+  if (small) {
+    const int *const dev[5] = {ds, dd, as, ad, aw};
+    const int *const *in = host ? host : dev;
+    sp::launch_check_small(g, in[0], in[1], n_del, in[2], in[3], in[4], n_add, host != nullptr,
+                           reset, launches);
+  } else {
+    sp::launch_ctl_reset(g, reset, launches);
+  }
   cudaError_t e = cudaSuccess;
   // (a small batch's plan does its searches and sort, below, beside the invalidation)
   if (!small) e = sp::launch_search_sort(g, ds, dd, n_del, as, ad, aw, n_add, launches);
@@ -405,25 +429,19 @@ sp_status restore_after(sp_graph *g, bool touched, sp_status rc) {
 // device's address space (cudaHostAlloc, torch's pinned memory), or nullptr
 // for any other pointer.  Kernels read and write such arrays directly across
 // the host link (NVLink-C2C on Grace machines), with no copy-engine transfer.
-const void *mapped_host(const void *p) {
+// *plain: ordinary host memory that CUDA does not know of.  Only the host writes
+// that, so the host may read it as soon as the graph's stream is idle; registered,
+// managed or device memory may still be written by work that the caller has
+// queued there.
+const void *mapped_host(const void *p, bool *plain = nullptr) {
+  if (plain) *plain = false;
   cudaPointerAttributes at;
   if (!p || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
+  if (plain) *plain = at.type == cudaMemoryTypeUnregistered;
   return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
-}
-
-// Ordinary host memory that CUDA does not know of: only the host writes it, so
-// the host may read it as soon as the graph's stream is idle.  Registered, managed
-// or device memory may still be written by work that the caller has queued there.
-bool unregistered_host(const void *p) {
-  cudaPointerAttributes at;
-  if (!p || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return at.type == cudaMemoryTypeUnregistered;
 }
 
 bool stream_idle(const sp_graph *g) {
@@ -902,71 +920,46 @@ sp_status apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
   // host arrays in page-locked, mapped memory are gathered into the staging
   // buffers by one kernel (16-byte loads across the host link); any other
   // host array is copied there by the copy engine
-  const void *m[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-  bool mapped = false;
-  if (!inputs_on_device) {
-    mapped = true;
-    if (n_del) {
-      m[0] = mapped_host(del_src);
-      m[1] = mapped_host(del_dst);
-      mapped = m[0] && m[1];
-    }
-    if (n_add && mapped) {
-      m[2] = mapped_host(add_src);
-      m[3] = mapped_host(add_dst);
-      m[4] = mapped_host(add_w);
-      mapped = m[2] && m[3] && m[4];
-    }
+  const int32_t *const src[5] = {del_src, del_dst, add_src, add_dst, add_w};
+  const long long cnt[5] = {n_del, n_del, n_add, n_add, n_add};
+  const int *m[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+  const bool small = nb > 0 && sp::plan_small(g, ni);
+  bool mapped = !inputs_on_device, plain = mapped && small;
+  for (int q = 0; q < 5 && (mapped || plain); ++q) {
+    bool ordinary = false;
+    if (!cnt[q]) continue;
+    m[q] = (const int *)mapped_host(src[q], &ordinary);
+    mapped = mapped && m[q];
+    plain = plain && ordinary;
   }
   // a small batch in page-locked or in ordinary host memory is read in place by
-  // the few kernels that need it, with no staging kernel or copy in front.
+  // its first kernel, the check, with no staging kernel or copy in front.
   // Ordinary arrays go through the handle's page-locked block, into which they
   // are copied here: not in stream order, so only if nothing is queued on the
   // graph's stream, and not where one of the arrays is memory that queued work
   // may write (a mix with page-locked or managed arrays takes the staged copies)
-  bool in_place = !inputs_on_device && nb > 0 && sp::plan_small(g, ni);
-  if (in_place && !mapped) {
-    const void *in[5] = {del_src, del_dst, add_src, add_dst, add_w};
-    for (int q = 0; q < 5; ++q)
-      if ((q < 2 ? n_del : n_add) > 0) in_place = in_place && unregistered_host(in[q]);
-    in_place = in_place && stream_idle(g);
-  }
-  sp_status rc =
-      ensure_batch_buffers(g, ni, inputs_on_device || in_place ? 0 : std::max(n_del, n_add));
+  const bool in_place = small && (mapped || (plain && stream_idle(g)));
+  sp_status rc = ensure_batch_buffers(g, ni, inputs_on_device ? 0 : std::max(n_del, n_add));
   if (rc != SP_OK) return rc;
   auto &b = g->bb;
   rec(g, timed, 0);
   int staged = 0;
-  if (in_place) {
-    const int32_t *src[5] = {del_src, del_dst, add_src, add_dst, add_w};
-    const int *in[5];
+  const int *in[5] = {m[0], m[1], m[2], m[3], m[4]};
+  int *const dst[5] = {b.in_del_src, b.in_del_dst, b.in_add_src, b.in_add_dst, b.in_add_w};
+  if (in_place && !mapped) {
     for (int q = 0; q < 5; ++q) {
-      const long long k = q < 2 ? n_del : n_add;
       int *h = g->small_host + q * sp::kSmallUpdates;
-      if (!mapped && k) std::memcpy(h, src[q], (size_t)k * 4);
-      in[q] = mapped ? (const int *)m[q] : h;
+      if (cnt[q]) std::memcpy(h, src[q], (size_t)cnt[q] * 4);
+      in[q] = h;
     }
-    ds = in[0]; dd = in[1]; as = in[2]; ad = in[3]; aw = in[4];
-  } else if (mapped) {
-    const int *src[5] = {(const int *)m[0], (const int *)m[1], (const int *)m[2],
-                         (const int *)m[3], (const int *)m[4]};
-    int *const dst[5] = {b.in_del_src, b.in_del_dst, b.in_add_src, b.in_add_dst, b.in_add_w};
-    const long long cnt[5] = {n_del, n_del, n_add, n_add, n_add};
-    sp::launch_stage_inputs(g, src, dst, cnt, &staged);
-    ds = b.in_del_src; dd = b.in_del_dst; as = b.in_add_src; ad = b.in_add_dst; aw = b.in_add_w;
-  } else if (!inputs_on_device) {
-    cudaStream_t s = g->stream;
-    const cudaMemcpyKind kind = inputs_on_device ? cudaMemcpyDeviceToDevice
-                                                 : cudaMemcpyHostToDevice;
-    if (n_del) {
-      cudaMemcpyAsync(b.in_del_src, del_src, n_del * 4, kind, s);
-      cudaMemcpyAsync(b.in_del_dst, del_dst, n_del * 4, kind, s);
-    }
-    if (n_add) {
-      cudaMemcpyAsync(b.in_add_src, add_src, n_add * 4, kind, s);
-      cudaMemcpyAsync(b.in_add_dst, add_dst, n_add * 4, kind, s);
-      cudaMemcpyAsync(b.in_add_w, add_w, n_add * 4, kind, s);
-    }
+  } else if (mapped && !in_place) {
+    sp::launch_stage_inputs(g, m, dst, cnt, &staged);
+  } else if (!inputs_on_device && !in_place) {
+    for (int q = 0; q < 5; ++q)
+      if (cnt[q])
+        cudaMemcpyAsync(dst[q], src[q], (size_t)cnt[q] * 4, cudaMemcpyHostToDevice, g->stream);
+  }
+  if (!inputs_on_device) {
     ds = b.in_del_src; dd = b.in_del_dst; as = b.in_add_src; ad = b.in_add_dst; aw = b.in_add_w;
   }
   int launches = 0, regrows = 0;
@@ -978,6 +971,7 @@ sp_status apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
     if (attempt) rec(g, timed, 0);
     cudaError_t e = cudaSuccess;
     bool replayed = false;
+    const int *const *host = in_place && attempt == 0 ? in : nullptr;   // (then it is staged)
     if (use_graph && attempt == 0) {
       if (!(g->bg_ready && g->bg_gen == g->gen && g->bg_nd == n_del && g->bg_na == n_add &&
             g->bg_timed == (int)timed)) {
@@ -986,7 +980,7 @@ sp_status apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
         if (cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
           g->capturing = 0;
           const cudaError_t ce = enqueue_batch(g, ds, dd, n_del, as, ad, aw, n_add, timed, &cl,
-                                               mode0);
+                                               mode0, host);
           g->capturing = -1;
           cudaGraph_t gr = nullptr;
           bool ok = cudaStreamEndCapture(g->stream, &gr) == cudaSuccess && ce == cudaSuccess && gr;
@@ -1000,6 +994,10 @@ sp_status apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
             g->bg_na = n_add;
             g->bg_timed = (int)timed;
             g->bg_launches = cl;
+            const int *const dev[5] = {ds, dd, as, ad, aw};
+            std::copy(dev, dev + 5, g->bg_dev);
+            std::copy(host ? host : dev, (host ? host : dev) + 5, g->bg_in);
+            g->bg_host = host != nullptr;
           } else {
             drop_batch_graphs(g);
           }
@@ -1007,9 +1005,10 @@ sp_status apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
         g->capturing = -1;
         cudaGetLastError();
       }
-      // a replay reads this call's inputs: the two nodes that read them are
-      // pointed at them (no copy of the batch)
-      if (g->bg_ready && retarget_input_nodes(g, ds, dd, n_del, as, ad, aw, n_add) != cudaSuccess) {
+      // a replay reads this call's inputs: the nodes that read them are pointed
+      // at them (no copy of the batch)
+      if (g->bg_ready &&
+          retarget_input_nodes(g, ds, dd, n_del, as, ad, aw, n_add, host) != cudaSuccess) {
         cudaGetLastError();
         drop_batch_graphs(g);
       }
@@ -1021,7 +1020,8 @@ sp_status apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
     }
     if (!replayed)
       e = enqueue_batch(g, ds, dd, n_del, as, ad, aw, n_add, timed, &launches,
-                        attempt == 0 ? mode0 : (mode0 == kInvalBeside ? kInvalKept : kInvalAfter));
+                        attempt == 0 ? mode0 : (mode0 == kInvalBeside ? kInvalKept : kInvalAfter),
+                        host);
     if (e != cudaSuccess) {
       g->last_err = (int)e;
       cudaGetLastError();

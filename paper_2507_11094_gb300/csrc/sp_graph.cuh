@@ -211,6 +211,10 @@ struct sp_graph {
   cudaGraphNode_t bg_sort = nullptr, bg_inval = nullptr,   // nodes that read the inputs
                   bg_search = nullptr, bg_plan = nullptr, bg_check = nullptr;
   bool bg_ready = false;
+  // what the nodes read: the check's arrays (of the host, or as the others), and
+  // the others'
+  const int *bg_in[5] = {}, *bg_dev[5] = {};
+  bool bg_host = false;
   int capturing = -1;                    // >= 0 while the pipeline is captured
   unsigned long long bg_gen = 0;
   long long bg_nd = -1, bg_na = -1;
@@ -290,17 +294,22 @@ const void *inval_fn();
 cudaError_t retarget_inval(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t node, const int *ds,
                            const int *dd, long long nd, int concurrent);
 // A small batch: its control reset and validation, and its searches, sort and
-// count, in one block each.
+// count, in one block each.  host: the check reads host memory and leaves the
+// batch in the staging buffers, for the kernels after it.
 bool plan_small(const sp_graph *g, long long ni);
 void launch_check_small(sp_graph *g, const int *ds, const int *dd, long long nd, const int *as,
-                        const int *ad, const int *aw, long long na, int reset, int *launches);
+                        const int *ad, const int *aw, long long na, bool host, int reset,
+                        int *launches);
 cudaError_t launch_plan(sp_graph *g, const int *ds, const int *dd, long long nd, const int *as,
                         const int *ad, const int *aw, long long na, int *launches);
 const void *plan_fn();
 const void *check_small_fn();
-cudaError_t retarget_plan(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t check,
-                          cudaGraphNode_t plan, const int *ds, const int *dd, long long nd,
-                          const int *as, const int *ad, const int *aw, long long na);
+cudaError_t retarget_check_small(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t node,
+                                 const int *ds, const int *dd, long long nd, const int *as,
+                                 const int *ad, const int *aw, long long na, bool host);
+cudaError_t retarget_plan(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t node, const int *ds,
+                          const int *dd, long long nd, const int *as, const int *ad,
+                          const int *aw, long long na);
 // The searches beside the batch sort; the graph's stream has to wait for
 // search_ev (with a side stream) before their results are read.
 cudaError_t launch_search_sort(sp_graph *g, const int *ds, const int *dd, long long nd,

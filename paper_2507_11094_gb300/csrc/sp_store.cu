@@ -1137,9 +1137,18 @@ __global__ void __launch_bounds__(kPlanT, 1) k_plan(PlanArgs a) {
   }
 }
 
+// Where a small batch in host memory is kept on the device (or all null).
+struct InputCopy {
+  int *ds, *dd, *as, *ad, *aw;
+};
+
 // A small batch's control reset and validation (k_check_batch in one block),
-// after which the invalidation may run beside the plan.
-__global__ void __launch_bounds__(kPlanT) k_check_small(SearchArgs in, Ctl *c, int reset) {
+// after which the invalidation may run beside the plan.  Host arrays are read
+// here and nowhere else: what was checked is copied to the device, and that is
+// what the plan and the invalidation read (they index by it), whatever happens
+// to the caller's arrays meanwhile.
+__global__ void __launch_bounds__(kPlanT)
+    k_check_small(SearchArgs in, Ctl *c, int reset, InputCopy out) {
   const int t = threadIdx.x;
   if (t == (int)blockDim.x - 1) {
     ctl_reset(c, reset);
@@ -1149,8 +1158,13 @@ __global__ void __launch_bounds__(kPlanT) k_check_small(SearchArgs in, Ctl *c, i
   for (long long i = t; i < in.nd + in.na; i += blockDim.x) {
     const bool del = i < in.nd;
     const long long j = del ? i : i - in.nd;
-    const int u = del ? in.ds[j] : in.as[j], v = del ? in.dd[j] : in.ad[j];
-    const int w = del ? 1 : in.aw[j];
+    const int u = __ldcv((del ? in.ds : in.as) + j), v = __ldcv((del ? in.dd : in.ad) + j);
+    const int w = del ? 1 : __ldcv(in.aw + j);   // (read once each)
+    if (out.ds) {
+      (del ? out.ds : out.as)[j] = u;
+      (del ? out.dd : out.ad)[j] = v;
+      if (!del) out.aw[j] = w;
+    }
     bad |= u < 0 || u >= in.n || v < 0 || v >= in.n || w < 1 || w > SP_WMAX;
   }
   if (__syncthreads_or(bad) && t == 0) set_status(c, SP_EINVAL);
@@ -1924,35 +1938,51 @@ cudaError_t launch_plan(sp_graph *g, const int *ds, const int *dd, long long nd,
   return cudaGetLastError();
 }
 
+static InputCopy input_copy(const sp_graph *g, bool host) {
+  const BatchBufs &b = g->bb;
+  return host ? InputCopy{b.in_del_src, b.in_del_dst, b.in_add_src, b.in_add_dst, b.in_add_w}
+              : InputCopy{};
+}
+
 void launch_check_small(sp_graph *g, const int *ds, const int *dd, long long nd, const int *as,
-                        const int *ad, const int *aw, long long na, int reset, int *launches) {
+                        const int *ad, const int *aw, long long na, bool host, int reset,
+                        int *launches) {
   k_check_small<<<1, plan_threads(2 * (nd + na)), 0, g->stream>>>(
-      search_args(g, ds, dd, nd, as, ad, aw, na), g->ctl, reset);
+      search_args(g, ds, dd, nd, as, ad, aw, na), g->ctl, reset, input_copy(g, host));
   ++*launches;
 }
 
 const void *plan_fn() { return (const void *)k_plan; }
 const void *check_small_fn() { return (const void *)k_check_small; }
 
-cudaError_t retarget_plan(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t check,
-                          cudaGraphNode_t plan, const int *ds, const int *dd, long long nd,
-                          const int *as, const int *ad, const int *aw, long long na) {
-  PlanArgs a = plan_args(g, ds, dd, nd, as, ad, aw, na);
+cudaError_t retarget_check_small(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t node,
+                                 const int *ds, const int *dd, long long nd, const int *as,
+                                 const int *ad, const int *aw, long long na, bool host) {
+  SearchArgs in = search_args(g, ds, dd, nd, as, ad, aw, na);
   int reset = 0;
-  void *cargs[3] = {&a.in, &a.ctl, &reset};
-  void *args[1] = {&a};
+  InputCopy out = input_copy(g, host);
+  void *args[4] = {&in, &g->ctl, &reset, &out};
   cudaKernelNodeParams p = {};
   p.func = (void *)k_check_small;
   p.gridDim = dim3(1);
   p.blockDim = dim3(plan_threads(2 * (nd + na)));
   p.sharedMemBytes = 0;
-  p.kernelParams = cargs;
-  const cudaError_t e = cudaGraphExecKernelNodeSetParams(ex, check, &p);
-  if (e != cudaSuccess) return e;
+  p.kernelParams = args;
+  return cudaGraphExecKernelNodeSetParams(ex, node, &p);
+}
+
+cudaError_t retarget_plan(sp_graph *g, cudaGraphExec_t ex, cudaGraphNode_t node, const int *ds,
+                          const int *dd, long long nd, const int *as, const int *ad,
+                          const int *aw, long long na) {
+  PlanArgs a = plan_args(g, ds, dd, nd, as, ad, aw, na);
+  void *args[1] = {&a};
+  cudaKernelNodeParams p = {};
   p.func = (void *)k_plan;
+  p.gridDim = dim3(1);
+  p.blockDim = dim3(plan_threads(2 * (nd + na)));
   p.sharedMemBytes = (unsigned)kPlanSmem;
   p.kernelParams = args;
-  return cudaGraphExecKernelNodeSetParams(ex, plan, &p);
+  return cudaGraphExecKernelNodeSetParams(ex, node, &p);
 }
 
 // The items' searches in their old rows run beside the batch sort (on the SMs

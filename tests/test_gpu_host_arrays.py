@@ -70,3 +70,44 @@ def test_arrays_that_queued_work_still_fills(k, pinned):
             for x, y in zip(g.export_csr(), ref.csr()):
                 np.testing.assert_array_equal(x, y)
             old = b
+
+
+# page-locked arrays of a small batch that another thread keeps changing, to ids
+# out of range too, while the call runs: they are read once, so what was checked
+# is what is applied, or nothing is (a mix of two batches at worst)
+@pytest.mark.parametrize("k", [6, 1024])
+def test_arrays_that_change_during_the_call(k):
+    import threading
+    import torch
+    n = 3000
+    ro, col, w = wl.er_digraph(n, 20000, 1, 100, seed=3)
+    rng = np.random.default_rng(k)
+    ref = oracle.OracleGraph(n, ro, col, w)
+    two = [batch(ref, n, k, rng) for _ in range(2)]
+    pins = [torch.empty(a.size, dtype=torch.int32, pin_memory=True).numpy() for a in two[0]]
+    stop = threading.Event()
+
+    def change():
+        i = 0
+        while not stop.is_set():
+            i += 1
+            for p, a in zip(pins, two[i % 2]):
+                p[:] = a
+            if i % 3 == 0:
+                pins[1][::2] = 0x7FFFFFF0
+                pins[3][1::2] = -5
+    with sp.Graph(n, ro, col, w, stream=torch.cuda.Stream()) as g:
+        g.sssp_init(0)
+        for p, a in zip(pins, two[0]):
+            p[:] = a
+        t = threading.Thread(target=change)
+        t.start()
+        codes = set()
+        for _ in range(300):
+            codes.add(g.apply_batch(*pins, raise_on_error=False)[0])
+        stop.set()
+        t.join()
+        assert codes <= {sp.SP_OK, sp.SP_EINVAL}
+        ref = oracle.OracleGraph(n, *g.export_csr())
+        assert g.m == ref.csr()[1].size
+        np.testing.assert_array_equal(g.get_dist(), ref.dijkstra(0))
