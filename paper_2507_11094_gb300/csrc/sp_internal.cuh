@@ -178,6 +178,11 @@ struct Limits {
 // Every barrier wait also ends after this many polls, whatever the clock
 // says (a poll sleeps 64 ns and reads one word: seconds in all).
 constexpr u32 kMaxPolls = 1u << 24;
+// Polls between two looks at the clock, less one: sixteen polls take about 10 us,
+// and many waits less, so a bound of that order is looked at on every poll.
+__device__ __forceinline__ u32 clock_polls(unsigned long long wait_ns) {
+  return wait_ns < 20000ull ? 0u : 15u;
+}
 
 // ---------------------------------------------------------------------------
 // Small device helpers.
@@ -235,15 +240,15 @@ __device__ __forceinline__ bool coop_barrier(u64 *bar, u64 target, Ctl *c, u64 w
     __threadfence();
     // the count before this arrival says whether it was the last one; the
     // wait polls the count alone and looks at the status and the clock every
-    // 16th poll.  (miss_site: block 0 does not arrive, and every wait of the
-    // barrier runs out.)
+    // 16th poll, or every one (clock_polls).  (miss_site: block 0 does not
+    // arrive, and every wait of the barrier runs out.)
     const bool miss = miss_site == site && blockIdx.x == 0;
     const u64 arrived = miss ? ld_acquire_u64_(bar) : atomicAdd((unsigned long long *)bar, 1ull) + 1;
     if (arrived < target) {
       const u64 t0 = globaltimer_ns();
       u32 polls = 0;
       while (ld_acquire_u64_(bar) < target) {
-        if ((++polls & 15u) == 0) {
+        if ((++polls & clock_polls(wait_ns)) == 0) {
           if (ld_cg_i32(&c->status) != 0) break;
           if (globaltimer_ns() - t0 > wait_ns || polls > kMaxPolls) {
             if (atomicCAS(&c->status, 0, SP_ETIMEOUT) == 0) {

@@ -74,7 +74,7 @@ __device__ __forceinline__ bool grid_sync(u64 *bar, u64 target, Ctl *c, const Li
     __threadfence();
     // the count before this arrival says whether it was the last one; the
     // wait polls the count alone and looks at the timeout flag and the
-    // clock every 16th poll
+    // clock every 16th poll (on every poll where the bound is that short)
     // (the test hook lim.miss_site == 2: block 0 does not arrive)
     const bool miss = lim.miss_site == 2u && blockIdx.x == 0;
     const u64 arrived = miss ? ld_acquire_u64(bar) : atomicAdd((unsigned long long *)bar, 1ull) + 1;
@@ -82,7 +82,7 @@ __device__ __forceinline__ bool grid_sync(u64 *bar, u64 target, Ctl *c, const Li
       const u64 t0 = globaltimer_ns();
       u32 polls = 0;
       while (ld_acquire_u64(bar) < target) {
-        if ((++polls & 15u) == 0) {
+        if ((++polls & clock_polls(lim.wait_ns)) == 0) {
           if (ld_cg_i32(&c->timeout) != 0) break;
           if (globaltimer_ns() - t0 > lim.wait_ns || polls > kMaxPolls) {
             raise_timeout(c, 2, 2, (u32)(target / gridDim.x));

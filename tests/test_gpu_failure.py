@@ -245,3 +245,21 @@ def test_pool_growth_failure_leaves_graph_unchanged(beside):
         check_all(g, ref, 0, store=True)
     finally:
         g.close()
+
+
+def test_a_wait_bound_below_sixteen_polls_is_kept():
+    """Small batches' repairs wait a few polls at a time: a 1 ns bound runs out
+    in (nearly) every call, not only in those that wait for long."""
+    W = wl.grid(96, 96, batch_frac=0.02, seed=5)
+    hits = 0
+    with sp.Graph(W.n, W.row_off, W.col, W.w) as g:
+        g.set_local_rounds(0)
+        for k in range(24):
+            g.set_limits(0, 0)
+            g.sssp_init(W.source)
+            d = g.get_dist()
+            g.set_limits(0, 1)
+            rc, _ = _apply(g, W.batch(k, dist=d))
+            assert rc in (sp.SP_OK, sp.SP_ETIMEOUT)
+            hits += rc == sp.SP_ETIMEOUT
+    assert hits >= 22, hits
