@@ -822,8 +822,9 @@ sp_status resolve_out(sp_graph *g, int32_t *dist, int32_t *parent, int out_on_de
     o->parent_d = parent;
     return SP_OK;
   }
-  int32_t *md = (int32_t *)mapped_host(dist);
-  int32_t *mp = parent ? (int32_t *)mapped_host(parent) : nullptr;
+  bool plain_d = false, plain_p = false;
+  int32_t *md = (int32_t *)mapped_host(dist, &plain_d);
+  int32_t *mp = parent ? (int32_t *)mapped_host(parent, &plain_p) : nullptr;
   if (md && (!parent || mp)) {   // page-locked and mapped: written in place
     o->dist_d = md;
     o->parent_d = mp;
@@ -831,7 +832,9 @@ sp_status resolve_out(sp_graph *g, int32_t *dist, int32_t *parent, int out_on_de
   }
   o->dist_h = dist;
   o->parent_h = parent;
-  if (g->n <= sp::kSmallOut) {   // through the handle's page-locked block
+  // through the handle's page-locked block, which the host copies from: only into
+  // memory that is the host's (the copy engine tells what else there is)
+  if (g->n <= sp::kSmallOut && (md || plain_d) && (!parent || mp || plain_p)) {
     o->dist_d = g->small_host + 5 * sp::kSmallUpdates;
     o->parent_d = parent ? o->dist_d + sp::kSmallOut : nullptr;
     o->from_block = true;
