@@ -1817,7 +1817,9 @@ void launch_merge(sp_graph *g, long long ni, int *launches) {
   a.bits = g->bits;
   a.n_items = (u32)ni;
   // exactly the resident blocks: every warp starts at once and the strips
-  // spread evenly over them (a small batch: a block per item at most)
+  // spread evenly over them.  A small batch starts no more blocks than there can
+  // be work for: one per item, and one per kMergeGrab strips a warp of all that
+  // the stores hold (one update of a hub's row is thousands of strips)
   static int per_sm = 0;
   if (per_sm == 0 &&
       (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_merge, kThreads, 0) !=
@@ -1825,7 +1827,9 @@ void launch_merge(sp_graph *g, long long ni, int *launches) {
        per_sm < 1))
     per_sm = 4;
   const long long full = std::max(1, g->num_sms * per_sm);
-  k_merge<<<(unsigned)std::min(full, ni), kThreads, 0, g->stream>>>(a);
+  const long long strips = (g->fwd.slots + g->rev.slots) / 2 / kStrip;   // two regions a row
+  const long long most = ni + strips / (kMergeGrab * (kThreads / 32)) + 1;
+  k_merge<<<(unsigned)std::min(full, most), kThreads, 0, g->stream>>>(a);
   *launches += 1;
 }
 

@@ -200,3 +200,32 @@ def test_searches_beside_the_sort_of_triangle_and_rank_batches(own_stream):
             np.testing.assert_allclose(g.pr_get(), want, rtol=2e-5, atol=1e-9)
             for x, y in zip(g.export_csr(), ref.csr()):
                 np.testing.assert_array_equal(x, y)
+
+
+def test_one_update_of_a_hub_merges_as_fast_as_many():
+    # the hub's row is 7,800 strips of the merge whatever the batch's size; seven
+    # hundred updates start the whole grid (with a block per item only, one
+    # update's merge took the time of two blocks: tens of times as long)
+    n = 2000003
+    ro = np.concatenate([[0], np.full(n, n - 1)]).astype(np.int64)
+    col = np.arange(1, n, dtype=np.int32)
+    z = np.zeros(0, np.int32)
+    best = {}
+    with sp.Graph(n, ro, col, np.ones(n - 1, np.int32)) as g:
+        g.sssp_init(0)
+        for k in (1, 700):
+            d = (np.arange(k, dtype=np.int32) * 2801 + 17).astype(np.int32)
+            o = np.zeros(k, np.int32)
+            ms = []
+            for _ in range(6):
+                for args in ((o, d, z, z, z), (z, z, o, d, np.ones(k, np.int32))):
+                    st = g.apply_batch(*args, stats=True)
+                    assert st.n_del_applied + st.n_add_applied == k
+                    ms.append(st.ms_phase[sp.PHASES.index("merge")])
+            best[k] = min(ms)
+        d = g.get_dist()
+        assert d[0] == 0 and (d[1:] == 1).all()
+        got = g.export_csr()
+        for x, y in zip(got, (ro, col, np.ones(n - 1, np.int32))):
+            np.testing.assert_array_equal(x, y)
+    assert best[1] < 3 * best[700] + 0.02, best
