@@ -40,6 +40,7 @@
 // cold gathers and the list reads through L2, about half each.
 #include <algorithm>
 
+#include "sp_acc.cuh"
 #include "sp_loop.cuh"
 
 namespace sp {
@@ -190,25 +191,6 @@ __device__ __forceinline__ void first_words(const Unit &x, uint4 w[2]) {
   const uint4 pad = make_uint4(kZeroPlace, kZeroPlace, kZeroPlace, kZeroPlace);
   w[0] = x.q0 < x.nq ? __ldcg(x.l + x.q0) : pad;
   w[1] = x.q0 + x.width < x.nq ? __ldcg(x.l + x.q0 + x.width) : pad;
-}
-
-// A sum of |a - b| kept as hi + lo with error-free sums of 32-bit floats: as
-// exact as in 64 bits, which this GPU adds at 1/64 of the rate.
-struct Acc {
-  float hi = 0.0f, lo = 0.0f;
-};
-
-__device__ __forceinline__ void acc_add(Acc &c, float x) {
-  const float s = __fadd_rn(c.hi, x), z = __fsub_rn(s, c.hi);
-  c.lo = __fadd_rn(c.lo, __fadd_rn(__fsub_rn(c.hi, __fsub_rn(s, z)), __fsub_rn(x, z)));
-  c.hi = s;
-}
-
-__device__ __forceinline__ void acc_diff(Acc &c, float a, float b) {
-  const float d = __fsub_rn(a, b), z = __fsub_rn(d, a);   // a - b = d + e exactly
-  const float e = __fsub_rn(__fsub_rn(a, __fsub_rn(d, z)), __fadd_rn(b, z));
-  acc_add(c, fabsf(d));
-  c.lo = __fadd_rn(c.lo, d < 0.0f ? -e : e);
 }
 
 // The new rank of the row at a position from the sum of its terms.
@@ -591,13 +573,19 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
                __ldcg(a.rank + pos), diff);
       }
     {
-      double x = (double)diff.hi + (double)diff.lo;
+      // (the warp's 32 sums meet as floats too: in 64 bits 1.8 us a step)
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-      if (lane == 0) s_sum[warp] = x;
+      for (int o = 16; o > 0; o >>= 1) {
+        Acc other;
+        other.hi = __shfl_xor_sync(kFull, diff.hi, o);
+        other.mid = __shfl_xor_sync(kFull, diff.mid, o);
+        other.lo = __shfl_xor_sync(kFull, diff.lo, o);
+        acc_merge(diff, other);
+      }
+      if (lane == 0) s_sum[warp] = acc_value(diff);
       __syncthreads();
       if (warp == 0) {
-        x = s_sum[lane];
+        double x = s_sum[lane];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
         if (lane == 0 && x != 0.0) atomicAdd(prd_ptr(c, it % 3), x);
