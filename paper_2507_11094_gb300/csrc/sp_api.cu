@@ -1553,7 +1553,9 @@ sp_status sp_tc_apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
     g->pr_state = 0;   // nor do ranks
   }
   const u64 *d = c.tc_del, *a = c.tc_ins;
-  if (d[0] % 2 || d[1] % 4 || d[2] % 6 || a[0] % 2 || a[1] % 4 || a[2] % 6) {
+  // (both directions of every update applied, and each triangle was seen from
+  // every updated edge of it; each sighting counts twice)
+  if (c.tc_skew[0] || c.tc_skew[1] || d[1] % 4 || d[2] % 6 || a[1] % 4 || a[2] % 6) {
     g->tc_state = 0;   // cannot happen on a symmetric graph and batch
     return SP_ECUDA;
   }

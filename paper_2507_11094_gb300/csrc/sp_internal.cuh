@@ -122,6 +122,7 @@ struct Ctl {
   alignas(128) u32 tc_spos;
   u64 tc_ntask[2];                 // corrections: tasks listed (deletions, insertions)
   alignas(128) u64 tc_tpos[2];     // ... and handed out so far
+  int tc_skew[2];                  // applied updates u -> v with u < v, less those with u > v
   // the invalidation's cut vertices (a plain list: the pull stage of the
   // push launch turns them into the affected list A)
   alignas(128) u32 ccnt;

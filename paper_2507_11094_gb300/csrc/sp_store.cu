@@ -317,6 +317,7 @@ __device__ __forceinline__ void ctl_reset(Ctl *c, int full) {
   c->tc_static = 0;
   c->tc_ngiant = c->tc_nbig = c->tc_nmid = c->tc_bpos = c->tc_spos = 0;
   c->tc_ntask[0] = c->tc_ntask[1] = c->tc_tpos[0] = c->tc_tpos[1] = 0;
+  c->tc_skew[0] = c->tc_skew[1] = 0;
   c->tc_del[0] = c->tc_del[1] = c->tc_del[2] = 0;
   c->tc_ins[0] = c->tc_ins[1] = c->tc_ins[2] = 0;
   c->lres = c->lcur = c->lround = c->lcap = 0;

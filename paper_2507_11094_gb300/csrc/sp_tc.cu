@@ -439,7 +439,9 @@ __global__ void __launch_bounds__(kThreads) k_tc_batch_sym(const u64 *keys, long
 
 // The corrections' work list.  Every updated pair is among the items in both
 // directions and both see the same common neighbours with the same number of
-// updated edges, so only u < v is walked and its sightings count twice.  An
+// updated edges, so only u < v is walked and its sightings count twice
+// (that both directions applied is counted here, for the host to check: a
+// replayed batch can leave the graph with one direction of an edge).  An
 // item whose shorter row is long is listed up to kMaxParts times, each part
 // a share of the walk: without the split one pair of hubs (a walk of
 // thousands of searches by one warp) outlasts the rest of the batch.
@@ -466,10 +468,13 @@ __global__ void __launch_bounds__(kThreads) k_tc_tasks(DeltaArgs a) {
   for (long long b = blockIdx.x * (long long)kThreads + (threadIdx.x & ~31); b < a.nb; b += step) {
     const long long i = b + lane;
     u32 parts[2] = {0, 0};
+    int skew[2] = {0, 0};
     if (i < a.nb) {
       const u64 key = __ldg(&a.keys[i]);
       const u32 u = (u32)((key >> (a.bits + 1)) & cmask), v = (u32)((key >> 1) & cmask);
-      if (u < v && (__ldg(&a.flags[i]) & 1)) {
+      const bool applied = __ldg(&a.flags[i]) & 1;
+      if (applied && u != v) skew[key & 1] = u < v ? 1 : -1;
+      if (u < v && applied) {
         const int du = __ldg(&a.st.row[u].deg), dv = __ldg(&a.st.row[v].deg);
         const int walk = du < dv ? du : dv;
         parts[key & 1] = (u32)min(kMaxParts, walk / kPartWalk + 1);
@@ -477,6 +482,8 @@ __global__ void __launch_bounds__(kThreads) k_tc_tasks(DeltaArgs a) {
     }
 #pragma unroll
     for (int kind = 0; kind < 2; ++kind) {
+      const int off = __reduce_add_sync(kFull, skew[kind]);
+      if (lane == 0 && off) atomicAdd(&a.c->tc_skew[kind], off);
       const u32 incl = warp_incl_scan(parts[kind]), total = __shfl_sync(kFull, incl, 31);
       if (!total) continue;
       u64 base = 0;

@@ -189,3 +189,39 @@ def test_an_asymmetric_edge_is_found(at):
         with pytest.raises(sp.SpError) as e:
             g.tc_init()
         assert e.value.code == sp.SP_EINVAL
+
+
+# a replayed batch that made the graph asymmetric behind the count's back: an
+# update that then applies in one direction only, either one, is noticed
+@pytest.mark.parametrize("u,v", [(3, 11), (11, 3)])
+@pytest.mark.parametrize("gone", [False, True])
+def test_a_batch_that_applies_in_one_direction_is_refused(u, v, gone):
+    import torch
+    n = 20
+    # u and v have one common neighbour; one edge between them, or both
+    pairs = [(u, 5), (v, 5), (5, 6)] + ([(u, v)] if gone else [])
+    e = sorted(set(pairs) | {(b, a) for a, b in pairs})
+    ro = np.zeros(n + 1, np.int64)
+    np.cumsum(np.bincount([a for a, _ in e], minlength=n), out=ro[1:])
+    i32 = lambda *x: np.array(x, np.int32)
+    z = i32()
+    with sp.Graph(n, ro, i32(*[b for _, b in e]), np.ones(len(e), np.int32),
+                  stream=torch.cuda.Stream()) as g:
+        g.sssp_init(0)
+        g.reserve(16)
+        one = (i32(u), i32(v), z, z, z) if gone else (z, z, i32(u), i32(v), i32(1))
+        x = g.capture(*[torch.from_numpy(a).cuda() for a in one])
+        assert g.tc_init() == (1 if gone else 0)
+        x.launch()
+        g.sync()
+        both = (i32(u, v), i32(v, u))
+        with pytest.raises(sp.SpError) as err:
+            if gone:     # v -> u alone is there to go
+                g.tc_apply_batch(*both, z, z, z)
+            else:        # v -> u alone is there to come
+                g.tc_apply_batch(z, z, *both, i32(1, 1))
+        assert err.value.code == sp.SP_ECUDA
+        with pytest.raises(sp.SpError) as err:
+            g.tc_apply_batch(z, z, z, z, z)
+        assert err.value.code == sp.SP_ESTATE
+        x.close()
