@@ -142,15 +142,22 @@ void fill_stats(sp_graph *g, const Ctl &c, sp_batch_stats *st, int launches, int
   st->n_launches = launches;
   st->regrows = regrows;
   // Algorithmic bytes: what each phase must move, counted from what it did.
-  const int passes = (2 * g->bits + 2 + 7) / 8;
   const long long nb = ni / 2;
-  // the sort phase also holds the old-row searches that run beside the sort
-  // (inputs 10 per item on average, the row's meta 16, the result 8)
-  st->alg_bytes[SP_PH_SORT] =
-      ni ? (int64_t)(nb * 20 + ni * 12 + (long long)passes * ni * 24 + ni * 34) : 0;
-  // key 8, number 4 and search result 8 read; opos 4, flags 1, weight 4 and
-  // prefix 8 written per item; 16 per touched row
-  st->alg_bytes[SP_PH_COUNT] = (int64_t)(ni * 37 + (long long)c.rows_touched * 16);
+  if (ni && sp::plan_small(g, ni)) {
+    // one block checks the batch (10 per update on average) and one plans it:
+    // inputs 10, row's meta 16 read, key 8, opos 4, weight 4, flags 1 and prefix 8
+    // written per item; 16 per touched row
+    st->alg_bytes[SP_PH_SORT] = (int64_t)(nb * 10);
+    st->alg_bytes[SP_PH_COUNT] = (int64_t)(ni * 51 + (long long)c.rows_touched * 16);
+  } else {
+    // the sort phase also holds the old-row searches that run beside the sort
+    // (inputs 10 per item on average, the row's meta 16, the result 8)
+    const long long passes = ni ? sp::batch_sort_passes(g, ni) : 0;
+    st->alg_bytes[SP_PH_SORT] = (int64_t)(nb * 20 + ni * 12 + passes * ni * 24 + ni * 34);
+    // key 8, number 4 and search result 8 read; opos 4, flags 1, weight 4 and
+    // prefix 8 written per item; 16 per touched row
+    st->alg_bytes[SP_PH_COUNT] = (int64_t)(ni * 37 + (long long)c.rows_touched * 16);
+  }
   st->alg_bytes[SP_PH_MERGE] = (int64_t)(c.merge_slots * 8 + c.rows_touched * 32 + ni * 21);
   st->alg_bytes[SP_PH_INVAL] =
       (int64_t)(c.affected * (16 + 8 + 8 + 4) + c.inval_edges * 16);
@@ -1312,6 +1319,7 @@ sp_status pr_phase(sp_graph *g, const int *ds, const int *dd, long long nd, cons
   if (rc != SP_OK) return rc;
   const Ctl &c = *g->ctl_host;
   acc.pull_edges += c.pull_edges;
+  acc.push_vertices += c.affected * c.pr_iters;   // the flagged, in every step
   acc.rounds_push += c.pr_iters;
   if (c.bad) return SP_ECUDA;
   if (c.timeout) return SP_ETIMEOUT;
@@ -1335,10 +1343,11 @@ void pr_stats(sp_graph *g, const Ctl &c, sp_batch_stats *st, int launches, int r
   st->n_launches = launches;
   st->regrows = regrows;
   // algorithmic bytes: flag propagation (as a frontier walk), the merge, and
-  // per pulled in-edge its source id (4), rank (4) and out-degree (4)
+  // per pulled in-edge its place (4) and term (4), per vertex and step its old
+  // and new rank, term, place, degree and list (24)
   st->alg_bytes[SP_PH_INVAL] = (int64_t)(c.affected * 16 + c.inval_edges * 12);
   st->alg_bytes[SP_PH_MERGE] = (int64_t)(c.merge_slots * 8 + c.rows_touched * 32);
-  st->alg_bytes[SP_PH_PULL] = (int64_t)(c.pull_edges * 12);
+  st->alg_bytes[SP_PH_PULL] = (int64_t)(c.pull_edges * 8 + c.push_vertices * 24);
   st->ms_total = ms;
   (void)g;
 }
@@ -1384,6 +1393,7 @@ sp_status sp_pr_init(sp_graph *g, float damping, float beta, int32_t max_iter,
   acc.pull_edges = c.pull_edges;
   acc.rounds_push = c.pr_iters;
   acc.affected = (u64)g->n;
+  acc.push_vertices = (u64)g->n * c.pr_iters;
   pr_stats(g, acc, stats, launches, 0, ms);
   return SP_OK;
 }

@@ -277,6 +277,7 @@ cudaError_t launch_batch_sort(sp_graph *g, const int *ds, const int *dd, long lo
 // the captured batch-sort / invalidation node of an instantiated graph,
 // pointed at another batch of the same shape
 bool is_batch_sort(const void *fn);
+int batch_sort_passes(const sp_graph *g, long long ni);
 // The old-row searches of a batch's items (their positions, whether the
 // edge is there, and their weights into bb.srch), for the count pass; they
 // read only the old stores, so they may run beside the batch sort.

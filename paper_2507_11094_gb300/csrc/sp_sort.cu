@@ -683,6 +683,25 @@ struct SortLaunch {
   int G;
 };
 
+// How ni items are sorted: in one half or two, and the digits.
+struct SortShape {
+  int halves, passes;
+  bool wide;   // ten bits a digit
+};
+
+SortShape sort_shape(const sp_graph *g, long long ni) {
+  int cap = g->sort_blocks;
+  if (g->loop_blocks_user > 0 && g->loop_blocks_user < cap) cap = g->loop_blocks_user;
+  SortShape s;
+  // two blocks or more: as many for either store
+  s.halves = ni > kBTile && cap >= 2 ? 2 : 1;
+  const int key_bits = 2 * g->bits + (s.halves == 1 ? 1 : 0);
+  const int p9 = std::max((key_bits + 8) / 9, 1), p10 = std::max((key_bits + 9) / 10, 1);
+  s.wide = p10 < p9;
+  s.passes = s.wide ? p10 : p9;
+  return s;
+}
+
 // Arguments and grid of the batch sort for these inputs.
 SortLaunch batch_sort_args(sp_graph *g, const int *ds, const int *dd, long long nd,
                            const int *as, const int *ad, const int *aw, long long na,
@@ -691,8 +710,8 @@ SortLaunch batch_sort_args(sp_graph *g, const int *ds, const int *dd, long long 
   BatchBufs &bb = g->bb;
   int cap = g->sort_blocks;
   if (g->loop_blocks_user > 0 && g->loop_blocks_user < cap) cap = g->loop_blocks_user;
-  // two blocks or more: as many for either store
-  a.halves = ni > kBTile && cap >= 2 ? 2 : 1;
+  const SortShape sh = sort_shape(g, ni);
+  a.halves = sh.halves;
   const long long nh = ni / (int)a.halves;
   const int Gh = (int)std::max(1ll, std::min<long long>((nh + kBTile - 1) / kBTile,
                                                         cap / (int)a.halves));
@@ -701,10 +720,7 @@ SortLaunch batch_sort_args(sp_graph *g, const int *ds, const int *dd, long long 
   a.nd = nd; a.na = na;
   a.n = g->n;
   a.bits = g->bits;
-  const int key_bits = 2 * g->bits + (a.halves == 1 ? 1 : 0);
-  const int p9 = std::max((key_bits + 8) / 9, 1), p10 = std::max((key_bits + 9) / 10, 1);
-  const bool wide = p10 < p9;
-  a.passes = wide ? p10 : p9;
+  a.passes = sh.passes;
   // the last pass writes keys/vals
   const int odd = a.passes & 1;
   a.kbuf[0] = odd ? bb.keys_alt : bb.keys;
@@ -720,11 +736,13 @@ SortLaunch batch_sort_args(sp_graph *g, const int *ds, const int *dd, long long 
   a.chunk = (u32)((nh + Gh - 1) / Gh);
   // a handle with a block share gives each block an SM of its own
   const size_t least = g->loop_blocks_user > 0 ? kExclusiveSmem : 0;
-  if (wide) return {k_batch_sort<10>, std::max(kBSmem<10>, least), G};
+  if (sh.wide) return {k_batch_sort<10>, std::max(kBSmem<10>, least), G};
   return {k_batch_sort<9>, std::max(kBSmem<9>, least), G};
 }
 
 }  // namespace
+
+int batch_sort_passes(const sp_graph *g, long long ni) { return sort_shape(g, ni).passes; }
 
 bool is_batch_sort(const void *fn) {
   return fn == (const void *)k_batch_sort<9> || fn == (const void *)k_batch_sort<10>;
