@@ -1516,8 +1516,7 @@ sp_status sp_tc_apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
   for (int attempt = 0;; ++attempt) {
     sp::launch_ctl_reset(g, 0, &launches);
     const cudaError_t es =
-        sp::launch_store_plan(g, ds, dd, n_del, as, ad, aw, n_add, &launches);
-    rec(g, true, 1);
+        sp::launch_store_plan(g, ds, dd, n_del, as, ad, aw, n_add, &launches, g->ev[1]);
     sp::launch_tc_batch_sym(g, nb, &launches);     // before anything changes
     sp::launch_tc_tasks(g, nb, &launches);
     rec(g, true, 2);

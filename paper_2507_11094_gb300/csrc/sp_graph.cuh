@@ -317,10 +317,11 @@ cudaError_t launch_search_sort(sp_graph *g, const int *ds, const int *dd, long l
                                const int *as, const int *ad, const int *aw, long long na,
                                int *launches);
 // Everything before a batch's merge on the graph's stream, by either way
-// (after a control reset).
+// (after a control reset).  sorted: an event between the sort phase and the
+// count phase (a small batch's plan is of the latter), or null.
 cudaError_t launch_store_plan(sp_graph *g, const int *ds, const int *dd, long long nd,
                               const int *as, const int *ad, const int *aw, long long na,
-                              int *launches);
+                              int *launches, cudaEvent_t sorted = nullptr);
 void launch_check_batch(sp_graph *g, const int *ds, const int *dd, long long nd, const int *as,
                         const int *ad, const int *aw, long long na, int *launches);
 

@@ -2012,11 +2012,14 @@ cudaError_t launch_search_sort(sp_graph *g, const int *ds, const int *dd, long l
 
 cudaError_t launch_store_plan(sp_graph *g, const int *ds, const int *dd, long long nd,
                               const int *as, const int *ad, const int *aw, long long na,
-                              int *launches) {
+                              int *launches, cudaEvent_t sorted) {
   const long long ni = 2 * (nd + na);
-  if (ni == 0) return cudaSuccess;
-  if (plan_small(g, ni)) return launch_plan(g, ds, dd, nd, as, ad, aw, na, launches);
-  const cudaError_t e = launch_search_sort(g, ds, dd, nd, as, ad, aw, na, launches);
+  const bool small = plan_small(g, ni);
+  cudaError_t e = cudaSuccess;
+  if (ni && !small) e = launch_search_sort(g, ds, dd, nd, as, ad, aw, na, launches);
+  if (sorted) cudaEventRecord(sorted, g->stream);
+  if (ni == 0) return e;
+  if (small) return launch_plan(g, ds, dd, nd, as, ad, aw, na, launches);
   if (g->side) cudaStreamWaitEvent(g->stream, g->search_ev, 0);
   launch_count(g, ni, launches);
   return e;

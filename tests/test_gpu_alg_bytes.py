@@ -56,3 +56,23 @@ def test_rank_bytes():
         st = g.pr_apply(insertions(n, 700, 2), stats=True)   # one phase
         assert st.alg_bytes[PH["pull"]] == (8 * st.relaxed_edges +
                                             24 * st.affected * st.rounds_push)
+
+
+def test_the_count_phase_of_a_triangle_batch():
+    # phases are those of an update batch: the plan of a small one (1,000 updates:
+    # searches, sort and count in one block) is of the count phase, after a sort
+    # phase in which only the control block is reset
+    import torch
+    W = wl.sym_er(65536, 600000, 250, 3)
+    sort, count = [], []
+    with sp.Graph(W.n, W.row_off, W.col, W.w) as g:
+        g.tc_init()
+        for k in range(6):
+            b = W.batch(k)
+            assert b.size <= 1024
+            dev = [torch.from_numpy(x).cuda() for x in
+                   (b.del_src, b.del_dst, b.add_src, b.add_dst, b.add_w)]
+            _, st = g.tc_apply_batch(*dev, stats=True)
+            sort.append(st.ms_phase[PH["sort"]])
+            count.append(st.ms_phase[PH["count"]])
+    assert min(sort) < 0.5 * min(count), (sort, count)
