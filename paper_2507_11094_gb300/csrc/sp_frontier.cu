@@ -334,53 +334,31 @@ __device__ __forceinline__ void prefetch_l2(const void *p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
-// Append each lane's improved near targets to pool list b (warp-collective).
-// A target with 1..kPoolDeg out-edges becomes an entry (x, nd, start / 4,
-// deg); with kMeta false the row is not known yet and the entry carries
-// kPoolUnknown instead (the drain reads it).  A target without out-edges
-// needs nothing; a larger one, or one that finds the list full, comes back
-// in rest[] for the global frontier.
-template <bool kMeta>
-__device__ __forceinline__ void pool_push(Pool *pl, u32 b, const u32 *x, const u32 *nd,
-                                          const bool *want, int kk, const u32 *ms4,
-                                          const int *mdg, bool *rest, u64 &n_in,
-                                          const RowMeta *row, const int2 *adj) {
+// Append each lane's improved near targets to the pool's first list
+// (warp-collective), as entries (x, nd, 0, kPoolUnknown): their rows are not
+// known yet, the drain reads them.  One that finds the list full comes back in
+// rest[] for the global frontier.
+__device__ __forceinline__ void pool_push(Pool *pl, const u32 *x, const u32 *nd, const bool *want,
+                                          int kk, bool *rest, u64 &n_in, const RowMeta *row) {
   const int lane = threadIdx.x & 31;
-  bool take[K];
   u32 cnt = 0;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     rest[k] = false;
-    take[k] = false;
-    if (k < kk && want[k]) {
-      if (!kMeta || (mdg[k] > 0 && mdg[k] <= kPoolDeg)) {
-        take[k] = true;
-        ++cnt;
-      } else if (mdg[k] > kPoolDeg) {
-        rest[k] = true;
-      }
-    }
+    cnt += k < kk && want[k];
   }
   if (!__ballot_sync(kFull, cnt > 0)) return;
   const u32 ci = warp_incl_scan(cnt), tot = __shfl_sync(kFull, ci, 31);
   u32 base = 0;
-  if (lane == 31) base = atomicAdd(&pl->n[b], tot);
+  if (lane == 31) base = atomicAdd(&pl->n[0], tot);
   base = __shfl_sync(kFull, base, 31) + ci - cnt;
-  uint4 *E = pl->e[b];
+  uint4 *E = pl->e[0];
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    if (take[k]) {
+    if (k < kk && want[k]) {
       if (base < kPoolCap) {
-        E[base] = kMeta ? make_uint4(x[k], nd[k], ms4[k], (u32)mdg[k])
-                        : make_uint4(x[k], nd[k], 0u, kPoolUnknown);
-        // what the entry's expansion reads first: its edges (or its row)
-        if (kMeta) {
-          const int2 *e0 = adj + ((long long)ms4[k] << 2);
-          prefetch_l2(e0);
-          prefetch_l2(e0 + mdg[k] - 1);
-        } else {
-          prefetch_l2(row + x[k]);
-        }
+        E[base] = make_uint4(x[k], nd[k], 0u, kPoolUnknown);
+        prefetch_l2(row + x[k]);   // what the entry's expansion reads first
         ++n_in;
       } else {
         rest[k] = true;
@@ -641,7 +619,7 @@ struct PushOp {
     }
     if (pool) {
       bool rest[K];
-      pool_push<false>(pool, 0, tx, nd, pw, KK, nullptr, nullptr, rest, n_in, row, nullptr);
+      pool_push(pool, tx, nd, pw, KK, rest, n_in, row);
 #pragma unroll
       for (int k = 0; k < KK; ++k)
         if (rest[k]) want[k] = atomicExch(qflag + tx[k], tag) != tag;
@@ -1664,8 +1642,7 @@ __global__ void __launch_bounds__(is_pool(OP) ? kPoolThreads : kPersistThreads, 
           moved += near[0];
           if (is_pool(OP)) {   // into the pool; what does not fit to the frontier
             bool rest[K];
-            pool_push<false>(&pool, 0, x, dx, near, 1, nullptr, nullptr, rest, pc.n_in,
-                             a.fwd.row, nullptr);
+            pool_push(&pool, x, dx, near, 1, rest, pc.n_in, a.fwd.row);
             near[0] = rest[0] && atomicExch(a.qflag + x[0], tag) != tag;
           }
           enqueue(qn, a.fwd.row, x, near, 1, n_enq);
