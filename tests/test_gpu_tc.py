@@ -225,3 +225,29 @@ def test_a_batch_that_applies_in_one_direction_is_refused(u, v, gone):
             g.tc_apply_batch(z, z, z, z, z)
         assert err.value.code == sp.SP_ESTATE
         x.close()
+
+
+# Three hubs joined to a rim of k in both directions and to each other in one
+# (h1 -> h2 -> h3 -> h1) or both: every row is as long in the forward store as in
+# the reverse one, and only the hubs' rows differ.  They are rows that a warp, a
+# block or the whole grid compares, at the bounds of each
+@pytest.mark.parametrize("k", [0, 1, 30, 31, 254, 255, 256, 65534, 65535, 65536, 70000])
+def test_rows_as_long_but_not_the_same_are_found(k):
+    n = k + 3
+    hubs = np.array([k // 3, k // 2 + 1, k + 2])
+    rim = np.setdiff1d(np.arange(n), hubs)
+    cyc = np.stack([hubs, np.roll(hubs, -1)])
+    uv = np.stack([np.repeat(hubs, k), np.tile(rim, 3)])
+    for both in (False, True):
+        e = np.concatenate([uv, uv[::-1], cyc] + ([cyc[::-1]] if both else []), axis=1)
+        u, v = e[:, np.lexsort((e[1], e[0]))]
+        ro = np.zeros(n + 1, np.int64)
+        np.cumsum(np.bincount(u, minlength=n), out=ro[1:])
+        np.testing.assert_array_equal(np.diff(ro), np.bincount(v, minlength=n))
+        with sp.Graph(n, ro, v.astype(np.int32), np.ones(v.size, np.int32)) as g:
+            if both:
+                assert g.tc_init() == 3 * k + 1
+            else:
+                with pytest.raises(sp.SpError) as err:
+                    g.tc_init()
+                assert err.value.code == sp.SP_EINVAL
