@@ -43,83 +43,121 @@ __device__ __forceinline__ void block_add(u64 v, u64 *sm, u64 *global) {
 // building a store from a CSR
 // --------------------------------------------------------------------------
 
-// A walk over the edges of a CSR, kWalk consecutive ones per warp whatever the
-// rows' lengths: lanes take consecutive edges, and each edge's row comes from
+// A walk over the edges of a CSR, a chunk of consecutive ones per warp whatever
+// the rows' lengths: lanes take consecutive edges, and each edge's row comes from
 // the offsets of the 32 rows from the current one on (a search of five
-// shuffles), found once per warp and window without progress by a search of
-// all offsets, 32 at a time.  16.8 M edges: their items 261 -> 70 us (a search
-// of all offsets per edge before), their export 272 -> 75 us (a warp per row
-// before), the forward store in one pass of 79 us.  body(e, on, row, first): the edges of this lane,
-// whether each exists, its row and the row's first edge.
-constexpr int kWalk = 1024;
-constexpr int kWK = 4;   // edges per lane in flight
+// shuffles); the chunk's first row is found by a search of all offsets, 32 at a
+// time.  16.8 M edges: their items 261 -> 70 us (a search of all offsets per edge
+// before), their export 272 -> 75 us (a warp per row before), the forward store in
+// one pass of 79 us.
+// Where 32 rows hold fewer than kWalkSparse edges, windows would come one after
+// the other with hardly an edge each: there they get wider, with 2^s rows between
+// two lanes', which each edge then searches too (10 M vertices, 10 k edges: export
+// 3.31 -> 0.19 ms, 1.00 with a warp per row; 1 M and 300 k: 216 -> 65 us; with 16
+// or 8 edges as the limit 67 and 80 us, and no difference from 4 edges a row on).
+// The kernels are bound by memory latency, so their registers are held at 40, for
+// six blocks an SM (R-MAT 20's export: 147 us with 56 registers, 130 with 40).
+// body(e, on, row, first): the edges of this lane, whether each exists, its row
+// and the row's first edge.
+constexpr int kWalk = 1024;   // edges of a chunk at most
+constexpr int kWK = 4;        // edges per lane in flight
+constexpr int kWalkSparse = 32;
 
 template <typename Off, typename Body>
-__device__ __forceinline__ void walk_edges(const Off *off, int n, long long m, Body body) {
+__device__ __forceinline__ void walk_edges(const Off *off, int n, long long m, int chunk,
+                                           Body body) {
   const int lane = threadIdx.x & 31;
   const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long c0 = warp * kWalk; c0 < m; c0 += nwarps * kWalk) {
-    const long long c1 = c0 + kWalk < m ? c0 + kWalk : m;
+  for (long long c0 = warp * chunk; c0 < m; c0 += nwarps * chunk) {
+    const long long c1 = c0 + chunk < m ? c0 + chunk : m;
     long long e0 = c0;
-    long long r = 0;      // the first row of the window
-    bool search = true;
-    while (e0 < c1) {
-      if (search) {   // the row of e0: off[lo] <= e0 < off[hi]
-        long long lo = 0, hi = n;
-        while (hi - lo > 1) {
-          const long long step = (hi - lo + 31) / 32;
-          const long long p = lo + step * (lane + 1);
-          const bool below = p < hi && (long long)off[p] <= e0;
-          const int k = __popc(__ballot_sync(kFull, below));
-          const long long nlo = lo + step * k;
-          hi = nlo + step < hi ? nlo + step : hi;
-          lo = nlo;
-        }
-        r = lo;
-        search = false;
+    long long r = 0;      // the first row of the window: that of e0
+    {
+      long long hi = n;   // off[r] <= e0 < off[hi]
+      while (hi - r > 1) {
+        const long long step = (hi - r + 31) / 32;
+        const long long p = r + step * (lane + 1);
+        const bool below = p < hi && (long long)off[p] <= e0;
+        const int k = __popc(__ballot_sync(kFull, below));
+        const long long nlo = r + step * k;
+        hi = nlo + step < hi ? nlo + step : hi;
+        r = nlo;
       }
+    }
+    int s = 0;            // log2 of the rows between two lanes' rows
+    while (e0 < c1) {
+      const long long rl = r + ((long long)lane << s), re = r + (32ll << s);
       // (relative to e0, in 32 bits: a graph has fewer than 2^31 edges)
-      const int mine = (int)((long long)off[r + lane < n ? r + lane : n] - e0);
-      const long long wend = (long long)off[r + 32 < n ? r + 32 : n];
+      const int mine = (int)((long long)off[rl < n ? rl : n] - e0);
+      const long long wend = (long long)off[re < n ? re : n];
+      if (wend < c1 && wend - e0 < kWalkSparse) {   // hardly an edge: a wider window
+        s += 4;
+        continue;
+      }
       const long long end = wend < c1 ? wend : c1;
       const int len = (int)(end - e0);
       for (int b = 0; b < len; b += 32 * kWK) {
+        int row[kWK], fst[kWK];   // the edges' rows and their first edges, less e0
+#pragma unroll
+        for (int k = 0; k < kWK; ++k) {
+          const int x = b + 32 * k + lane < len ? b + 32 * k + lane : 0;
+          int o = 0;   // last row of the window that starts at or before x
+#pragma unroll
+          for (int step = 16; step > 0; step >>= 1)
+            if (__shfl_sync(kFull, mine, o + step) <= x) o += step;
+          fst[k] = __shfl_sync(kFull, mine, o);
+          row[k] = (int)(r + ((long long)o << s));
+        }
+#pragma unroll 1
+        for (int t = s - 1; t >= 0; --t) {   // ... among the rows between two lanes'
+#pragma unroll
+          for (int k = 0; k < kWK; ++k) {
+            const long long p = row[k] + (1ll << t);
+            const int x = b + 32 * k + lane < len ? b + 32 * k + lane : 0;
+            const int f = p < n ? (int)((long long)off[p] - e0) : x + 1;
+            if (f <= x) {
+              row[k] = (int)p;
+              fst[k] = f;
+            }
+          }
+        }
         long long e[kWK], first[kWK];
-        int row[kWK];
         bool on[kWK];
 #pragma unroll
         for (int k = 0; k < kWK; ++k) {
           const int j = b + 32 * k + lane;
           on[k] = j < len;
-          const int x = on[k] ? j : 0;
-          int o = 0;   // last row of the window that starts at or before x
-#pragma unroll
-          for (int step = 16; step > 0; step >>= 1)
-            if (__shfl_sync(kFull, mine, o + step) <= x) o += step;
           e[k] = e0 + j;
-          first[k] = e0 + __shfl_sync(kFull, mine, o);
-          row[k] = (int)(r + o);
+          first[k] = e0 + fst[k];
         }
         body(e, on, row, first);
       }
-      search = end <= e0;   // 32 rows without edges: find the next one
-      e0 = end > e0 ? end : e0;
-      r += 32;
+      e0 = end;
+      r = re;
     }
   }
 }
 
+// Edges of a chunk: as few as keep the grid within about one wave of warps, down
+// to what a warp has in flight, so that small graphs are spread over the GPU too.
+inline int walk_chunk(long long m) {
+  int c = 32 * kWK;
+  while (c < kWalk && (long long)c * 8192 < m) c *= 2;
+  return c;
+}
+
 // One chunk per warp: the grid's tail then costs a chunk, not a second round.
 inline unsigned walk_grid(long long m) {
-  return blocks_for(m, kWalk * (kThreads / 32), 1 << 30);
+  return blocks_for(m, walk_chunk(m) * (kThreads / 32), 1 << 30);
 }
 
 // One item per input edge: key = row << bits | col (reverse: col << bits | row).
-__global__ void k_edge_items(const long long *__restrict__ row_off, const int *__restrict__ col,
-                             const int *__restrict__ w, int n, long long m, int bits, int reverse,
-                             u64 *keys, u32 *vals) {
-  walk_edges(row_off, n, m,
+__global__ void __launch_bounds__(kThreads, 6)
+    k_edge_items(const long long *__restrict__ row_off, const int *__restrict__ col,
+                 const int *__restrict__ w, int n, long long m, int bits, int reverse, int chunk,
+                 u64 *keys, u32 *vals) {
+  walk_edges(row_off, n, m, chunk,
              [&](const long long *e, const bool *on, const int *row, const long long *) {
     int c[kWK], x[kWK];
 #pragma unroll
@@ -141,9 +179,9 @@ __global__ void k_edge_items(const long long *__restrict__ row_off, const int *_
 // if some are not (or hold an edge twice), and the rows are then filled again.
 __global__ void k_fill_csr(const long long *__restrict__ row_off, const int *__restrict__ col,
                            const int *__restrict__ w, int n, long long m,
-                           const RowMeta *__restrict__ row, int2 *adj, int *flag) {
+                           const RowMeta *__restrict__ row, int chunk, int2 *adj, int *flag) {
   bool bad = false;
-  walk_edges(row_off, n, m,
+  walk_edges(row_off, n, m, chunk,
              [&](const long long *e, const bool *on, const int *rw, const long long *first) {
     int c[kWK], p[kWK], x[kWK];
     long long at[kWK];
@@ -252,12 +290,13 @@ __global__ void k_row_degs(const RowMeta *__restrict__ row, int n, u64 *deg) {
 }
 
 // `off`: the rows' offsets in the export (a prefix sum of their degrees).
-__global__ void k_export_rows(const RowMeta *__restrict__ row, const int2 *__restrict__ adj, int n,
-                              const u64 *__restrict__ off, long long *row_off, int *col, int *w) {
+__global__ void __launch_bounds__(kThreads, 6)
+    k_export_rows(const RowMeta *__restrict__ row, const int2 *__restrict__ adj, int n,
+                  const u64 *__restrict__ off, int chunk, long long *row_off, int *col, int *w) {
   for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r <= n;
        r += (long long)gridDim.x * blockDim.x)
     row_off[r] = (long long)off[r];
-  walk_edges(off, n, (long long)off[n],
+  walk_edges(off, n, (long long)off[n], chunk,
              [&](const long long *e, const bool *on, const int *rw, const long long *first) {
     int2 x[kWK];
 #pragma unroll
@@ -1582,8 +1621,8 @@ sp_status store_build(sp_graph *g, Store *st, const long long *row_off_d, const 
   int hflag = 0;
   // the edges sorted by (row, col) of this store, into keys and vals
   auto sort_edges = [&](int lo_bit) {
-    k_edge_items<<<walk_grid(m), kThreads, 0, s>>>(row_off_d, col_d, w_d, n, m, bits, reverse, keys,
-                                                     vals);
+    k_edge_items<<<walk_grid(m), kThreads, 0, s>>>(row_off_d, col_d, w_d, n, m, bits, reverse,
+                                                     walk_chunk(m), keys, vals);
     ++*launches;
     if (sort_pairs(keys, vals, keys_alt, vals_alt, m, lo_bit, 2 * bits, tmp, s, launches)) {
       std::swap(keys, keys_alt);
@@ -1627,8 +1666,8 @@ sp_status store_build(sp_graph *g, Store *st, const long long *row_off_d, const 
     ++*launches;
     if (m > 0 && !reverse) {
       cudaMemsetAsync(flag, 0, sizeof(int), s);
-      k_fill_csr<<<walk_grid(m), kThreads, 0, s>>>(row_off_d, col_d, w_d, n, m, st->row, st->adj,
-                                                   flag);
+      k_fill_csr<<<walk_grid(m), kThreads, 0, s>>>(row_off_d, col_d, w_d, n, m, st->row,
+                                                   walk_chunk(m), st->adj, flag);
       ++*launches;
       read_flag();
       *in_order = hflag == 0;
@@ -1682,8 +1721,8 @@ sp_status store_export(sp_graph *g, const Store *st, long long *row_off_d, int *
   void *tmp = (void *)(((uintptr_t)(off + n + 1) + 255) & ~(uintptr_t)255);
   k_row_degs<<<grid, kThreads, 0, s>>>(st->row, n, deg);
   scan_exclusive_u64(deg, off, (long long)n + 1, tmp, s, launches);
-  k_export_rows<<<std::max(grid, walk_grid(g->m)), kThreads, 0, s>>>(st->row, st->adj, n, off,
-                                                                     row_off_d, col_d, w_d);
+  k_export_rows<<<std::max(grid, walk_grid(g->m)), kThreads, 0, s>>>(
+      st->row, st->adj, n, off, walk_chunk(g->m), row_off_d, col_d, w_d);
   *launches += 2;
   sp_status rc = cudaStreamSynchronize(s) == cudaSuccess ? SP_OK : SP_ECUDA;
   g->al.put(buf, need);

@@ -80,3 +80,57 @@ def test_stores_of_a_csr(n, m, kind):
             with pytest.raises(sp.SpError) as e:
                 sp.Graph(n, *args)
             assert e.value.code == sp.SP_EINVAL
+
+
+# graphs with far fewer edges than vertices, in part or in whole: a warp's window
+# of rows gets wider, among dense rows too, at every distance between edges
+@pytest.mark.parametrize("n,gaps", [(70000, (1, 2, 15, 16, 17)), (3000001, (31, 33, 255, 256, 511)),
+                                    (5000000, (4095, 4096, 8191, 70000)), (4000000, (1, 900, 1))])
+def test_stores_of_sparse_rows(n, gaps):
+    rng = np.random.default_rng(n)
+    rows = []
+    at = 0
+    for k in range(400):          # runs of rows `gap` apart, dense rows between them
+        gap = gaps[k % len(gaps)]
+        rows.append(at + gap * np.arange(60))
+        at = int(rows[-1][-1]) + gap
+        if k % 7 == 3:
+            rows.append(np.full(int(rng.integers(1, 1500)), at))
+            at += 1
+        if at >= n - 70 * max(gaps):
+            break
+    u = np.r_[0, np.concatenate(rows), n - 1]
+    key = np.unique(np.minimum(u, n - 1) * n + rng.integers(0, n, u.size))
+    w = rng.integers(1, sp.SP_WMAX + 1, size=key.size)
+    ro, col, ww = csr(n, key, w)
+    with sp.Graph(n, ro, col, ww) as g:
+        for rev in (False, True):
+            for got, want in zip(g.export_csr(reverse=rev), csr(n, key, w, rev)):
+                np.testing.assert_array_equal(got, want)
+
+
+def test_few_edges_among_many_vertices_are_not_slow():
+    # 10,000 edges on 10 M vertices load and export in less time than 10 M edges
+    # on as many (warps that walked 32 rows at a time took three times as long)
+    import time
+    import torch
+    n = 10 ** 7
+    best = {}
+    for m in (10 ** 4, 10 ** 7):
+        k = np.unique(np.random.default_rng(m).integers(0, n * n, m))
+        ro, col, w = csr(n, k, np.ones(k.size, np.int64))
+        d = [torch.from_numpy(x).cuda() for x in (ro, col, w)]
+        o = [torch.empty_like(x) for x in d]
+        load, export = [], []
+        for _ in range(5):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            with sp.Graph(n, *d) as g:
+                t1 = time.perf_counter()
+                g.export_csr_device(*o)
+                t2 = time.perf_counter()
+            load.append(t1 - t0)
+            export.append(t2 - t1)
+        assert all(torch.equal(x, y) for x, y in zip(d, o))
+        best[m] = min(load), min(export)
+    assert best[10 ** 4][0] < best[10 ** 7][0] and best[10 ** 4][1] < best[10 ** 7][1], best
