@@ -315,16 +315,20 @@ __device__ __forceinline__ u32 count_lists(const u32 *ptr, u32 len, const u32 *t
 // as sparse as the memory allows (an eighth or less filled up to 1,024 members;
 // symmetric R-MAT 18: 710 us at a quarter, 544 so).
 __global__ void __launch_bounds__(kThreads) k_tc_count(Store st, int n, const u32 *__restrict__ cnt,
-                                                       const u32 *__restrict__ big, Ctl *c) {
+                                                       const u32 *__restrict__ big, int per,
+                                                       Ctl *c) {
   __shared__ __align__(16) u32 tab[kTabMax];
   __shared__ u32 s_u, s_pos;
   if (ld_cg_i32(&c->status) != 0) return;   // not symmetric (the same answer in every block)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const u32 nlong = ld_cg_u32(&c->tc_nbig), nbig = nlong + ld_cg_u32(&c->tc_nmid);
   u64 sum = 0;
-  for (;;) {
+  // (what a block, and below a warp, takes first needs no counter: a small graph's
+  // grid would queue up at one word to be told that nothing is left)
+  for (bool first = true;; first = false) {
     __syncthreads();
-    if (threadIdx.x == 0) s_u = atomicAdd(&c->tc_bpos, 1u);
+    if (threadIdx.x == 0)
+      s_u = first ? blockIdx.x : gridDim.x + atomicAdd(&c->tc_bpos, 1u);
     __syncthreads();
     if (s_u >= nbig) break;
     const u32 u = big[s_u < nlong ? s_u : (u32)n - 1u - (s_u - nlong)];
@@ -360,15 +364,17 @@ __global__ void __launch_bounds__(kThreads) k_tc_count(Store st, int n, const u3
     }
   }
   __syncthreads();
-  // short lists: a warp takes 32 vertices, then those with two members or more
+  // short lists: a warp takes `per` vertices, then those with two members or more
   u32 *wtab = tab + warp * kWarpTab;
-  for (;;) {
-    u32 v0 = 0;
-    if (lane == 0) v0 = atomicAdd(&c->tc_spos, 1u);
-    const long long b = 32LL * __shfl_sync(kFull, v0, 0);
+  const u32 gw = (u32)warp * gridDim.x + blockIdx.x, nw = gridDim.x * (kThreads / 32);
+  for (bool first = true;; first = false) {
+    u32 v0 = gw;
+    if (!first && lane == 0) v0 = nw + atomicAdd(&c->tc_spos, 1u);
+    const long long b = (long long)per * __shfl_sync(kFull, v0, 0);
     if (b >= n) break;
-    const u32 dl = b + lane < n ? cnt[b + lane] : 0u;
-    const long long al = b + lane < n ? st.alt[b + lane] : 0;
+    const bool mine = lane < per && b + lane < n;
+    const u32 dl = mine ? cnt[b + lane] : 0u;
+    const long long al = mine ? st.alt[b + lane] : 0;
     u32 todo = __ballot_sync(kFull, dl >= 2 && dl <= kWarpList);
     while (todo) {
       const int o = __ffs(todo) - 1;
@@ -520,9 +526,11 @@ __global__ void __launch_bounds__(kThreads) k_tc_delta(DeltaArgs a, int kind) {
   const u64 cmask = (1ull << a.bits) - 1;
   const u64 ntask = ld_cg_u64(&c->tc_ntask[kind]);
   u64 k1 = 0, k2 = 0, k3 = 0;
-  for (;;) {
-    u64 t = 0;
-    if (lane == 0) t = atomicAdd(&c->tc_tpos[kind], 1ull);
+  const u64 gw = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  const u64 nw = gridDim.x * (kThreads / 32);
+  for (bool first = true;; first = false) {   // (a warp's first task is that of its number)
+    u64 t = gw;
+    if (!first && lane == 0) t = nw + atomicAdd(&c->tc_tpos[kind], 1ull);
     t = __shfl_sync(kFull, t, 0);
     if (t >= ntask || (long long)t >= a.cap) break;
     const u64 task = __ldcg(&a.tasks[kind ? a.cap - 1 - t : t]);
@@ -622,14 +630,20 @@ void launch_tc_static(sp_graph *g, int *launches) {
   k_tc_orient<<<grid_for(g->n, a.rpw * (kThreads / 32), g->num_sms * 16), kThreads, 0, g->stream>>>(
       a);
   ++*launches;
-  // (whether there is such a row is known on the device only: the host's edge
-  // count may lag behind the stores)
-  k_tc_orient_giant<<<(unsigned)g->num_sms * 4, kThreads, 0, g->stream>>>(a);
+  // such a row takes two regions of that length (the host's edge count would not
+  // do: it may lag behind the stores)
+  if (g->fwd.slots > 2 * kOrientGiant) {
+    k_tc_orient_giant<<<(unsigned)g->num_sms * 4, kThreads, 0, g->stream>>>(a);
+    ++*launches;
+  }
   k_tc_lists<<<grid_for(g->n, kThreads, g->num_sms * 8), kThreads, 0, g->stream>>>(a.cnt, g->n,
                                                                                    g->cut, g->ctl);
+  // a small graph's vertices are spread over all warps: 32 of them one after the
+  // other took 43 of the 74 us that 1,000 vertices' count was long
+  const int per = std::max(1, std::min(32, (int)(g->n / (g->num_sms * 6 * (kThreads / 32)))));
   k_tc_count<<<(unsigned)g->num_sms * 6, kThreads, 0, g->stream>>>(g->fwd, g->n, a.cnt, g->cut,
-                                                                   g->ctl);
-  *launches += 3;
+                                                                   per, g->ctl);
+  *launches += 2;
 }
 
 void launch_tc_batch_sym(sp_graph *g, long long nb, int *launches) {

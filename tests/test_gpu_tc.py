@@ -251,3 +251,27 @@ def test_rows_as_long_but_not_the_same_are_found(k):
                 with pytest.raises(sp.SpError) as err:
                     g.tc_init()
                 assert err.value.code == sp.SP_EINVAL
+
+
+def test_a_small_graph_is_spread_over_the_gpu():
+    # a thousand vertices' lists are one pass of the warps, not 32 after the other
+    # by 32 warps: the count takes hardly longer than the call on two vertices
+    # (twice as long before)
+    import time
+    best = {}
+    for n, k in ((2, 1), (1000, 4000)):
+        rng = np.random.default_rng(n)
+        u, v = (np.array([0]), np.array([1])) if n == 2 else rng.integers(0, n, (2, k))
+        u, v = u[u != v], v[u != v]
+        key = np.unique(np.concatenate([u * n + v, v * n + u]))
+        ro = np.zeros(n + 1, np.int64)
+        np.cumsum(np.bincount(key // n, minlength=n), out=ro[1:])
+        with sp.Graph(n, ro, (key % n).astype(np.int32), np.ones(key.size, np.int32)) as g:
+            g.tc_init()
+            times = []
+            for _ in range(200):
+                t0 = time.perf_counter()
+                g.tc_init()
+                times.append(time.perf_counter() - t0)
+            best[n] = min(times)
+    assert best[1000] < 1.5 * best[2], best
