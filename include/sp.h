@@ -543,7 +543,12 @@ sp_status sp_server_get_dist(sp_server *s, int32_t graph_id, int32_t *dist);
 /* staticPR: all ranks start at 1/n and S is every vertex.  Sets the PageRank
  * settings used by later batches.  SP_EINVAL for damping outside [0, 1],
  * beta < 0 or max_iter < 1.  stats (nullable): rounds_push = Jacobi steps,
- * relaxed_edges = in-edges pulled. */
+ * relaxed_edges = in-edges pulled.
+ * Memory: the first call takes 20 bytes a vertex, and 4.5 bytes an edge (and 13.5
+ * a vertex at most) for packed in-neighbour lists, kept until the handle is
+ * destroyed.  A later call or rank batch that finds more edges than there is
+ * room for takes a larger buffer before it gives the old one back; where it cannot
+ * be had, the lists go to the store's alternate regions and the call takes longer. */
 sp_status sp_pr_init(sp_graph *g, float damping, float beta, int32_t max_iter,
                      sp_batch_stats *stats);
 
@@ -601,12 +606,15 @@ sp_status sp_tc_apply_batch(sp_graph *g, int64_t n_del, const int32_t *del_src,
                             int inputs_on_device, int64_t *count, sp_batch_stats *stats);
 
 /*
- * sp_apply_batch runs its kernels (seven per batch) as a cached CUDA graph
- * when a batch has the same shape (deletion and insertion counts, stats or
- * not) as the one before it: one graph launch replaces the kernel launches.
- * Device inputs are read where they are (the three kernels that read them
- * are pointed at this call's arrays before the launch); host inputs are
- * first moved to internal buffers.  The graph is rebuilt when a buffer or a
+ * sp_apply_batch runs its kernels (seven per batch, five for one of at most
+ * 1,024 updates) as a cached CUDA graph when a batch has the same shape
+ * (deletion and insertion counts, stats or not) as the one before it: one
+ * graph launch replaces the kernel launches.  Device inputs are read where
+ * they are (the kernels that read them -- the sort, the searches and the
+ * invalidation, or a small batch's check, plan and invalidation -- are pointed
+ * at this call's arrays before the launch); host inputs are first moved to
+ * internal buffers, or read by a small batch's check (see sp_apply_batch).
+ * The graph is rebuilt when a buffer or a
  * setting changes.  on = 0 turns it off (every call launches kernels one by
  * one); the default is 1.  Results do not depend on it.  Requires a
  * non-default stream (graphs are never used on the legacy stream).

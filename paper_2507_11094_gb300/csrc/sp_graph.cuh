@@ -147,7 +147,7 @@ struct LoopArgs {
 
 namespace sp {
 // Batches of at most this many updates are planned by one block, and read from
-// host memory in place; distances of at most kSmallOut vertices reach pageable
+// host memory by their check, without a staging copy; distances of at most kSmallOut vertices reach pageable
 // arrays through the handle's page-locked block (5 x 4 KB + 2 x 64 KB).
 constexpr int kSmallUpdates = 1024;
 constexpr int kSmallOut = 16384;

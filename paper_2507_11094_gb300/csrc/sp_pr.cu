@@ -58,9 +58,9 @@ constexpr u32 kRowTile = 4096;           // rows a block sums before it finishes
 constexpr size_t kPrSmem = (size_t)(kHot + 4 + kRowTile) * sizeof(float);
 // in-degree classes: a row of more than kSegLen in-edges in segments of that
 // length, a warp each; down to kGroupMax a warp; down to kLaneMax eight
-// lanes; the rest a lane; rows without in-edges take the constant term
+// lanes; the rest a lane; rows without in-edges take the constant term in every
+// step.  The vertices of no phase come last.
 constexpr u32 kSegLen = 1024, kGroupMax = 64, kLaneMax = 8;
-// in every step.  The vertices of no phase come last.
 enum { kClsHub = 0, kClsWarp, kClsGroup, kClsLane, kClsZero, kClsOut, kClasses };
 
 // Zeroed before every launch.

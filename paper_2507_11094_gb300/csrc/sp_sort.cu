@@ -241,8 +241,8 @@ k_scatter(const u64 *__restrict__ keys, const u32 *__restrict__ vals, long long 
 // more, half of them sorts the forward items and half the reverse ones, each
 // within its own half of the positions, and the store's bit is not sorted on
 // either.  That leaves 2 * bits key bits, in digits of ten bits where this
-// saves a pass over nine (19, 20 and 23 to 25 bits an id): on R-MAT 20 four
-// passes instead of five, on R-MAT 22 five (nine bits) instead of six.  A pass
+// saves a pass over nine (ids of 5, 10, 14, 15, 19, 20, 23 to 25 and 28 to 30
+// bits): on R-MAT 20 four passes instead of five, on R-MAT 22 five (nine bits) instead of six.  A pass
 // is two grid barriers, a scatter and a read back.  A batch and its undo of
 // 1,000,000 updates on R-MAT 22: 2,398 -> 2,369 us, of 161,000 on 32 graphs
 // together: 1,070 -> 1,058 us, of 20,971 pairs in the triangle count: 1,012 ->

@@ -842,13 +842,16 @@ __global__ void __launch_bounds__(kCT, 3) k_search(SearchArgs a) {
   }
 }
 
-// The searches interpolate where the store is well beyond the L2: there they
+// The searches interpolate where the store is many times the L2: there they
 // are bound by random reads from DRAM (twice the threads made them slower),
 // and three rounds of reads take the place of ten.  A million updates on
-// R-MAT 22 (1.7 GB a store): search 355 -> 238 us, the batch 1.42 -> 1.25 ms.
-// In stores that the L2 half holds a halving step costs less than a guess:
-// R-MAT 20 (0.42 GB) 51 against 50 us, 32 small R-MATs (0.38 GB) 57 against
-// 71 us.
+// R-MAT 22 (1.9 GB a store): search 355 -> 238 us, the batch 1.42 -> 1.25 ms.
+// On smaller stores a halving step, whose first reads are the same few sectors
+// for every update of a row, costs less than a guess.  Sort (with the searches
+// beside it) and count of a 1% batch, halving and interpolating: R-MAT 19 (0.24
+// GB) 125 and 124 us, R-MAT 20 (0.47 GB) 162 and 156, R-MAT 21 (0.94 GB) 289 and
+// 265, R-MAT 22 518 and 425; the searches of 32 small R-MATs (0.38 GB) 57 and
+// 71 us.  20,000 updates take the same time either way on all of them (within 1%).
 bool search_guesses(const sp_graph *g) {
   return std::max(g->fwd.slots, g->rev.slots) * (long long)sizeof(int2) >= (1LL << 30);
 }
@@ -890,8 +893,11 @@ unsigned search_grid(const sp_graph *g, const SearchArgs &a) {
 // scans that of the grid barriers.  Before it one more block resets the control
 // block and checks the batch, so that the invalidation runs beside all of it.
 // A call with 64 updates on 1,024 vertices: 136 -> 112 us; with 1,001 on
-// 100,003: 195 -> 172 us.  Above kPlanItems one block's searches and sort take
-// longer than the grid's.
+// 100,003: 195 -> 172 us.  The line lies where the block's threads hold two items
+// each and its shared memory (40 KB) is what every launch may have, not where
+// the two ways meet: device time of a call by the plan and by the grid's sort,
+// with 64, 512 and 1,024 updates: 105 and 145, 122 and 164, 140 and 171 us on
+// R-MAT 20; 119 and 155, 136 and 172, 148 and 181 us on 300,000 vertices.
 constexpr int kPlanT = 1024;             // threads at most: as many as the items need,
 constexpr int kPlanItems = 2 * kPlanT;   // two items each (a power of two of threads)
 static_assert(kPlanItems == 2 * kSmallUpdates, "two items an update");
