@@ -227,6 +227,7 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
   if (!repair_enabled_block(c)) return;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const u32 n = (u32)a.n, G = gridDim.x;
+  constexpr int kF = kRowTile / kPrThreads;   // rows that a thread takes at a time
   const u32 chunk = (n + G - 1) / G;
   const u32 cb = min(blockIdx.x * chunk, n), ce = min(cb + chunk, n);
   u64 *bar = &c->bar_push;
@@ -240,22 +241,32 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
   if (t == 0) s_segs = 0;
   __syncthreads();
   u64 edges = 0;
-  for (u32 b = cb + (t & ~31); b < ce; b += kPrThreads) {
-    const u32 v = b + lane;
-    const bool on = v < ce;
-    const bool sel = on && (a.all || __ldcg(a.flag + v) == a.tag);
-    const u32 od = on ? (u32)__ldg(&a.fwd.row[v].deg) : 0u;
-    const u32 id = sel ? (u32)__ldg(&a.rev.row[v].deg) : 0u;
-    if (on) atomicAdd(&s_bins[min(od, kPrBins - 1)], 1u);
-    const int cls = sel ? in_class(id) : on ? kClsOut : -1;
+  for (u32 b = cb + (t & ~31); b < ce; b += kF * kPrThreads) {
+    u32 od[kF], id[kF], fl[kF];
 #pragma unroll
-    for (int k = 0; k < kClasses; ++k) {
-      const u32 m = __ballot_sync(kFull, cls == k);
-      const u32 w = __reduce_add_sync(kFull, cls == k ? (id + 3) / 4 : 0u);
-      if (lane == 0 && m) atomicAdd(&s_cls[k], ((u64)__popc(m) << 32) | w);
+    for (int q = 0; q < kF; ++q) {   // kF vertices' loads in flight together
+      const u32 v = b + q * kPrThreads + lane;
+      const bool on = v < ce;
+      fl[q] = on && !a.all ? __ldcg(a.flag + v) : a.tag;
+      od[q] = on ? (u32)__ldg(&a.fwd.row[v].deg) : 0u;
+      id[q] = on ? (u32)__ldg(&a.rev.row[v].deg) : 0u;
     }
-    if (cls == kClsHub) atomicAdd(&s_segs, (id + kSegLen - 1) / kSegLen);
-    edges += id;
+#pragma unroll
+    for (int q = 0; q < kF; ++q) {
+      const bool on = b + q * kPrThreads + lane < ce, sel = on && fl[q] == a.tag;
+      if (!sel) id[q] = 0;
+      if (on) atomicAdd(&s_bins[min(od[q], kPrBins - 1)], 1u);
+      const int cls = sel ? in_class(id[q]) : on ? kClsOut : -1;
+#pragma unroll
+      for (int k = 0; k < kClasses; ++k) {
+        const u32 m = __ballot_sync(kFull, cls == k);
+        if (!m) continue;
+        const u32 w = __reduce_add_sync(kFull, cls == k ? (id[q] + 3) / 4 : 0u);
+        if (lane == 0) atomicAdd(&s_cls[k], ((u64)__popc(m) << 32) | w);
+      }
+      if (cls == kClsHub) atomicAdd(&s_segs, (id[q] + kSegLen - 1) / kSegLen);
+      edges += id[q];
+    }
   }
   edges = warp_sum(edges);
   if (lane == 0 && edges) atomicAdd(&a.sc->edges, edges);
@@ -309,13 +320,26 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
   }
   u32 *lists = packed ? a.lists : (u32 *)a.rev.adj;
   const u32 T = s_T, nhot = s_nhot;
+  u32 nfl = a.tag;   // the next vertex's flag, out-degree and rank, read one ahead
+  int nod = 0;
+  float nr = a.init;
+  auto ahead = [&](u32 v) {
+    if (v >= ce) return;
+    nod = __ldg(&a.fwd.row[v].deg);
+    if (!a.all) {
+      nfl = __ldcg(a.flag + v);
+      nr = __ldcg(a.pr + v);
+    }
+  };
+  ahead(cb + t);
   for (u32 b = cb + (t & ~31); b < ce && !stop; b += kPrThreads) {
     const u32 v = b + lane;
     const bool on = v < ce;
-    const bool sel = on && (a.all || __ldcg(a.flag + v) == a.tag);
-    const int od = on ? __ldg(&a.fwd.row[v].deg) : 0;
-    const RowMeta in = on && sel ? a.rev.row[v] : RowMeta{0, 0, 0};
-    const float r = on ? (a.all ? a.init : __ldcg(a.pr + v)) : 0.0f;
+    const bool sel = on && nfl == a.tag;
+    const int od = on ? nod : 0;
+    const float r = on ? nr : 0.0f;
+    const RowMeta in = sel ? a.rev.row[v] : RowMeta{0, 0, 0};
+    ahead(v + kPrThreads);
     const int cls = sel ? in_class((u32)in.deg) : on ? kClsOut : -1;
     u32 pos = 0, wpos = 0;
     const u32 nw4 = ((u32)in.deg + 3) / 4;
@@ -423,6 +447,8 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
   }
   __syncthreads();
 
+  // a block's share of k positions: one run of them
+  auto share = [&](u32 k, u32 b) { return (u32)((u64)k * b / G); };
   // 4. Jacobi steps
   u32 it = 0, cur = 0;
   for (;;) {
@@ -542,7 +568,6 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
       if (t == 0) s_unit = 0;
       // then a thread per row finishes them, so that ranks and terms go 32
       // consecutive positions to a warp
-      constexpr int kF = kRowTile / kPrThreads;
       u32 pos[kF];
       int p[kF], od[kF];
       float rk[kF];
@@ -565,13 +590,29 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
       __syncthreads();
     }
     // no in-edges: the constant term, from the first step on (and into both
-    // term buffers)
-    if (it < 2)
-      for (u32 i = blockIdx.x * kPrThreads + t; i < cnt[kClsZero]; i += G * kPrThreads) {
-        const u32 pos = first[kClsZero] + i;
-        finish(a, next, pos, 0.0f, __ldcg(&a.lenp[pos].y), __ldcg(&a.degv[pos].x),
-               __ldcg(a.rank + pos), diff);
+    // term buffers); kF rows' loads together (10 M such rows: 450 us a step when
+    // each waited alone, 85 so)
+    if (it < 2) {
+      const u32 z1 = first[kClsZero] + share(cnt[kClsZero], blockIdx.x + 1);
+      for (u32 z0 = first[kClsZero] + share(cnt[kClsZero], blockIdx.x); z0 < z1;
+           z0 += kF * kPrThreads) {
+        int p[kF], od[kF];
+        float rk[kF];
+#pragma unroll
+        for (int k = 0; k < kF; ++k) {
+          const u32 pos = z0 + k * kPrThreads + t;
+          if (pos < z1) {
+            p[k] = __ldcg(&a.lenp[pos].y);
+            od[k] = __ldcg(&a.degv[pos].x);
+            rk[k] = __ldcg(a.rank + pos);
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < kF; ++k)
+          if (z0 + k * kPrThreads + t < z1)
+            finish(a, next, z0 + k * kPrThreads + t, 0.0f, p[k], od[k], rk[k], diff);
       }
+    }
     {
       // (the warp's 32 sums meet as floats too: in 64 bits 1.8 us a step)
 #pragma unroll
@@ -599,10 +640,11 @@ __global__ void __launch_bounds__(kPrThreads, 1) k_pr(PrArgs a) {
     cur ^= 1;
     if (!(d > a.beta) || it >= (u32)a.max_iter) break;
   }
-  if (!stop)
-    for (u32 i = blockIdx.x * kPrThreads + t; i < first[kClsZero] + cnt[kClsZero];
-         i += G * kPrThreads)
+  if (!stop) {
+    const u32 all = first[kClsZero] + cnt[kClsZero], i1 = share(all, blockIdx.x + 1);
+    for (u32 i = share(all, blockIdx.x) + t; i < i1; i += kPrThreads)
       a.pr[(u32)__ldcg(&a.degv[i].y)] = __ldcg(a.rank + i);
+  }
   if (blockIdx.x == 0 && t == 0) {
     volatile Ctl *vc = c;
     vc->pull_edges = (u64)it * __ldcg(&a.sc->edges);
