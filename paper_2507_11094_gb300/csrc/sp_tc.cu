@@ -513,10 +513,12 @@ __global__ void __launch_bounds__(kThreads) k_tc_tasks(DeltaArgs a) {
 // at a time, and searches the longer one with the lanes' searches in lockstep,
 // so that kDK loads per lane are in flight at every level; a hit is looked up
 // only among the batch items of rows v1 and v2, whose bounds are found once
-// per task (four lanes at once).  Bound by the searches' dependent levels
-// through L2.  R-MAT 18, 1% of the pairs deleted and as many inserted: a batch
-// 1.93 -> 0.54 ms against a warp per item over both directions, one search
-// chain per lane, and every hit looked up among all items.
+// per task (four lanes at once), at its first hit (a sparse graph's tasks have
+// hardly one: 60,000 pairs on 100,000 vertices, two batches, 534 -> 500 us).
+// Bound by the searches' dependent levels through L2.  R-MAT 18, 1% of the pairs
+// deleted and as many inserted: a batch 1.93 -> 0.54 ms against a warp per item
+// over both directions, one search chain per lane, and every hit looked up among
+// all items.
 constexpr int kDK = 4;
 
 __global__ void __launch_bounds__(kThreads) k_tc_delta(DeltaArgs a, int kind) {
@@ -543,14 +545,7 @@ __global__ void __launch_bounds__(kThreads) k_tc_delta(DeltaArgs a, int kind) {
     const int wdeg = walk1 ? r1.deg : r2.deg;
     const int2 *srow = a.st.adj + (walk1 ? r2.start : r1.start);
     const int sdeg = walk1 ? r2.deg : r1.deg;
-    // the batch items of rows v1 (lanes 0, 1) and v2 (lanes 2, 3)
-    long long bound = 0;
-    if (lane < 4) {
-      const u64 row = (u64)(lane < 2 ? v1 : v2) + (u64)(lane & 1);
-      bound = item_lower(a.keys, 0, a.nb, row << (a.bits + 1));
-    }
-    const long long lo1 = __shfl_sync(kFull, bound, 0), hi1 = __shfl_sync(kFull, bound, 1);
-    const long long lo2 = __shfl_sync(kFull, bound, 2), hi2 = __shfl_sync(kFull, bound, 3);
+    long long bound = -1;
     for (int b = part * 32 * kDK; b < wdeg; b += parts * 32 * kDK) {
       int x[kDK], lo[kDK], hi[kDK];
 #pragma unroll
@@ -578,11 +573,27 @@ __global__ void __launch_bounds__(kThreads) k_tc_delta(DeltaArgs a, int kind) {
             if (y[k] < x[k]) lo[k] = mid[k] + 1; else hi[k] = mid[k];
           }
       }
+      bool hit[kDK], any = false;
 #pragma unroll
       for (int k = 0; k < kDK; ++k) {
         const u32 v3 = (u32)x[k];
-        if (x[k] < 0 || v3 == v1 || v3 == v2) continue;
-        if (lo[k] >= sdeg || __ldg(&srow[lo[k]].x) != x[k]) continue;
+        hit[k] = x[k] >= 0 && v3 != v1 && v3 != v2 && lo[k] < sdeg &&
+                 __ldg(&srow[lo[k]].x) == x[k];
+        any |= hit[k];
+      }
+      if (!__any_sync(kFull, any)) continue;
+      if (__shfl_sync(kFull, bound, 0) < 0 && lane < 4) {
+        // the batch items of rows v1 (lanes 0, 1) and v2 (lanes 2, 3)
+        const u64 row = (u64)(lane < 2 ? v1 : v2) + (u64)(lane & 1);
+        bound = item_lower(a.keys, 0, a.nb, row << (a.bits + 1));
+      }
+      __syncwarp();
+      const long long lo1 = __shfl_sync(kFull, bound, 0), hi1 = __shfl_sync(kFull, bound, 1);
+      const long long lo2 = __shfl_sync(kFull, bound, 2), hi2 = __shfl_sync(kFull, bound, 3);
+#pragma unroll
+      for (int k = 0; k < kDK; ++k) {
+        if (!hit[k]) continue;
+        const u32 v3 = (u32)x[k];
         const u64 tail = ((u64)v3 << 1) | (u64)kind;
         const int kk = 1 +
             item_applied(a.keys, a.flags, lo1, hi1, ((u64)v1 << (a.bits + 1)) | tail) +
